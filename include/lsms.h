@@ -52,7 +52,7 @@ typedef enum {
 } lsms_status;
 
 typedef enum {
-  LSMS_FP64 = 0,   /* every step in float64                                                    */
+  LSMS_FP64 = 0,   /* float64 throughout (products of large sums as exact sums of digits)      */
   LSMS_MIXED = 1   /* FP32 translation, split-BF16 tensor-core contour contractions, FP64 refinement */
 } lsms_precision;
 

@@ -72,6 +72,14 @@ int need_particles(lsms_ctx* c) {
   return LSMS_OK;
 }
 
+int translate_f64(lsms_ctx* c, int nrhs, const double2* xs, double2* alpha, cudaStream_t st, int row0, int nrows) {
+  if (nrows < 0) nrows = c->n - row0;
+  if (c->n == 0 || nrhs == 0 || nrows <= 0) return LSMS_OK;
+  if (c->f64tc.ready) return translate_f64_tc(c, nrhs, xs, alpha, st, row0, nrows);
+  launch_translate_f64(c->d_cx, c->d_cy, c->n, c->p, c->k2, xs, alpha, nrhs, st, row0, nrows);
+  return LSMS_OK;
+}
+
 // Reflected coupling, FP64: alpha += E' (U * sigma(P, Q)), with P, Q from E * xs.
 int reflection_f64(lsms_ctx* c, int nrhs, const double2* xs, double2* alpha, cudaStream_t st) {
   const int ns = c->ns, P = c->P, n = c->n;
@@ -133,8 +141,8 @@ int apply_device(lsms_ctx* c, int nrhs, const double2* x, double2* y, int flags,
       launches += 3 + (c->near_nnz > 0 ? 1 : 0);
       if ((rc = translate_mixed(c, nrhs, xs, alpha, st))) return rc;
     } else {
-      launches += 1;
-      launch_translate_f64(c->d_cx, c->d_cy, n, c->p, c->k2, xs, alpha, nrhs, st);
+      launches += c->f64tc.ready ? 3 + (c->f64tc.nnz > 0 ? 1 : 0) : 1;
+      if ((rc = translate_f64(c, nrhs, xs, alpha, st))) return rc;
     }
   } else {
     cudaMemsetAsync(alpha, 0, len * sizeof(double2), st);
@@ -204,8 +212,8 @@ int apply_rows_device(lsms_ctx* c, int nrhs, int row0, int row1, const double2* 
   if (!(flags & LSMS_APPLY_NO_TRANSLATION)) {
     if (mixed) {
       if ((rc = translate_mixed_rows(c, nrhs, xs, arows, row0, nrows, st))) return rc;
-    } else {
-      launch_translate_f64(c->d_cx, c->d_cy, n, c->p, c->k2, xs, arows, nrhs, st, row0, nrows);
+    } else if ((rc = translate_f64(c, nrhs, xs, arows, st, row0, nrows))) {
+      return rc;
     }
   } else {
     cudaMemsetAsync(arows, 0, len_rows * sizeof(double2), st);
@@ -376,6 +384,7 @@ extern "C" void lsms_destroy(lsms_ctx* c) {
     if (b->ptr) cudaFree(b->ptr);
   tc_free(c);
   fmm_free(c);
+  f64tc_free(c);
   if (c->h_pinned) cudaFreeHost(c->h_pinned);
   if (c->gm_ring) cudaFreeHost(c->gm_ring);
   for (cudaEvent_t e : c->ev)
@@ -411,6 +420,7 @@ extern "C" int lsms_set_particles(lsms_ctx* c, int n, const double* xy) {
   std::vector<double> xs(n);
   for (int j = 0; j < n; ++j) xs[j] = c->cx[j] - c->xc;
   tc_free(c);
+  f64tc_free(c);
   void* old[] = {c->d_cx, c->d_cy, c->d_eagg, c->d_edis, c->d_eagg_lp, c->d_edis_lp, c->d_lp_misc};
   for (void* q : old)
     if (q) cudaFree(q);
@@ -437,9 +447,12 @@ extern "C" int lsms_set_particles(lsms_ctx* c, int n, const double* xy) {
     if ((rc = check_cuda(c, "set_particles"))) return rc;
     if ((rc = build_lowp_tables(c))) return rc;
   }
-  if (c->fmm.box_width > 0.0) return fmm_setup(c);
-  fmm_free(c);
-  return LSMS_OK;
+  if (c->fmm.box_width > 0.0) {
+    if ((rc = fmm_setup(c))) return rc;
+  } else {
+    fmm_free(c);
+  }
+  return f64tc_sequences(c);
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -482,8 +495,7 @@ extern "C" int lsms_apply_ex(lsms_ctx* c, int nrhs, const double* x, double* y, 
   if ((rc = ensure(c, c->ws_y, len * sizeof(double2)))) return rc;
   if ((rc = apply_device(c, nrhs, (const double2*)c->ws_x.ptr, (double2*)c->ws_y.ptr, flags, c->stream))) return rc;
   if ((rc = copy_out(c, y, c->ws_y.ptr, len))) return rc;
-  if (!(flags & LSMS_APPLY_MIXED)) return LSMS_OK;
-  return is_batch(c) ? batch_mixed_check(c) : mixed_check(c);
+  return mixed_check(c);
 }
 
 extern "C" int lsms_apply(lsms_ctx* c, int nrhs, const double* x, double* y) {
@@ -514,10 +526,11 @@ extern "C" int lsms_translate(lsms_ctx* c, int nrhs, const double* beta, double*
       return rc;
   } else if (precision == LSMS_MIXED) {
     if ((rc = translate_mixed(c, nrhs, (const double2*)c->ws_x.ptr, (double2*)c->ws_alpha.ptr, c->stream))) return rc;
-  } else
-    launch_translate_f64(c->d_cx, c->d_cy, c->n, c->p, c->k2, (const double2*)c->ws_x.ptr, (double2*)c->ws_alpha.ptr, nrhs, c->stream);
+  } else if ((rc = translate_f64(c, nrhs, (const double2*)c->ws_x.ptr, (double2*)c->ws_alpha.ptr, c->stream)))
+    return rc;
   if ((rc = check_cuda(c, "translate"))) return rc;
-  return copy_out(c, alpha, c->ws_alpha.ptr, len);
+  if ((rc = copy_out(c, alpha, c->ws_alpha.ptr, len))) return rc;
+  return mixed_check(c);
 }
 
 extern "C" int lsms_aggregate(lsms_ctx* c, int nrhs, const double* beta, double* p_plus,

@@ -924,7 +924,10 @@ extern "C" int lsms_set_fmm(lsms_ctx* c, double box_width, int order) {
     const int rc = lsms_set_fmm(k, box_width, order);
     if (rc) return ctx_fail(c, rc, std::string("set_fmm: ") + k->err);
   }
-  if (c->kids.empty() && c->n >= 0) return fmm_setup(c);
+  if (c->kids.empty() && c->n >= 0) {
+    const int rc = fmm_setup(c);
+    return rc ? rc : f64tc_sequences(c);
+  }
   return LSMS_OK;
 }
 
@@ -935,8 +938,11 @@ extern "C" int lsms_set_fmm_scope(lsms_ctx* c, int scope) {
   cudaStreamSynchronize(c->stream);
   batch_clear_graphs(c);
   c->fmm.scope = scope;
-  for (lsms_ctx* k : c->kids) k->fmm.scope = scope;
-  return LSMS_OK;
+  for (lsms_ctx* k : c->kids) {
+    const int rc = lsms_set_fmm_scope(k, scope);
+    if (rc) return ctx_fail(c, rc, std::string("set_fmm_scope: ") + k->err);
+  }
+  return f64tc_sequences(c);
 }
 
 extern "C" int lsms_fmm_stats(lsms_ctx* c, long long* near_pairs, double* far_ms, double* near_ms) {

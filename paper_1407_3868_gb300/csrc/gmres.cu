@@ -606,7 +606,7 @@ int gmres_finish(lsms_ctx* c, const GmPtrs& g, const GmSys& s, std::vector<int>&
                  int flags, int* iters, double2* x, cudaStream_t stream) {
   int rc;
   (void)maxiter;
-  if ((flags & LSMS_APPLY_MIXED) && (rc = mixed_check(c))) return rc;
+  if ((rc = mixed_check(c))) return rc;
   const int nb = s.nb;
   bool all = true;
   for (int b = 0; b < nb; ++b) {
@@ -770,7 +770,7 @@ int gmres_batch_t(lsms_ctx* c, const GmSys& s, const double2* rhs, double2* x, b
       return rc;
     if (loop_k >= 0) {
       if (nonfinite) {
-        if ((flags & LSMS_APPLY_MIXED) && (rc = mixed_check(c))) return rc;
+        if ((rc = mixed_check(c))) return rc;
         return ctx_fail(c, LSMS_ERR_NONFINITE, "non-finite value in GMRES");
       }
       return gmres_finish<T>(c, g, s, kdone, loop_k, maxiter, flags, iters, x, stream);
@@ -827,7 +827,7 @@ int gmres_batch_t(lsms_ctx* c, const GmSys& s, const double2* rhs, double2* x, b
   if (exec) cudaGraphExecDestroy(exec);
   cudaStreamSynchronize(stream);
   if (nonfinite) {
-    if ((flags & LSMS_APPLY_MIXED) && (rc = mixed_check(c))) return rc;
+    if ((rc = mixed_check(c))) return rc;
     return ctx_fail(c, LSMS_ERR_NONFINITE, "non-finite value in GMRES");
   }
   return gmres_finish<T>(c, g, s, kdone, checked, maxiter, flags, iters, x, stream);

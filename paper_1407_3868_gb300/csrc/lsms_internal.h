@@ -79,6 +79,17 @@ struct FmmState {
   cudaEvent_t ev[3] = {nullptr, nullptr, nullptr};   // far start, near start, near end (timing)
 };
 
+// FP64 translation on the tensor cores (translate_f64_tc.cu): tables of the current layout.
+struct F64Tc {
+  bool ready = false;               // the layout's FP64 all-pairs translation runs there
+  void* d_table = nullptr;          // longlong2 [256]: e^{i (2 pi j / 256 - pi / 4)} in Q62
+  int* d_ptr = nullptr;             // [n + 1] near pairs (k2 rho below pair_z_near) by target
+  int* d_idx = nullptr;             // [nnz] sources, then [nnz] targets
+  void* d_seq = nullptr;            // double2 [nnz][4p + 1]: their Hankel sequences (f64tc_sequences)
+  int nnz = 0;
+  DevBuf ws;                        // scales and digit images of the coefficients
+};
+
 struct lsms_ctx {
   // medium and discretisation: layers ks[0] (top) .. ks[L-1] (bottom), interior thicknesses
   // ds[0..L-3]; the discs lie in layer `layer` (1-based, 2 <= layer <= L-1), whose top interface is
@@ -102,6 +113,7 @@ struct lsms_ctx {
   DevBuf theta_buf;                 // [N] rotation angles (valid when has_theta)
   bool has_theta = false;
   FmmState fmm;
+  F64Tc f64tc;
   // side stream of the mixed operator: the reflected coupling runs beside the translation
   cudaStream_t side = nullptr;
   cudaEvent_t ev_fork = nullptr, ev_join = nullptr;

@@ -19,6 +19,16 @@ int fmm_setup(lsms_ctx* c);
 void fmm_free(lsms_ctx* c);
 // mixed: the near field in FP32 (adjacent boxes) plus the FP32 near-pair kernel; else all FP64
 int fmm_translate(lsms_ctx* c, int nrhs, const double2* xs, double2* alpha, bool mixed, cudaStream_t st);
+// FP64 all-pairs translation on the tensor cores (translate_f64_tc.cu): tables from the layout's
+// near-pair candidates (ready stays false where the FP64 pipe is kept), rows of alpha = T xs
+int f64tc_setup(lsms_ctx* c, const std::vector<int>& ptr, const std::vector<int>& idx);
+void f64tc_free(lsms_ctx* c);
+int f64tc_sequences(lsms_ctx* c);     // after a change of the layout or of the box translation
+int translate_f64_tc(lsms_ctx* c, int nrhs, const double2* xs, double2* alpha, cudaStream_t st, int row0, int nrows);
+// rows row0 .. row0 + nrows - 1 (nrows < 0: to the last disc) of alpha = T xs in FP64, by whichever
+// path the layout takes
+int translate_f64(lsms_ctx* c, int nrhs, const double2* xs, double2* alpha, cudaStream_t st, int row0 = 0,
+                  int nrows = -1);
 // drop the captured batched applications (their kernels depend on the context's settings)
 void batch_clear_graphs(lsms_ctx* c);
 int check_cuda(lsms_ctx* c, const char* where);

@@ -13,13 +13,13 @@
 #include <cmath>
 #include <mutex>
 #include <numeric>
-#include <unordered_map>
 #include <vector>
 
 #include "lsms_internal.h"
 #include "lsms_ops.h"
 #include "ff_hankel.cuh"
 #include "near_pairs.cuh"
+#include "pair_fixed.cuh"
 
 namespace {
 
@@ -763,8 +763,10 @@ void launch_translate_sym(cudaStream_t st, const float4* cff, int n, int p, floa
 
 }  // namespace
 
-// CSR list of near pairs (k2 rho < 25) by target, from a cell grid, and their H_0, H_1 (FP64-built).
-static int build_near_pairs(lsms_ctx* c) {
+// CSR list of near pairs (k2 rho < 25) by target, from a cell grid, and their H_0, H_1 (FP64-built);
+// `wide_ptr`, `wide_idx`: the same for the distances the FP64 tensor-core translation leaves out
+// (a margin of 1e-6 included: its kernels decide in their own rounding).
+static int build_near_pairs(lsms_ctx* c, std::vector<int>& wide_ptr, std::vector<int>& wide_idx) {
   void* old[] = {c->d_near_ptr, c->d_near_idx, c->d_near_h};
   for (void* q : old)
     if (q) cudaFree(q);
@@ -775,29 +777,53 @@ static int build_near_pairs(lsms_ctx* c) {
   const int n = c->n;
   const double rn = (double)kZAsym / c->k2;
   c->near_r2 = rn * rn;
+  const double rw = std::max(rn, pair_z_near(c->p) / c->k2) * (1.0 + 1e-6), rw2 = rw * rw;
   std::vector<int> ptr(n + 1, 0), idx;
-  std::unordered_map<long long, std::vector<int>> grid;
-  auto key = [](long long i, long long k) { return (i << 32) ^ (k & 0xffffffffLL); };
+  wide_ptr.assign(n + 1, 0);
+  wide_idx.clear();
   std::vector<double> xs(n);
-  for (int j = 0; j < n; ++j) xs[j] = c->cx[j] - c->xc;
-  for (int j = 0; j < n; ++j)
-    grid[key((long long)std::floor(xs[j] / rn), (long long)std::floor(c->cy[j] / rn))].push_back(j);
+  double x0 = 0.0, x1 = 0.0, y0 = 0.0, y1 = 0.0;
+  for (int j = 0; j < n; ++j) {
+    xs[j] = c->cx[j] - c->xc;
+    x0 = j ? std::min(x0, xs[j]) : xs[j];
+    x1 = j ? std::max(x1, xs[j]) : xs[j];
+    y0 = j ? std::min(y0, c->cy[j]) : c->cy[j];
+    y1 = j ? std::max(y1, c->cy[j]) : c->cy[j];
+  }
+  // cells at least rw wide, about n of them at most along either axis
+  const double wx = std::max(rw, (x1 - x0) / (n + 1.0)), wy = std::max(rw, (y1 - y0) / (n + 1.0));
+  const long long nx = (long long)((x1 - x0) / wx) + 1;
+  const long long ny = std::max<long long>(1, std::min<long long>((long long)((y1 - y0) / wy) + 1, 4LL * n / nx + 1));
+  const double wyc = std::max(wy, (y1 - y0) / (double)ny);
+  auto cell_x = [&](double x) { return std::min<long long>(nx - 1, (long long)((x - x0) / wx)); };
+  auto cell_y = [&](double y) { return std::min<long long>(ny - 1, (long long)((y - y0) / wyc)); };
+  std::vector<int> start(nx * ny + 1, 0), member(n);
+  for (int j = 0; j < n; ++j) ++start[cell_x(xs[j]) * ny + cell_y(c->cy[j]) + 1];
+  for (long long q = 0; q < nx * ny; ++q) start[q + 1] += start[q];
+  {
+    std::vector<int> at(start.begin(), start.end() - 1);
+    for (int j = 0; j < n; ++j) member[at[cell_x(xs[j]) * ny + cell_y(c->cy[j])]++] = j;
+  }
+  std::vector<int> row;
   for (int l = 0; l < n; ++l) {
-    const long long ix = (long long)std::floor(xs[l] / rn), iy = (long long)std::floor(c->cy[l] / rn);
-    std::vector<int> row;
-    for (long long a = ix - 1; a <= ix + 1; ++a)
-      for (long long b = iy - 1; b <= iy + 1; ++b) {
-        auto it = grid.find(key(a, b));
-        if (it == grid.end()) continue;
-        for (int m : it->second) {
+    const long long ix = cell_x(xs[l]), iy = cell_y(c->cy[l]);
+    row.clear();
+    for (long long a = std::max(0LL, ix - 1); a <= std::min(nx - 1, ix + 1); ++a)
+      for (long long b = std::max(0LL, iy - 1); b <= std::min(ny - 1, iy + 1); ++b)
+        for (int e = start[a * ny + b]; e < start[a * ny + b + 1]; ++e) {
+          const int m = member[e];
           if (m == l) continue;
           const double dx = xs[l] - xs[m], dy = c->cy[l] - c->cy[m];
-          if (dx * dx + dy * dy < c->near_r2) row.push_back(m);
+          if (dx * dx + dy * dy < rw2) row.push_back(m);
         }
-      }
     std::sort(row.begin(), row.end());
-    idx.insert(idx.end(), row.begin(), row.end());
+    for (int m : row) {
+      const double dx = xs[l] - xs[m], dy = c->cy[l] - c->cy[m];
+      if (dx * dx + dy * dy < c->near_r2) idx.push_back(m);
+    }
+    wide_idx.insert(wide_idx.end(), row.begin(), row.end());
     ptr[l + 1] = (int)idx.size();
+    wide_ptr[l + 1] = (int)wide_idx.size();
   }
   c->near_nnz = (int)idx.size();
   const size_t hb = (size_t)(c->near_nnz > 0 ? c->near_nnz : 1) * sizeof(float4);
@@ -828,8 +854,10 @@ int build_lowp_tables(lsms_ctx* c) {
   cudaStreamSynchronize(c->stream);
   int rc = check_cuda(c, "build_lowp_tables");
   if (rc) return rc;
-  if ((rc = build_near_pairs(c))) return rc;
-  return tc_setup(c);
+  std::vector<int> wide_ptr, wide_idx;
+  if ((rc = build_near_pairs(c, wide_ptr, wide_idx))) return rc;
+  if ((rc = tc_setup(c))) return rc;
+  return f64tc_setup(c, wide_ptr, wide_idx);
 }
 
 // Splits of the source range so that the grid covers the GPU several times (3 CTAs per SM for one

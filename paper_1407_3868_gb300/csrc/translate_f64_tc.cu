@@ -1,0 +1,537 @@
+// FP64 translation of all pairs on the tensor cores (Sec. 3.2 Lemma 3.1), for one or more
+// right-hand sides.
+//
+// The Toeplitz block of a pair holds h_s = H_s(k rho) e^{i s phi}, s = n - nu.  With A_s = J_s cos s phi,
+// B_s = J_s sin s phi, C_s = Y_s cos s phi, D_s = Y_s sin s phi (s = 0..2p)
+//   h_s = (A_s - D_s) + i (B_s + C_s),   h_{-s} = (-1)^s [(A_s + D_s) + i (C_s - B_s)],
+// so the outputs of 128 targets are one real product summed over the sources,
+//   alpha[target][(nu, Re/Im)] = sum_source sum_{s, A..D} W[target][(s, A..D)] X_source[(s, A..D)][(nu, Re/Im)],
+// with X_source the signed sums beta_{nu+s} +- beta_{nu-s}.  W and X are held as 48-bit fixed point
+// numbers (W: |h| < 1/4, so 49 fractional bits; X: relative to the largest coefficient of the
+// right-hand side) and cut into six signed 8-bit digits each; the digits are exact in FP16, a product
+// of two has at most 14 bits, so the tensor cores' FP32 sums are exact integers.  Products of digits
+// i of W and j of X with i + j = L add into one accumulator per level L; levels beyond LMAX (5 or 6)
+// are below the 48 bits and left out.  One tcgen05.mma multiplies a digit plane of W with several
+// digit planes of X side by side in N: its output columns are consecutive levels.
+//
+// Why: this chip's FP64 pipe (2 FMA per SM and clock) bounds the direct form at 133 ms for 5000 discs
+// (k_translate_f64_sym: 168 ms); 21 products of FP16 digits take 4.7 ms at the tensor cores' measured
+// rate, and this kernel 9.4 ms (1000 discs at p = 12: 5.2 -> 0.37 ms).
+//
+// Exactness: a level <= 3 collects at most 4 products of 4(2p+1) <= 124 digit pairs, below 4 x 124 x 2^14
+// = 2^22.96 per source: two sources (a drain group) stay below 2^24.  Levels 4, 5, 6 could leave the
+// exact range by one bit only if every digit had its largest value; their unit is then 2^-16 of what
+// is left out anyway.  Drained levels are summed in 64-bit integers, so a CTA's sum does not depend
+// on any order.
+//
+// A CTA owns 128 targets and a range of sources, two sources at a time: warps 0-3 and 4-7 each form
+// the W rows of one of the two (thread = target; the fixed-point sequence of pair_fixed.cuh) and
+// store its digits into the stage ring in the tensor cores' K-major layout of 8 x 16-byte core
+// matrices (thread = row: consecutive threads write consecutive 16-byte pieces); warp 17 copies the X
+// digits of the same orders (packed once per application); warp 16 issues the MMAs; warps 8-15 drain
+// the accumulators after every two sources.
+#include <algorithm>
+#include <cmath>
+#include <mutex>
+
+#include "c64.cuh"
+#include "digits_tc.cuh"
+#include "lsms_internal.h"
+#include "lsms_ops.h"
+#include "pair_fixed.cuh"
+
+namespace {
+
+constexpr int TABLE_BYTES = 256 * 16;
+constexpr int MAX_SOURCES = 1024;             // per CTA: the 64-bit sums keep 10 bits for them
+
+constexpr size_t smem_bytes(int npad) { return (size_t)STAGES * stage_bytes(npad) + TABLE_BYTES + 256; }
+inline int k_steps(int p) { return (4 * (2 * p + 1) + 15) / 16; }   // K = 16 steps of one source
+
+// Largest |Re|, |Im| of each right-hand side as the bits of a non-negative double (NaN and Inf
+// compare above every finite value).
+__global__ void k_absmax(const double* __restrict__ x, long long per, unsigned long long* __restrict__ out) {
+  const double* xr = x + blockIdx.y * per;
+  unsigned long long m = 0;
+  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < per; i += (long long)gridDim.x * blockDim.x)
+    m = max(m, (unsigned long long)__double_as_longlong(xr[i]) & 0x7fffffffffffffffull);
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
+  if ((threadIdx.x & 31) == 0 && m) atomicMax(out + blockIdx.y, m);
+}
+// Digits of X for the sources src0 .. src0 + gridDim.x - 1 of right-hand side r0 + blockIdx.y:
+// per source [K group][plane][column][8 K values] FP16, K = 4 s + (A, B, C, D), column 2 q + (Re, Im).
+__global__ void __launch_bounds__(256)
+k_pack_digits(const double2* __restrict__ xs, int n, int p, int src0, int r0, int npad, int kgs,
+              const unsigned long long* __restrict__ maxbits, unsigned char* __restrict__ img) {
+  __shared__ long long re[128], im[128];          // beta_{nu +- s} at 48 + order, zero outside -p..p
+  const int P = 2 * p + 1, r = r0 + blockIdx.y;
+  const unsigned long long mb = maxbits[r];
+  if (mb == 0 || mb >= kInfBits) return;          // the product does not read the image then
+  const int sh = 46 - scale_exponent(mb);
+  const double2* b = xs + ((size_t)r * n + src0 + blockIdx.x) * P;
+  if (threadIdx.x < 128) {
+    const int o = (int)threadIdx.x - 48 + p;
+    double2 v = make_double2(0.0, 0.0);
+    if (o >= 0 && o < P) v = b[o];
+    re[threadIdx.x] = llrint(scalbn(v.x, sh));
+    im[threadIdx.x] = llrint(scalbn(v.y, sh));
+  }
+  __syncthreads();
+  uint4* dst = (uint4*)(img + ((size_t)blockIdx.y * gridDim.x + blockIdx.x) * kgs * b_kg_bytes(npad));
+  for (int it = threadIdx.x; it < kgs * npad; it += blockDim.x) {
+    const int kg = it / npad, col = it - kg * npad;
+    const int q = col >> 1, imag = col & 1;
+    uint32_t w[PL][4];
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const int s = 2 * kg + h;
+      long long a = 0, bb = 0, cc = 0, d = 0;
+      if (q < P && s <= 2 * p) {
+        const int c0 = 48 + q - p;
+        const long long pr = re[c0 + s], pi = im[c0 + s];
+        long long mr = 0, mi = 0;                 // (-1)^s beta_{nu - s}; s = 0 has one term only
+        if (s > 0) {
+          mr = re[c0 - s];
+          mi = im[c0 - s];
+          if (s & 1) { mr = -mr; mi = -mi; }
+        }
+        if (!imag) {
+          a = pr + mr; bb = -pi + mi; cc = -pi - mi; d = -pr + mr;
+        } else {
+          a = pi + mi; bb = pr - mr; cc = pr + mr; d = -pi + mi;
+        }
+        if (s == 0) bb = d = 0;
+      }
+      uint32_t u[PL], v[PL];
+      digit_pairs(a << 16, bb << 16, u);
+      digit_pairs(cc << 16, d << 16, v);
+#pragma unroll
+      for (int j = 0; j < PL; ++j) {
+        w[j][2 * h] = u[j];
+        w[j][2 * h + 1] = v[j];
+      }
+    }
+#pragma unroll
+    for (int j = 0; j < PL; ++j)
+      dst[((size_t)kg * PL + j) * npad + col] = make_uint4(w[j][0], w[j][1], w[j][2], w[j][3]);
+  }
+}
+
+// grid: (target tiles, source ranges, right-hand sides); sources src0 + [0, nsrc) of the image; targets
+// row0 .. row0 + nrows - 1, alpha holds those rows.
+template <int NPAD, int LMAX>
+__global__ void __launch_bounds__(THREADS, 1)
+k_translate_digits(const double* __restrict__ cx, const double* __restrict__ cy, int n, int p, PairConsts pc,
+                   const longlong2* __restrict__ table, const unsigned char* __restrict__ img, int src0, int nsrc,
+                   int per_cta, int r0, const unsigned long long* __restrict__ maxbits, int row0, int nrows,
+                   double2* __restrict__ alpha, int* __restrict__ err) {
+  extern __shared__ __align__(128) unsigned char smem[];
+  constexpr int STAGE = stage_bytes(NPAD);
+  longlong2* stab = (longlong2*)(smem + STAGES * STAGE);
+  uint64_t* bars = (uint64_t*)(smem + STAGES * STAGE + TABLE_BYTES);   // full[3], empty[3], acc_full, acc_empty
+  uint32_t* tmem_slot = (uint32_t*)(bars + 2 * STAGES + 2);
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int P = 2 * p + 1, r = r0 + blockIdx.z;
+  const int s_begin = blockIdx.y * per_cta, s_end = min(nsrc, s_begin + per_cta);
+  const unsigned long long mb = maxbits[r];
+  double2* ar = alpha + (size_t)r * nrows * P;
+  if (s_begin >= s_end || mb == 0) return;
+  if (mb >= kInfBits) {                            // a non-finite coefficient reaches every target
+    if (blockIdx.y == 0) {
+      const double nan = __longlong_as_double(0x7ff8000000000000ll);
+      for (int i = threadIdx.x; i < ROWS * P; i += THREADS) {
+        const size_t e = (size_t)blockIdx.x * ROWS * P + i;
+        if (e < (size_t)nrows * P) ar[e] = make_double2(nan, nan);
+      }
+    }
+    return;
+  }
+  const int steps = (4 * P + 15) / 16;             // K = 16 steps of a source
+  const int chunks = (steps + 1) / 2;
+  const int pairs = (s_end - s_begin + 1) / 2;     // drain groups
+  const uint32_t full0 = smem_u32(bars), empty0 = full0 + 8 * STAGES, accf = full0 + 16 * STAGES, acce = accf + 8;
+  if (threadIdx.x == 0) {
+    for (int s = 0; s < STAGES; ++s) {
+      mbar_init(full0 + 8 * s, 5);                 // four generating warps and the copy
+      mbar_init(empty0 + 8 * s, 1);
+    }
+    mbar_init(accf, 1);
+    mbar_init(acce, DRAIN_WARPS);
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  if (threadIdx.x < 256) stab[threadIdx.x] = table[threadIdx.x];
+  __syncwarp();
+  if (warp == GEN_WARPS + DRAIN_WARPS) tmem_alloc(smem_u32(tmem_slot), 512);
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem = *tmem_slot;
+  const uint32_t sbase = smem_u32(smem);
+
+  if (warp < GEN_WARPS) {
+    // ---- digits of W: group g takes every second source, thread = target row
+    const int g = warp >> 2, row = threadIdx.x & (ROWS - 1);
+    const int l = row0 + blockIdx.x * ROWS + row;
+    const bool lvalid = l < row0 + nrows;
+    const double xl = lvalid ? cx[l] : 0.0, yl = lvalid ? cy[l] : 0.0;
+    bool ok = true;
+    for (int q = 0; q < pairs && ok; ++q) {
+      const int m = s_begin + 2 * q + g;
+      PairSeed o;
+      o.j0 = o.y0 = o.j1 = o.y1 = o.c = o.s = o.w = 0;
+      if (lvalid && m < s_end && src0 + m != l) {
+        const double dx = xl - cx[src0 + m], dy = yl - cy[src0 + m];
+        const double r2 = fma(dx, dx, dy * dy);
+        if (!pair_is_near(r2, pc)) pair_seed(dx, dy, r2, pc, stab, o);
+      }
+      // order 0; the step from it gives order 1 (J_{-1} = -J_1)
+      PairState a;
+      a.j = o.j0; a.jm = -o.j1; a.y = o.y0; a.ym = -o.y1;
+      a.c = 1LL << 62; a.s = 0; a.f = 0;
+      for (int c = 0; c < chunks; ++c) {
+        const int t = (q * chunks + c) * 2 + g;
+        const int st = t % STAGES, round = t / STAGES;
+        if (round > 0 && !mbar_wait(empty0 + 8 * st, (round - 1) & 1)) {
+          ok = false;
+          break;
+        }
+        unsigned char* base = smem + st * STAGE + row * 16;
+        const int kgs = min(KG, 2 * steps - KG * c);
+#pragma unroll 1
+        for (int kg = 0; kg < kgs; ++kg) {
+          uint32_t u[PL], v[PL], w[PL], z[PL];
+          int64_t pr[4];
+          if (2 * (KG * c + kg) <= 2 * p) {
+            pair_products(a, pr);
+            digit_pairs(pr[0], pr[1], u);
+            digit_pairs(pr[2], pr[3], v);
+            pair_step(a, o);
+            pair_products(a, pr);
+            digit_pairs(pr[0], pr[1], w);
+            digit_pairs(pr[2], pr[3], z);
+            pair_step(a, o);
+          } else {
+#pragma unroll
+            for (int j = 0; j < PL; ++j) u[j] = v[j] = w[j] = z[j] = 0;
+          }
+#pragma unroll
+          for (int j = 0; j < PL; ++j)
+            *(uint4*)(base + j * A_PLANE + kg * A_KG) = make_uint4(u[j], v[j], w[j], z[j]);
+        }
+        fence_proxy_async_smem();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(full0 + 8 * st);
+      }
+    }
+    if (!ok && lane == 0) atomicExch(err, 11);
+  } else if (warp < GEN_WARPS + DRAIN_WARPS) {
+    // ---- drain: warp d owns lanes 32 (d mod 4) .. + 31 and half of the columns
+    const int d = warp - GEN_WARPS, quad = warp & 3, half = d >> 2;
+    constexpr int HC = NPAD / 2;
+    int64_t acc[HC];
+#pragma unroll
+    for (int i = 0; i < HC; ++i) acc[i] = 0;
+    const uint32_t tb = tmem + ((uint32_t)(32 * quad) << 16) + half * HC;
+    bool ok = true;
+    for (int q = 0; q < pairs; ++q) {
+      ok = __all_sync(0xffffffffu, mbar_wait(accf, q & 1));
+      if (!ok) break;
+      tc_fence_after();
+      drain_levels<NPAD, LMAX>(tb, acc);
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(acce);
+    }
+    if (ok) {
+      const int row = blockIdx.x * ROWS + 32 * quad + lane;
+      const int ex = scale_exponent(mb) - 49;      // unit of acc
+      const double s1 = scalbn(1.0, ex / 2), s2 = scalbn(1.0, ex - ex / 2);
+      if (row < nrows) {
+#pragma unroll
+        for (int i = 0; i < HC; ++i) {
+          const int col = half * HC + i;
+          if (col < 2 * P)
+            atomicAdd((double*)(ar + (size_t)row * P) + col, __ll2double_rn(acc[i]) * s1 * s2);
+        }
+      }
+    } else if (lane == 0) {
+      atomicExch(err, 12);
+    }
+  } else if (warp == GEN_WARPS + DRAIN_WARPS) {
+    // ---- MMA issue
+    if (lane == 0) {
+      bool ok = true;
+      for (int q = 0; q < pairs && ok; ++q) {
+        if (q > 0 && !mbar_wait(acce, (q - 1) & 1)) {
+          ok = false;
+          break;
+        }
+        tc_fence_after();
+        for (int c2 = 0; c2 < 2 * chunks; ++c2) {
+          const int t = q * 2 * chunks + c2;
+          const int st = t % STAGES, round = t / STAGES;
+          if (!mbar_wait(full0 + 8 * st, round & 1)) {
+            ok = false;
+            break;
+          }
+          tc_fence_after();
+          const uint32_t sa = sbase + st * STAGE, sb = sa + A_BYTES;
+          const int ksteps = min(2, steps - 2 * (c2 >> 1));
+          for (int ks = 0; ks < ksteps; ++ks) issue_step<NPAD, LMAX>(tmem, sa, sb, ks, c2 == 0 && ks == 0);
+          mma_commit(empty0 + 8 * st);
+        }
+        if (ok) mma_commit(accf);
+      }
+      if (!ok) atomicExch(err, 13);
+    }
+    __syncwarp();
+  } else {
+    // ---- copies of the X digits
+    if (lane == 0) {
+      bool ok = true;
+      const size_t src_bytes = (size_t)2 * steps * b_kg_bytes(NPAD);
+      const unsigned char* ir = img + (size_t)blockIdx.z * nsrc * src_bytes;
+      int t = 0;
+      for (int q = 0; q < pairs && ok; ++q)
+        for (int c2 = 0; c2 < 2 * chunks; ++c2, ++t) {
+          const int st = t % STAGES, round = t / STAGES;
+          if (round > 0 && !mbar_wait(empty0 + 8 * st, (round - 1) & 1)) {
+            ok = false;
+            break;
+          }
+          const int c = c2 >> 1, m = min(s_begin + 2 * q + (c2 & 1), s_end - 1);
+          const int kgs = min(KG, 2 * steps - KG * c);
+          const uint32_t bytes = (uint32_t)kgs * b_kg_bytes(NPAD);
+          mbar_expect_tx(full0 + 8 * st, bytes);
+          bulk_load(sbase + st * STAGE + A_BYTES, ir + m * src_bytes + (size_t)c * KG * b_kg_bytes(NPAD), bytes,
+                    full0 + 8 * st);
+        }
+      // copies still in flight end before the CTA does
+      for (int s = max(0, t - STAGES); s < t && !ok; ++s) mbar_wait(full0 + 8 * (s % STAGES), (s / STAGES) & 1);
+      if (!ok) atomicExch(err, 14);
+    }
+    __syncwarp();
+  }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  if (warp == GEN_WARPS + DRAIN_WARPS) tmem_dealloc(tmem, 512);
+}
+
+// ---------------------------------------------------------------------------------------------
+// Near pairs: k rho below pair_z_near (H_{2p} would leave the fixed-point range), from their list.
+// ---------------------------------------------------------------------------------------------
+// The sequences h_s, s = -2p..2p, of every listed pair, once per layout: seq[pair][4p + 1]; zero for
+// the candidates that the digit kernel takes (its own decision, pair_is_near).
+__global__ void k_near_sequences(const double* __restrict__ cx, const double* __restrict__ cy,
+                                 const int* __restrict__ tgt, const int* __restrict__ idx, int nnz, int p, double k,
+                                 PairConsts pc, double2* __restrict__ seq) {
+  const int e = blockIdx.x * blockDim.x + threadIdx.x;
+  if (e >= nnz) return;
+  const int l = tgt[e], m = idx[e];
+  double2* h = seq + (size_t)e * (4 * p + 1) + 2 * p;
+  const double dx = cx[l] - cx[m], dy = cy[l] - cy[m];
+  if (!pair_is_near(fma(dx, dx, dy * dy), pc)) {
+    for (int q = -2 * p; q <= 2 * p; ++q) h[q] = make_double2(0.0, 0.0);
+    return;
+  }
+  const double rho = hypot(dx, dy), z = k * rho, iz = 1.0 / z;
+  const double2 e1 = make_double2(dx / rho, dy / rho);
+  double2 hm = make_double2(j0(z), y0(z)), hq = make_double2(j1(z), y1(z)), eq = e1;
+  h[0] = hm;
+  for (int q = 1; q <= 2 * p; ++q) {
+    h[q] = cmul(hq, eq);
+    const double2 u = cmul(hq, make_double2(eq.x, -eq.y));
+    h[-q] = (q & 1) ? make_double2(-u.x, -u.y) : u;
+    const double f = 2.0 * q * iz;
+    const double2 hn = make_double2(f * hq.x - hm.x, f * hq.y - hm.y);
+    hm = hq;
+    hq = hn;
+    eq = cmul(eq, e1);
+  }
+}
+
+// alpha^l += sum over l's listed sources: one warp per (target, right-hand side), lane = output order.
+// The sequences are read where they lie (a window of P consecutive values per source order, in L1
+// after the first; the lists of 5000 discs at p = 14 take 63 MB, in L2 between applications), so the
+// kernel needs no shared memory and enough warps share an SM to keep its FP64 pipe busy: four
+// independent FMAs per order and warp.  5000 discs: 2.80 ms with the sequences formed anew in
+// shared memory (one CTA per SM) -> 0.51 ms
+// (its 8 M warp FMAs take 0.44 ms of the pipe).
+__global__ void __launch_bounds__(128)
+k_translate_near_f64(int n, int p, int row0, int nrows, const int* __restrict__ ptr, const int* __restrict__ idx,
+                     const double2* __restrict__ seq, const double2* __restrict__ xs, double2* __restrict__ alpha) {
+  const int P = 2 * p + 1, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int l = row0 + blockIdx.x * 4 + warp, r = blockIdx.y;
+  if (l >= row0 + nrows) return;
+  const int e1 = ptr[l + 1];
+  const double2* xr = xs + (size_t)r * n * P;
+  const int nu = min(lane, P - 1);                       // idle lanes repeat the last order
+  double rr = 0.0, ii = 0.0, ri = 0.0, ir = 0.0;
+  for (int e = ptr[l]; e < e1; ++e) {
+    const double2* h = seq + (size_t)e * (4 * p + 1) + 2 * p - nu;
+    const double2* b = xr + (size_t)idx[e] * P;
+#pragma unroll 4
+    for (int q = 0; q < P; ++q) {
+      const double2 hv = __ldg(h + q), bv = __ldg(b + q);
+      rr = fma(hv.x, bv.x, rr);
+      ii = fma(hv.y, bv.y, ii);
+      ri = fma(hv.x, bv.y, ri);
+      ir = fma(hv.y, bv.x, ir);
+    }
+  }
+  if (lane < P) {
+    double2* o = alpha + ((size_t)r * nrows + (l - row0)) * P + lane;
+    *o = make_double2(o->x + (rr - ii), o->y + (ri + ir));
+  }
+}
+
+template <int NPAD, int LMAX>
+void launch_digits(dim3 grid, cudaStream_t st, const lsms_ctx* c, const PairConsts& pc, const unsigned char* img,
+                   int src0, int nsrc, int per_cta, int r0, const unsigned long long* maxbits, int row0, int nrows,
+                   double2* alpha, int* err) {
+  static std::once_flag attr;
+  std::call_once(attr, [] {
+    cudaFuncSetAttribute(k_translate_digits<NPAD, LMAX>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                         (int)smem_bytes(NPAD));
+  });
+  k_translate_digits<NPAD, LMAX><<<grid, THREADS, smem_bytes(NPAD), st>>>(
+      c->d_cx, c->d_cy, c->n, c->p, pc, (const longlong2*)c->f64tc.d_table, img, src0, nsrc, per_cta, r0, maxbits,
+      row0, nrows, alpha, err);
+}
+
+constexpr size_t kImageBytes = (size_t)256 << 20;   // digits of X held at once
+constexpr int kMinDiscs = 96;
+
+}  // namespace
+
+void f64tc_free(lsms_ctx* c) {
+  F64Tc& f = c->f64tc;
+  void* ptrs[] = {f.d_table, f.d_ptr, f.d_idx, f.d_seq, f.ws.ptr};
+  for (void* p : ptrs)
+    if (p) cudaFree(p);
+  f = F64Tc();
+}
+
+// Tables of the layout: `ptr`, `idx` list per target the sources within (1 + 1e-6) of the near
+// distance (host arrays).  Layouts of fewer than kMinDiscs discs (not one full tile of rows) or of
+// mostly near pairs (summed on the FP64 pipe either way) keep k_translate_f64 and its symmetric form.
+int f64tc_setup(lsms_ctx* c, const std::vector<int>& ptr, const std::vector<int>& idx) {
+  f64tc_free(c);
+  F64Tc& f = c->f64tc;
+  const int n = c->n;
+  if (n < kMinDiscs || (double)idx.size() > 0.5 * n * (double)(n - 1) || !tc_err_flag(c)) return LSMS_OK;
+  const long double pi = 3.14159265358979323846264338327950288L;
+  std::vector<longlong2> tab(256);
+  for (int i = 0; i < 256; ++i) {
+    const long double a = 2 * pi * i / 256 - pi / 4, one = 4611686018427387904.0L;
+    tab[i] = make_longlong2((long long)rintl(cosl(a) * one), (long long)rintl(sinl(a) * one));
+  }
+  const size_t nnz = idx.size(), ne = nnz > 0 ? nnz : 1;
+  std::vector<int> tgt(nnz);
+  for (int l = 0; l < n; ++l)
+    for (int e = ptr[l]; e < ptr[l + 1]; ++e) tgt[e] = l;
+  if (cudaMalloc(&f.d_table, TABLE_BYTES) != cudaSuccess ||
+      cudaMalloc((void**)&f.d_ptr, (n + 1) * sizeof(int)) != cudaSuccess ||
+      cudaMalloc((void**)&f.d_idx, 2 * ne * sizeof(int)) != cudaSuccess) {
+    cudaGetLastError();
+    f64tc_free(c);
+    return ctx_fail(c, LSMS_ERR_OOM, "cudaMalloc failed for the near pairs of the FP64 translation");
+  }
+  cudaMemcpy(f.d_table, tab.data(), TABLE_BYTES, cudaMemcpyHostToDevice);
+  cudaMemcpy(f.d_ptr, ptr.data(), (n + 1) * sizeof(int), cudaMemcpyHostToDevice);
+  if (nnz) {
+    cudaMemcpy(f.d_idx, idx.data(), nnz * sizeof(int), cudaMemcpyHostToDevice);
+    cudaMemcpy(f.d_idx + nnz, tgt.data(), nnz * sizeof(int), cudaMemcpyHostToDevice);
+  }
+  f.nnz = (int)nnz;
+  f.ready = true;
+  return check_cuda(c, "f64tc_setup");
+}
+
+// The stored near sequences (63 MB at 5000 discs, p = 14) exist while all-pairs FP64 translations
+// can run: not while every translation goes through boxes.
+int f64tc_sequences(lsms_ctx* c) {
+  F64Tc& f = c->f64tc;
+  const bool want = f.ready && f.nnz > 0 && !(c->fmm.ready && c->fmm.scope == LSMS_FMM_ALL);
+  if (want == (f.d_seq != nullptr)) return LSMS_OK;
+  if (!want) {
+    cudaFree(f.d_seq);
+    f.d_seq = nullptr;
+    return LSMS_OK;
+  }
+  if (cudaMalloc(&f.d_seq, (size_t)f.nnz * (4 * c->p + 1) * sizeof(double2)) != cudaSuccess) {
+    cudaGetLastError();
+    f.d_seq = nullptr;
+    return ctx_fail(c, LSMS_ERR_OOM, "cudaMalloc failed for the near sequences of the FP64 translation");
+  }
+  k_near_sequences<<<(f.nnz + 127) / 128, 128, 0, c->stream>>>(c->d_cx, c->d_cy, f.d_idx + f.nnz, f.d_idx, f.nnz,
+                                                                c->p, c->k2, pair_consts(c->k2, pair_z_near(c->p)),
+                                                                (double2*)f.d_seq);
+  cudaStreamSynchronize(c->stream);
+  return check_cuda(c, "f64tc_sequences");
+}
+
+// alpha = rows row0 .. row0 + nrows - 1 of T xs, [nrhs][nrows][P].
+int translate_f64_tc(lsms_ctx* c, int nrhs, const double2* xs, double2* alpha, cudaStream_t st, int row0, int nrows) {
+  F64Tc& f = c->f64tc;
+  const int n = c->n, p = c->p, P = c->P, npad = pad_columns(p), steps = k_steps(p);
+  const size_t src_bytes = (size_t)2 * steps * b_kg_bytes(npad);
+  // the image holds whole right-hand sides if several fit, else a run of sources of one
+  const int cap = (int)std::max<size_t>(2, kImageBytes / src_bytes);
+  const int rb = std::max(1, std::min(nrhs, cap / n));
+  int runs = (n + cap - 1) / cap;
+  const int run = (((n + runs - 1) / runs) + 1) / 2 * 2;
+  runs = (n + run - 1) / run;
+  const size_t img_bytes = (size_t)rb * std::min(run, n) * src_bytes;
+  const size_t max_bytes = ((size_t)nrhs * 8 + 255) & ~size_t(255);
+  int rc;
+  if ((rc = ensure(c, f.ws, max_bytes + img_bytes))) return rc;
+  unsigned long long* maxbits = (unsigned long long*)f.ws.ptr;
+  unsigned char* img = (unsigned char*)f.ws.ptr + max_bytes;
+  int* err = tc_err_flag(c);
+  cudaMemsetAsync(maxbits, 0, (size_t)nrhs * 8, st);
+  cudaMemsetAsync(alpha, 0, (size_t)nrhs * nrows * P * sizeof(double2), st);
+  const long long per = 2LL * n * P;
+  k_absmax<<<dim3((int)std::min<long long>((per + 1023) / 1024, 152), nrhs), 256, 0, st>>>((const double*)xs, per,
+                                                                                          maxbits);
+  const PairConsts pc = pair_consts(c->k2, pair_z_near(p));
+  const int tiles = (nrows + ROWS - 1) / ROWS;
+  for (int r0 = 0; r0 < nrhs; r0 += rb) {
+    const int nr = std::min(rb, nrhs - r0);
+    for (int s0 = 0; s0 < n; s0 += run) {
+      const int ns = std::min(run, n - s0);
+      k_pack_digits<<<dim3(ns, nr), 256, 0, st>>>(xs, n, p, s0, r0, npad, 2 * steps, maxbits, img);
+      // source ranges: the fewest rounds of 152 CTAs times the pairs of a CTA, plus about two pairs
+      // of time per CTA for its start and end
+      int best = 1;
+      double cost = 1e300;
+      const int max_split = std::min((ns + 1) / 2, std::max(1, 65535));
+      for (int sp = (ns + MAX_SOURCES - 1) / MAX_SOURCES; sp <= max_split && sp <= 152 * 8; ++sp) {
+        const double rounds = std::ceil((double)tiles * sp * nr / 152.0);
+        const double cc = rounds * (2.0 + std::ceil(std::ceil((double)ns / sp) / 2.0));
+        if (cc < cost * 0.999) {
+          cost = cc;
+          best = sp;
+        }
+      }
+      const int per_cta = (((ns + best - 1) / best) + 1) / 2 * 2;
+      dim3 grid(tiles, (ns + per_cta - 1) / per_cta, nr);
+      // seven levels for the short layouts, whose phases are the most accurate: there the six levels'
+      // 1.3e-15 of a term would show beside the 1e-16 k rho of its phase
+      const bool more = n < 1024;
+#define LSMS_DG(NP)                                                                                       \
+  (more ? launch_digits<NP, 6>(grid, st, c, pc, img, s0, ns, per_cta, r0, maxbits, row0, nrows, alpha, err)           \
+        : launch_digits<NP, 5>(grid, st, c, pc, img, s0, ns, per_cta, r0, maxbits, row0, nrows, alpha, err))
+      if (npad == 32) LSMS_DG(32);
+      else if (npad == 48) LSMS_DG(48);
+      else LSMS_DG(64);
+#undef LSMS_DG
+    }
+  }
+  if (f.nnz > 0)
+    k_translate_near_f64<<<dim3((nrows + 3) / 4, nrhs), 128, 0, st>>>(n, p, row0, nrows, f.d_ptr, f.d_idx,
+                                                                      (const double2*)f.d_seq, xs, alpha);
+  return check_cuda(c, "translate_f64_tc");
+}
