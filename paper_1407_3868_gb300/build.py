@@ -11,7 +11,7 @@ ROOT = os.path.dirname(HERE)
 CSRC = os.path.join(HERE, "csrc")
 OUT_DIR = os.path.join(HERE, "_build")
 LIB = os.path.join(OUT_DIR, "liblsms.so")
-SOURCES = ["abi.cu", "kernels_f64.cu", "mixed.cu", "contour_tc.cu", "translate_tc.cu", "translate_f64_tc.cu", "gmres.cu", "batch.cu",
+SOURCES = ["abi.cu", "kernels_f64.cu", "mixed.cu", "contour_tc.cu", "translate_tc.cu", "translate_f64_tc.cu", "contour_f64_tc.cu", "contour_direct.cu", "gmres.cu", "batch.cu",
            "host_setup.cpp", "inclusion.cpp", "fmm.cu"]
 # The benchmark's FMA-pipe probe: a library of its own, outside the lsms ABI.
 PROBE_SRC = os.path.join(CSRC, "probe", "fma_probe.cu")

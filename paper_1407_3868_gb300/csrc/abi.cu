@@ -88,11 +88,14 @@ int reflection_f64(lsms_ctx* c, int nrhs, const double2* xs, double2* alpha, cud
   if ((rc = ensure(c, c->ws_v, (size_t)nrhs * 2 * ns * P * sizeof(double2)))) return rc;
   double2* G = (double2*)c->ws_g.ptr;
   double2* V = (double2*)c->ws_v.ptr;
+  if ((double)2 * ns * n < kZgemmMinTable) {
+    launch_node_direct(ns, n, P, nrhs, c->d_eagg, xs, c->d_fagg, c->d_refl, c->d_udis, V, st);
+    return zgemm_f64(c, false, nrhs, V, alpha, st);
+  }
   cudaMemsetAsync(G, 0, (size_t)nrhs * 2 * ns * P * sizeof(double2), st);
-  launch_zgemm_rows(c->d_eagg, 2 * ns, n, xs, G, P, nrhs, st);
+  if ((rc = zgemm_f64(c, true, nrhs, xs, G, st))) return rc;
   launch_node_stage(ns, P, nrhs, G, c->d_fagg, nullptr, c->d_refl, c->d_udis, nullptr, nullptr, V, st);
-  launch_zgemm_rows(c->d_edis, n, 2 * ns, V, alpha, P, nrhs, st);
-  return LSMS_OK;
+  return zgemm_f64(c, false, nrhs, V, alpha, st);
 }
 
 // y = x - s_out (T + R)(s_in x) on device buffers (the operator of lsms_apply_dev).
@@ -141,7 +144,7 @@ int apply_device(lsms_ctx* c, int nrhs, const double2* x, double2* y, int flags,
       launches += 3 + (c->near_nnz > 0 ? 1 : 0);
       if ((rc = translate_mixed(c, nrhs, xs, alpha, st))) return rc;
     } else {
-      launches += c->f64tc.ready ? 3 + (c->f64tc.nnz > 0 ? 1 : 0) : 1;
+      launches += c->f64tc.digits ? 3 + (c->f64tc.nnz > 0 ? 1 : 0) : 1;
       if ((rc = translate_f64(c, nrhs, xs, alpha, st))) return rc;
     }
   } else {
@@ -385,6 +388,7 @@ extern "C" void lsms_destroy(lsms_ctx* c) {
   tc_free(c);
   fmm_free(c);
   f64tc_free(c);
+  zgemm_free(c);
   if (c->h_pinned) cudaFreeHost(c->h_pinned);
   if (c->gm_ring) cudaFreeHost(c->gm_ring);
   for (cudaEvent_t e : c->ev)
@@ -421,6 +425,7 @@ extern "C" int lsms_set_particles(lsms_ctx* c, int n, const double* xy) {
   for (int j = 0; j < n; ++j) xs[j] = c->cx[j] - c->xc;
   tc_free(c);
   f64tc_free(c);
+  zgemm_free(c);
   void* old[] = {c->d_cx, c->d_cy, c->d_eagg, c->d_edis, c->d_eagg_lp, c->d_edis_lp, c->d_lp_misc};
   for (void* q : old)
     if (q) cudaFree(q);
@@ -551,7 +556,7 @@ extern "C" int lsms_aggregate(lsms_ctx* c, int nrhs, const double* beta, double*
   if (precision == LSMS_MIXED) {
     if ((rc = aggregate_mixed(c, nrhs, (const double2*)c->ws_x.ptr, G, c->stream))) return rc;
   } else {
-    launch_zgemm_rows(c->d_eagg, 2 * ns, c->n, (const double2*)c->ws_x.ptr, G, P, nrhs, c->stream);
+    if ((rc = zgemm_f64(c, true, nrhs, (const double2*)c->ws_x.ptr, G, c->stream))) return rc;
   }
   launch_node_stage(ns, P, nrhs, G, c->d_fagg, nullptr, nullptr, nullptr, (double2*)c->ws_pq.ptr,
                     nullptr, nullptr, c->stream);
@@ -625,7 +630,7 @@ extern "C" int lsms_disaggregate(lsms_ctx* c, int nrhs, const double* s_plus, co
   if (precision == LSMS_MIXED) {
     if ((rc = disaggregate_mixed(c, nrhs, (const double2*)c->ws_v.ptr, (double2*)c->ws_alpha.ptr, c->stream))) return rc;
   } else {
-    launch_zgemm_rows(c->d_edis, c->n, 2 * ns, (const double2*)c->ws_v.ptr, (double2*)c->ws_alpha.ptr, P, nrhs, c->stream);
+    if ((rc = zgemm_f64(c, false, nrhs, (const double2*)c->ws_v.ptr, (double2*)c->ws_alpha.ptr, c->stream))) return rc;
   }
   if ((rc = check_cuda(c, "disaggregate"))) return rc;
   if ((rc = copy_out(c, alpha, c->ws_alpha.ptr, len))) return rc;
@@ -641,7 +646,7 @@ int incident_device(lsms_ctx* c, int nsrc, const double* d_src, double2* out, cu
   launch_incident_sigma(ns, nsrc, d_src, c->xc, c->d_lam, c->d_g1, c->d_inc, (double2*)c->ws_sig.ptr, st);
   launch_sigma_to_v(ns, P, nsrc, (const double2*)c->ws_sig.ptr, c->d_udis, (double2*)c->ws_v.ptr, st);
   cudaMemsetAsync(out, 0, (size_t)nsrc * c->n * P * sizeof(double2), st);
-  launch_zgemm_rows(c->d_edis, c->n, 2 * ns, (const double2*)c->ws_v.ptr, out, P, nsrc, st);
+  if ((rc = zgemm_f64(c, false, nsrc, (const double2*)c->ws_v.ptr, out, st))) return rc;
   return check_cuda(c, "incident");
 }
 
@@ -696,7 +701,7 @@ extern "C" int lsms_eval_field(lsms_ctx* c, int src_index, int ntgt, const doubl
     double2* G = (double2*)c->ws_g.ptr;
     cudaMemsetAsync(G, 0, (size_t)2 * ns * P * sizeof(double2), c->stream);
     const double2* beta = (const double2*)c->sol.ptr + (size_t)src_index * c->n * P;
-    launch_zgemm_rows(c->d_eagg, 2 * ns, c->n, beta, G, P, 1, c->stream);
+    if ((rc = zgemm_f64(c, true, 1, beta, G, c->stream))) return rc;
     launch_node_stage(ns, P, 1, G, c->d_fagg, nullptr, nullptr, nullptr, (double2*)c->ws_pq.ptr,
                       nullptr, nullptr, c->stream);
     pq = (const double2*)c->ws_pq.ptr;

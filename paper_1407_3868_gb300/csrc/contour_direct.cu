@@ -1,0 +1,84 @@
+// FP64 contour contractions of small tables (below 1.5e5 complex elements) on the FP64 pipe: a warp per
+// output row, lane = output order, the table element a broadcast and the right operand's row a
+// coalesced load.  What bounds them is latency, so the aggregate, the order sums, the reflection and
+// the disaggregate's right operand are one kernel (a warp per contour node), and K is cut so that the
+// products spread over the chip.  16 discs, 256 nodes:
+// 15 and 8 us for the two kernels, 32 us the whole reflected coupling with its neighbours (98 us with
+// tiled products in shared memory).
+#include <algorithm>
+
+#include "c64.cuh"
+#include "lsms_internal.h"
+#include "lsms_ops.h"
+
+namespace {
+
+// sum_{k0 <= k < k1} a[k] b[k][lane] over the P orders (idle lanes repeat the last one)
+__device__ __forceinline__ double2 row_sum(const double2* __restrict__ a, const double2* __restrict__ b, int P, int q,
+                                           int k0, int k1) {
+  double rr = 0.0, ii = 0.0, ri = 0.0, ir = 0.0;
+#pragma unroll 4
+  for (int k = k0; k < k1; ++k) {
+    const double2 u = __ldg(a + k), v = __ldg(b + (size_t)k * P + q);
+    rr = fma(u.x, v.x, rr);
+    ii = fma(u.y, v.y, ii);
+    ri = fma(u.x, v.y, ri);
+    ir = fma(u.y, v.x, ir);
+  }
+  return make_double2(rr - ii, ri + ir);
+}
+
+// C[r][m][q] += sum_k A[m][k] B[r][k][q]; a warp per (row, K range, right-hand side).
+__global__ void __launch_bounds__(128)
+k_zgemm_direct(const double2* __restrict__ A, int M, int K, const double2* __restrict__ B, double2* __restrict__ C,
+               int P, int per) {
+  const int w = blockIdx.x * 4 + (threadIdx.x >> 5), lane = threadIdx.x & 31, r = blockIdx.y;
+  const int chunks = (K + per - 1) / per, m = w / chunks;
+  if (m >= M) return;
+  const int k0 = (w - m * chunks) * per;
+  const double2 s = row_sum(A + (size_t)m * K, B + (size_t)r * K * P, P, min(lane, P - 1), k0, min(K, k0 + per));
+  if (lane < P) {
+    double* o = (double*)(C + ((size_t)r * M + m) * P + lane);
+    atomicAdd(o, s.x);
+    atomicAdd(o + 1, s.y);
+  }
+}
+
+// Per contour node (warp): G = E_agg x for its two rows, the order sums P+, Q-, the reflection and
+// V = U sigma (k_node_stage with the aggregate inside).
+__global__ void __launch_bounds__(128)
+k_node_direct(int ns, int n, int P, const double2* __restrict__ eagg, const double2* __restrict__ xs,
+              const double2* __restrict__ fagg, const double2* __restrict__ refl, const double2* __restrict__ udis,
+              double2* __restrict__ V) {
+  const int v = blockIdx.x * 4 + (threadIdx.x >> 5), lane = threadIdx.x & 31, r = blockIdx.y;
+  if (v >= ns) return;
+  const int q = min(lane, P - 1);
+  const double2* b = xs + (size_t)r * n * P;
+  double2 gp = row_sum(eagg + (size_t)v * n, b, P, q, 0, n);
+  double2 gm = row_sum(eagg + (size_t)(ns + v) * n, b, P, q, 0, n);
+  gp = lane < P ? cmul(fagg[(size_t)v * P + q], gp) : make_double2(0.0, 0.0);
+  gm = lane < P ? cmul(fagg[(size_t)(ns + v) * P + q], gm) : make_double2(0.0, 0.0);
+  const double2 Pp = warp_sum(gp), Qm = warp_sum(gm);
+  const double2 sp = cadd(cmul(refl[4 * v], Pp), cmul(refl[4 * v + 1], Qm));
+  const double2 sm = cadd(cmul(refl[4 * v + 2], Pp), cmul(refl[4 * v + 3], Qm));
+  if (lane < P) {
+    V[((size_t)r * 2 * ns + v) * P + lane] = cmul(udis[(size_t)v * P + lane], sp);
+    V[((size_t)r * 2 * ns + ns + v) * P + lane] = cmul(udis[(size_t)(ns + v) * P + lane], sm);
+  }
+}
+
+}  // namespace
+
+void launch_zgemm_direct(const double2* A, int M, int K, const double2* B, double2* C, int P, int nrhs,
+                         cudaStream_t st) {
+  if (M == 0 || K == 0 || nrhs == 0) return;
+  // about 16 warps per SM, at least 16 elements of K each
+  const int chunks = (int)std::max<long long>(1, std::min<long long>((K + 15) / 16, 152LL * 16 / std::max(1LL, (long long)M * nrhs)));
+  const int per = (K + chunks - 1) / chunks, nc = (K + per - 1) / per;
+  k_zgemm_direct<<<dim3((unsigned)(((long long)M * nc + 3) / 4), nrhs), 128, 0, st>>>(A, M, K, B, C, P, per);
+}
+
+void launch_node_direct(int ns, int n, int P, int nrhs, const double2* eagg, const double2* xs, const double2* fagg,
+                        const double2* refl, const double2* udis, double2* V, cudaStream_t st) {
+  k_node_direct<<<dim3((ns + 3) / 4, nrhs), 128, 0, st>>>(ns, n, P, eagg, xs, fagg, refl, udis, V);
+}

@@ -1,9 +1,11 @@
-// Products of 48-bit fixed-point operands on the tensor cores (the FP64 translation,
-// translate_f64_tc.cu).
+// Products of 48-bit fixed-point operands on the tensor cores, shared by the FP64 translation
+// (translate_f64_tc.cu) and the FP64 contour contractions (contour_f64_tc.cu).
 //
 // Both operands W (128 rows per CTA) and X (NPAD columns) are cut into six balanced 8-bit digits held
 // as FP16 integers; digit products have at most 14 bits and the FP32 accumulators sum them exactly
-// while a level's sum stays below 2^24.  Level L collects the products of W digit i and X digit j with
+// while a level's sum stays below 2^24: levels 0 to 3 collect at most four products per K value, so
+// 256 K values always fit before the accumulators are drained into 64-bit integers.  The lowest levels
+// may leave the exact range; their unit is far below what is left out.  Level L collects the products of W digit i and X digit j with
 // i + j = L, weight 2^(8 (10 - L)); its NPAD columns follow those of level L - 1 in tensor memory, so
 // that one tcgen05.mma of W plane i with several X planes side by side in N fills consecutive levels.
 //
@@ -14,19 +16,20 @@
 
 #include <cuda_fp16.h>
 
+#include "fixed64.cuh"
 #include "tc_ptx.cuh"
 
 namespace {
 
 constexpr int PL = 6;                         // digit planes of either operand
 constexpr int ROWS = 128;                     // rows of W (MMA M) per CTA
-constexpr int KG = 4;                         // groups of 8 K values per stage
+constexpr int KG = 4;                         // groups of 8 K values per stage: two MMA steps of K = 16
 constexpr int A_KG = ROWS * 16;               // bytes of one K group of one plane
 constexpr int A_PLANE = KG * A_KG;
 constexpr int A_BYTES = PL * A_PLANE;         // 49152
 constexpr int STAGES = 3;
-constexpr int GEN_WARPS = 8, DRAIN_WARPS = 8;
-constexpr int THREADS = (GEN_WARPS + DRAIN_WARPS + 2) * 32;
+constexpr int DRAIN_WARPS = 8;
+constexpr int DRAIN = 8;                      // stages per drain: 256 K values, 4 products x 256 x 2^14 = 2^24
 
 __host__ __device__ constexpr int b_kg_bytes(int npad) { return PL * npad * 16; }
 __host__ __device__ constexpr int stage_bytes(int npad) { return A_BYTES + KG * b_kg_bytes(npad); }
@@ -51,11 +54,11 @@ __device__ __forceinline__ void tmem_ld4(uint32_t taddr, uint32_t* v) {
 }
 __device__ __forceinline__ void tmem_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
 
-// The six balanced digits of two 48-bit values (bits 16..63 of a and b, most significant first) as
-// pairs of FP16 integers in [-128, 127]: byte + 128 sits in the low mantissa bits of 1024 + byte.
-__device__ __forceinline__ void digit_pairs(int64_t a, int64_t b, uint32_t* out) {
-  const uint64_t bias = 0x8080808080808000ull;     // +128 per digit, and half a unit to round
-  const uint64_t wa = (uint64_t)a + bias, wb = (uint64_t)b + bias;
+// The six balanced digits of two 48-bit values (bits 16..63 of wa and wb less kDigitBias, most
+// significant first) as pairs of FP16 integers in [-128, 127]: byte + 128 sits in the low mantissa
+// bits of 1024 + byte.
+constexpr uint64_t kDigitBias = 0x8080808080808000ull;   // +128 per digit, and half a unit to round
+__device__ __forceinline__ void biased_digit_pairs(uint64_t wa, uint64_t wb, uint32_t* out) {
   const uint32_t ah = (uint32_t)(wa >> 32), al = (uint32_t)wa, bh = (uint32_t)(wb >> 32), bl = (uint32_t)wb;
   const uint32_t t0 = __byte_perm(ah, bh, 0x6273);  // a3 b3 a2 b2 (byte 3 the most significant)
   const uint32_t t1 = __byte_perm(ah, bh, 0x4051);  // a1 b1 a0 b0
@@ -74,18 +77,21 @@ __device__ __forceinline__ void digit_pairs(int64_t a, int64_t b, uint32_t* out)
   out[4] = pair(t2, 0x4140);
   out[5] = pair(t2, 0x4342);
 }
+__device__ __forceinline__ void digit_pairs(int64_t a, int64_t b, uint32_t* out) {
+  biased_digit_pairs((uint64_t)a + kDigitBias, (uint64_t)b + kDigitBias, out);
+}
 
 // Levels of one accumulated element -> units of level 5 / 64, added to acc.
 template <int LMAX>
 __device__ __forceinline__ void add_levels(int64_t& acc, const uint32_t* f) {
   int lo = __float2int_rn(__uint_as_float(f[5]));
   if (LMAX >= 6) lo += (__float2int_rn(__uint_as_float(f[6])) + 128) >> 8;
-  int64_t s = (int64_t)__float2int_rn(__uint_as_float(f[4])) * 4 + ((lo + 32) >> 6);
-  s += (int64_t)__float2int_rn(__uint_as_float(f[3])) * (1 << 10);
-  s += (int64_t)__float2int_rn(__uint_as_float(f[2])) * (1 << 18);
-  s += (int64_t)__float2int_rn(__uint_as_float(f[1])) * (1 << 26);
-  s += (int64_t)(__float2int_rn(__uint_as_float(f[0])) * 16) * (1 << 30);
-  acc += s;
+  acc = mad_wide((lo + 32) >> 6, 1, acc);
+  acc = mad_wide(__float2int_rn(__uint_as_float(f[4])), 1 << 2, acc);
+  acc = mad_wide(__float2int_rn(__uint_as_float(f[3])), 1 << 10, acc);
+  acc = mad_wide(__float2int_rn(__uint_as_float(f[2])), 1 << 18, acc);
+  acc = mad_wide(__float2int_rn(__uint_as_float(f[1])), 1 << 26, acc);
+  acc = mad_wide(__float2int_rn(__uint_as_float(f[0])) * 16, 1 << 30, acc);
 }
 
 constexpr unsigned long long kInfBits = 0x7ff0000000000000ull;
@@ -97,7 +103,21 @@ __device__ __forceinline__ int scale_exponent(unsigned long long bits) {
   return m > 0.99 ? e + 1 : e;
 }
 
-// The MMAs of one K = 16 step `ks` of the stage at sa (W) and sb (X); `first`: the step that starts
+// v 2^ex, rounded to nearest, in integer instructions (the FP64 pipe takes 64 cycles of a scheduler
+// per warp instruction).
+__device__ __forceinline__ double fixed_to_double(int64_t v, int ex) {
+  if (v == 0) return 0.0;
+  const uint64_t u = v < 0 ? 0ull - (uint64_t)v : (uint64_t)v;
+  const int lz = __clzll((long long)u);
+  const uint64_t m = u << lz;
+  const uint64_t keep = (m >> 11) + ((m >> 10) & 1);          // 53 bits, or 2^53
+  const int e = 63 - lz + ex + 1022;                          // exponent field less one: keep brings the other
+  if (e < 1 || e > 2044) return scalbn(scalbn(__ll2double_rn(v), ex / 2), ex - ex / 2);
+  const uint64_t bits = ((uint64_t)e << 52) + keep;
+  return __longlong_as_double((long long)(v < 0 ? bits | 0x8000000000000000ull : bits));
+}
+
+// The MMAs of step `ks` of the stage at sa (W) and sb (X); `first`: the step that starts
 // the accumulators (W plane 0 covers levels 0..5; level 6 starts with W plane 1 and X plane 5, issued
 // apart).
 template <int NPAD, int LMAX>

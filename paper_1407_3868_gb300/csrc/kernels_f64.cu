@@ -258,55 +258,6 @@ __global__ void k_etables(const double* __restrict__ cx, const double* __restric
 }
 
 // ---------------------------------------------------------------------------------------------
-// C[r][m][n] += sum_k A[m][k] B[r][k][n]  (complex FP64, split-K with atomics)
-// ---------------------------------------------------------------------------------------------
-constexpr int GT = 32;
-
-__global__ void __launch_bounds__(256)
-k_zgemm_rows(const double2* __restrict__ A, int M, int K, const double2* __restrict__ B,
-             double2* __restrict__ C, int P, int kchunk) {
-  __shared__ double2 As[GT][GT + 1];
-  __shared__ double2 Bs[GT][GT + 1];
-  const int r = blockIdx.y;
-  const int m0 = blockIdx.x * GT;
-  const int kbeg = blockIdx.z * kchunk;
-  const int kend = min(K, kbeg + kchunk);
-  const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
-  const double2* Br = B + (size_t)r * K * P;
-  double2 acc[4];
-#pragma unroll
-  for (int q = 0; q < 4; ++q) acc[q] = make_double2(0.0, 0.0);
-  for (int k0 = kbeg; k0 < kend; k0 += GT) {
-    for (int e = threadIdx.x; e < GT * GT; e += blockDim.x) {
-      const int i = e >> 5, kk = e & 31;
-      const int m = m0 + i, kx = k0 + kk;
-      As[i][kk] = (m < M && kx < kend) ? A[(size_t)m * K + kx] : make_double2(0.0, 0.0);
-      const int nn = kk;   // reuse e for B: row i is k, column kk is n
-      Bs[i][nn] = (k0 + i < kend && nn < P) ? Br[(size_t)(k0 + i) * P + nn] : make_double2(0.0, 0.0);
-    }
-    __syncthreads();
-#pragma unroll 4
-    for (int kk = 0; kk < GT; ++kk) {
-      const double2 b = Bs[kk][tx];
-#pragma unroll
-      for (int q = 0; q < 4; ++q) acc[q] = cfma(As[ty + 8 * q][kk], b, acc[q]);
-    }
-    __syncthreads();
-  }
-  if (tx < P) {
-#pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      const int m = m0 + ty + 8 * q;
-      if (m < M) {
-        double2* c = C + ((size_t)r * M + m) * P + tx;
-        atomicAdd(&c->x, acc[q].x);
-        atomicAdd(&c->y, acc[q].y);
-      }
-    }
-  }
-}
-
-// ---------------------------------------------------------------------------------------------
 // Per-node stage: order dots (aggregate epilogue), reflection (Eq. "sommerfeldsys" closed form),
 // and the disaggregate's right operand V = U * sigma.
 // G, V: [r][2ns][P]; pq, sig: [r][2][ns].
@@ -493,20 +444,6 @@ void launch_etables(const double* cx, const double* cy, int n, const double2* la
   const long long total = (long long)ns * n;
   if (total == 0) return;
   k_etables<<<grid_for(total, 256), 256, 0, st>>>(cx, cy, n, lam, g2, ns, d, eagg, edis);
-}
-
-void launch_zgemm_rows(const double2* A, int M, int K, const double2* B, double2* C, int P,
-                       int nrhs, cudaStream_t st) {
-  if (M == 0 || K == 0 || nrhs == 0) return;
-  const int mt = (M + GT - 1) / GT;
-  const int kt = (K + GT - 1) / GT;
-  int split = (152 * 4 + mt * nrhs - 1) / (mt * nrhs);
-  if (split > kt) split = kt;
-  if (split < 1) split = 1;
-  const int kchunk = ((kt + split - 1) / split) * GT;
-  split = (K + kchunk - 1) / kchunk;
-  dim3 grid(mt, nrhs, split);
-  k_zgemm_rows<<<grid, 256, 0, st>>>(A, M, K, B, C, P, kchunk);
 }
 
 void launch_node_stage(int ns, int P, int nrhs, const double2* G, const double2* fagg,

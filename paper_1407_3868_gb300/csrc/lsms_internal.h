@@ -65,6 +65,7 @@ struct FmmState {
   int* d_cptr = nullptr;            // [n + 1] mixed near field: pairs in the same or adjacent box by
   int* d_csrc = nullptr;            //   target in box order, source disc of each pair
   float2* d_cseq = nullptr;         // [pairs][4p + 2] their Hankel sequences (FP64-built, stored FP32)
+  double2* d_cseq64 = nullptr;      // [pairs][4p + 1] the same in FP64 (null: formed anew, k_fmm_near)
   float2* d_tab32 = nullptr;        // FP32 copies of the shift tables, the transformed kernel, the
   float2* d_khat32 = nullptr;       // work array, the box coefficients and expansions, the
   float2* d_grid32 = nullptr;       // direct-offset kernels and the twiddles (mixed-precision far
@@ -81,13 +82,21 @@ struct FmmState {
 
 // FP64 translation on the tensor cores (translate_f64_tc.cu): tables of the current layout.
 struct F64Tc {
-  bool ready = false;               // the layout's FP64 all-pairs translation runs there
+  bool ready = false;               // the layout's FP64 all-pairs translation runs there:
+  bool digits = false;              //   far pairs as digits, or all pairs from stored sequences
   void* d_table = nullptr;          // longlong2 [256]: e^{i (2 pi j / 256 - pi / 4)} in Q62
   int* d_ptr = nullptr;             // [n + 1] near pairs (k2 rho below pair_z_near) by target
   int* d_idx = nullptr;             // [nnz] sources, then [nnz] targets
   void* d_seq = nullptr;            // double2 [nnz][4p + 1]: their Hankel sequences (f64tc_sequences)
   int nnz = 0;
   DevBuf ws;                        // scales and digit images of the coefficients
+};
+
+// FP64 contour contractions on the tensor cores (contour_f64_tc.cu).
+struct ZgemmTc {
+  bool ready = false;
+  int* d_exp = nullptr;             // [2ns] row exponents of E_agg, [2ns] column exponents of E_dis
+  DevBuf ws;                        // scales and digit images of the right operand
 };
 
 struct lsms_ctx {
@@ -114,6 +123,7 @@ struct lsms_ctx {
   bool has_theta = false;
   FmmState fmm;
   F64Tc f64tc;
+  ZgemmTc zgemm;
   // side stream of the mixed operator: the reflected coupling runs beside the translation
   cudaStream_t side = nullptr;
   cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
@@ -253,9 +263,13 @@ void launch_translate_f64(const double* cx, const double* cy, int n, int p, doub
 void launch_etables(const double* cx, const double* cy, int n, const double2* lam,
                     const double2* g2, int ns, double d, double2* eagg, double2* edis,
                     cudaStream_t st);
-// C[r][m][n] += sum_k A[m][k] B[r][k][n];  C must be pre-zeroed (split-K uses atomics)
-void launch_zgemm_rows(const double2* A, int M, int K, const double2* B, double2* C, int P,
-                       int nrhs, cudaStream_t st);
+// C[r][m][n] += sum_k A[m][k] B[r][k][n] on the FP64 pipe (contour_direct.cu; K ranges add atomically)
+void launch_zgemm_direct(const double2* A, int M, int K, const double2* B, double2* C, int P,
+                         int nrhs, cudaStream_t st);
+// the aggregate, the reflection and V = U sigma in one kernel (small tables)
+void launch_node_direct(int ns, int n, int P, int nrhs, const double2* eagg, const double2* xs,
+                        const double2* fagg, const double2* refl, const double2* udis, double2* V,
+                        cudaStream_t st);
 // per node: P,Q from G (if G) else from pq_in; optional outputs pq_out, sig_out, V
 void launch_node_stage(int ns, int P, int nrhs, const double2* G, const double2* fagg,
                        const double2* pq_in, const double2* refl, const double2* udis,

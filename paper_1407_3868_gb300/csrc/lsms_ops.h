@@ -29,6 +29,12 @@ int translate_f64_tc(lsms_ctx* c, int nrhs, const double2* xs, double2* alpha, c
 // path the layout takes
 int translate_f64(lsms_ctx* c, int nrhs, const double2* xs, double2* alpha, cudaStream_t st, int row0 = 0,
                   int nrows = -1);
+// FP64 contour contractions: C[r][M][P] += E_agg . B (agg) or E_dis . B; tables for the tensor cores
+// (contour_f64_tc.cu)
+constexpr double kZgemmMinTable = 1.5e5;   // complex elements of a table; smaller: contour_direct.cu
+int zgemm_setup(lsms_ctx* c);
+void zgemm_free(lsms_ctx* c);
+int zgemm_f64(lsms_ctx* c, bool agg, int nrhs, const double2* B, double2* C, cudaStream_t st);
 // drop the captured batched applications (their kernels depend on the context's settings)
 void batch_clear_graphs(lsms_ctx* c);
 int check_cuda(lsms_ctx* c, const char* where);

@@ -857,6 +857,7 @@ int build_lowp_tables(lsms_ctx* c) {
   std::vector<int> wide_ptr, wide_idx;
   if ((rc = build_near_pairs(c, wide_ptr, wide_idx))) return rc;
   if ((rc = tc_setup(c))) return rc;
+  if ((rc = zgemm_setup(c))) return rc;
   return f64tc_setup(c, wide_ptr, wide_idx);
 }
 

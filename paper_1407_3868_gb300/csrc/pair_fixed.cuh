@@ -16,46 +16,22 @@
 #include <cmath>
 #include <cstdint>
 
+#include "fixed64.cuh"
+
 // Constants of a layer (host: pair_consts).
 struct PairConsts {
   double turn_hi, turn_lo;   // k / (2 pi) as a sum of two doubles
   double inv_k;              // 1 / k
-  double amp;                // sqrt(2 / (pi k))
+  double amp;                // sqrt(2 / (pi k)) / R, see PairState
   float near_r2;             // pairs with r^2 below this are left out (summed from the near-pair list)
 };
 
-// H_0, H_1 (Q65), e^{i phi} (Q62) and 2/z (Q62) of a pair.
+// H_0 / R, H_1 / R (Q65), e^{i phi} (Q62) and 2/z (Q62) of a pair.
 struct PairSeed {
   int64_t j0, y0, j1, y1, c, s, w;
 };
 
 namespace {
-
-#define LSMS_HD __host__ __device__ __forceinline__
-
-LSMS_HD int32_t mulhi_s32(int32_t a, int32_t b) {
-#ifdef __CUDA_ARCH__
-  return __mulhi(a, b);
-#else
-  return (int32_t)(((int64_t)a * b) >> 32);
-#endif
-}
-LSMS_HD int32_t hi_s32(int64_t a) { return (int32_t)(a >> 32); }
-LSMS_HD int32_t half_lo(int64_t a) { return (int32_t)((uint32_t)a >> 1); }   // low word / 2, >= 0
-
-// a b / 2^64, a few units low: the three leading partial products, the cross terms with the low
-// words halved so that all factors are signed 32-bit.
-LSMS_HD int64_t mulq(int64_t a, int64_t b) {
-  const int32_t t = mulhi_s32(hi_s32(a), half_lo(b)) + mulhi_s32(half_lo(a), hi_s32(b));
-  return (int64_t)hi_s32(a) * hi_s32(b) + (int64_t)t * 2;
-}
-// (a b + c d) / 2^64
-LSMS_HD int64_t mulq2(int64_t a, int64_t b, int64_t c, int64_t d) {
-  const int32_t t = mulhi_s32(hi_s32(a), half_lo(b)) + mulhi_s32(half_lo(a), hi_s32(b)) +
-                    mulhi_s32(hi_s32(c), half_lo(d)) + mulhi_s32(half_lo(c), hi_s32(d));
-  return (int64_t)hi_s32(a) * hi_s32(b) + (int64_t)hi_s32(c) * hi_s32(d) + (int64_t)t * 2;
-}
-LSMS_HD int64_t shl(int64_t a, int n) { return (int64_t)((uint64_t)a << n); }
 
 LSMS_HD int64_t to_fixed(double x) {
 #ifdef __CUDA_ARCH__
@@ -70,7 +46,7 @@ LSMS_HD int64_t to_fixed(double x) {
 LSMS_HD int64_t series(int64_t x, int64_t c0, int64_t c1, int32_t c2, int32_t c3, int32_t c4, int32_t c5) {
   const int32_t h = hi_s32(x);
   const int32_t r = c2 + mulhi_s32(h, c3 + mulhi_s32(h, c4 + mulhi_s32(h, c5)));
-  return c0 + (mulq(x, c1 + (((int64_t)h * r) >> 9)) >> 8);  // Q71 -> Q62, Q70 -> Q62
+  return c0 + (mulq(x, c1 + (mul_wide(h, r) >> 9)) >> 8);  // Q71 -> Q62, Q70 -> Q62
 }
 
 #define LSMS_Q(x, n) ((int64_t)((x) * (double)(1LL << ((n) / 2)) * (double)(1LL << ((n) - (n) / 2))))
@@ -133,9 +109,9 @@ LSMS_HD void pair_seed(double dx, double dy, double r2, const PairConsts& q, con
   const int64_t t2 = shl(mulq(th, th), 5);                                       // theta^2, Q75
   const int32_t t2h = hi_s32(t2);                                                // Q43
   const int32_t kc = LSMS_Q32(1.0 / 24.0, 35) - mulhi_s32(t2h, LSMS_Q32(1.0 / 720.0, 24));
-  const int64_t gc = (((int64_t)t2h * kc) >> 16) - (1LL << 61);                  // -1/2 + theta^2/24 - ..., Q62
+  const int64_t gc = (mul_wide(t2h, kc) >> 16) - (1LL << 61);                  // -1/2 + theta^2/24 - ..., Q62
   const int64_t cm = mulq(t2, gc) >> 9;                                          // cos theta - 1, Q64
-  const int64_t gs = (((int64_t)t2h * LSMS_Q32(1.0 / 120.0, 37)) >> 18) - LSMS_Q(1.0 / 6.0, 62);
+  const int64_t gs = (mul_wide(t2h, LSMS_Q32(1.0 / 120.0, 37)) >> 18) - LSMS_Q(1.0 / 6.0, 62);
   const int64_t sv = mulq(t2, gs);                                               // sin theta / theta - 1, Q73
   const int64_t sn = (th >> 3) + (mulq(th, sv) >> 12);                           // Q64
   const auto tab = table[idx];
@@ -152,31 +128,53 @@ LSMS_HD void pair_seed(double dx, double dy, double r2, const PairConsts& q, con
   o.y1 = -(ac + mulq2(ac, p1, as, -q1));
 }
 
-// One step of the order: (J, Y)_{s+1} = (2s/z) (J, Y)_s - (J, Y)_{s-1} and e^{i (s+1) phi}; f = 2s/z.
+// The sequence around an even order s: sigma_s J_s and sigma_{s-1} J_{s-1}, the same of Y (Q63), R e^{i s phi}
+// (Q63; the radius R = 1 - 2^-30 keeps them below 1, the amplitude of the seed carries 1 / R), 2s/z and
+// -2(s+1)/z (Q62).  The signs sigma = + + - - (s mod 4) turn the recurrence's subtraction into an
+// addition, which a multiply-add does by itself: with f = 2s/z, sigma_{s+1} J_{s+1} =
+// +-f sigma_s J_s + sigma_{s-1} J_{s-1}, plus for even s, minus for odd s.
 struct PairState {
-  int64_t j, jm, y, ym, c, s, f;
+  int64_t je, jo, ye, yo, c, s, fe, fo;
 };
-LSMS_HD void pair_step(PairState& a, const PairSeed& o) {
-  const int64_t jn = shl(mulq(a.f, a.j), 2) - a.jm;
-  const int64_t yn = shl(mulq(a.f, a.y), 2) - a.ym;
-  a.jm = a.j; a.j = jn;
-  a.ym = a.y; a.y = yn;
-  a.f += o.w;
-  const int64_t cn = shl(mulq2(a.c, o.c, a.s, -o.s), 2);
-  a.s = shl(mulq2(a.s, o.c, a.c, o.s), 2);
-  a.c = cn;
+// Factors that stay the same along the orders: e^{i phi} (Q62) and minus its sine.
+struct PairStep {
+  Factor c, s, ns;
+  int64_t w2;                // 4/z
+};
+constexpr int64_t kRadius = ((int64_t)1 << 62) - ((int64_t)1 << 32);   // R / 2 in Q63
+
+// Order 0: J_{-1} = -J_1, sigma_{-1} = -1.
+LSMS_HD void pair_start(const PairSeed& o, PairState& a, PairStep& t) {
+  a.je = o.j0 >> 2; a.jo = o.j1 >> 2; a.ye = o.y0 >> 2; a.yo = o.y1 >> 2;
+  a.c = shl(kRadius, 1); a.s = 0; a.fe = 0; a.fo = -o.w;
+  t.c = factor(o.c); t.s = factor(o.s); t.ns = factor(-o.s);
+  t.w2 = shl(o.w, 1);
 }
-// The four products of order s (Q65): J cos, J sin, Y cos, Y sin of s phi.
-LSMS_HD void pair_products(const PairState& a, int64_t* v) {
-  v[0] = shl(mulq(a.j, a.c), 2);
-  v[1] = shl(mulq(a.j, a.s), 2);
-  v[2] = shl(mulq(a.y, a.c), 2);
-  v[3] = shl(mulq(a.y, a.s), 2);
+// v[0..3] = bias + sigma_s (J cos, J sin, Y cos, Y sin of s phi) (Q64) of the order with J_s = j, Y_s = y,
+// then e^{i (s+1) phi}, and jn, yn from order s - 1 to s + 1 with the factor f.
+LSMS_HD void pair_order(int64_t j, int64_t y, int64_t& jn, int64_t& yn, int64_t fs, PairState& a, const PairStep& t,
+                        int64_t bias, int64_t* v) {
+  const Factor jf = factor(shl(j, 2)), yf = factor(shl(y, 2));         // Q65
+  const Factor c = factor(a.c), s = factor(a.s), f = factor(fs);
+  v[0] = madq(jf, c, bias);
+  v[1] = madq(jf, s, bias);
+  v[2] = madq(yf, c, bias);
+  v[3] = madq(yf, s, bias);
+  jn = madq(jf, f, jn);                                          // Q63
+  yn = madq(yf, f, yn);
+  a.c = shl(mulq2(c, t.c, s, t.ns), 2);
+  a.s = shl(mulq2(s, t.c, c, t.s), 2);
+}
+// The products of the even order s (v[0..3]) and of s + 1 (v[4..7]), then on to s + 2.
+LSMS_HD void pair_two_orders(PairState& a, const PairStep& t, int64_t bias, int64_t* v) {
+  pair_order(a.je, a.ye, a.jo, a.yo, a.fe, a, t, bias, v);
+  pair_order(a.jo, a.yo, a.je, a.ye, a.fo, a, t, bias, v + 4);
+  a.fe += t.w2;
+  a.fo -= t.w2;
 }
 
 #undef LSMS_Q
 #undef LSMS_Q32
-#undef LSMS_HD
 
 }  // namespace
 
@@ -188,7 +186,7 @@ inline PairConsts pair_consts(double k, double z_near) {
   q.turn_hi = (double)t;
   q.turn_lo = (double)(t - (long double)q.turn_hi);
   q.inv_k = (double)(1.0L / (long double)k);
-  q.amp = (double)sqrtl(2.0L / (pi * (long double)k));
+  q.amp = (double)(sqrtl(2.0L / (pi * (long double)k)) / (1.0L - 0x1p-30L));   // 1 / R of PairState
   q.near_r2 = (float)((z_near / k) * (z_near / k));
   return q;
 }

@@ -7,7 +7,7 @@
 // so the outputs of 128 targets are one real product summed over the sources,
 //   alpha[target][(nu, Re/Im)] = sum_source sum_{s, A..D} W[target][(s, A..D)] X_source[(s, A..D)][(nu, Re/Im)],
 // with X_source the signed sums beta_{nu+s} +- beta_{nu-s}.  W and X are held as 48-bit fixed point
-// numbers (W: |h| < 1/4, so 49 fractional bits; X: relative to the largest coefficient of the
+// numbers (W: 48 fractional bits; X: relative to the largest coefficient of the
 // right-hand side) and cut into six signed 8-bit digits each; the digits are exact in FP16, a product
 // of two has at most 14 bits, so the tensor cores' FP32 sums are exact integers.  Products of digits
 // i of W and j of X with i + j = L add into one accumulator per level L; levels beyond LMAX (5 or 6)
@@ -16,20 +16,18 @@
 //
 // Why: this chip's FP64 pipe (2 FMA per SM and clock) bounds the direct form at 133 ms for 5000 discs
 // (k_translate_f64_sym: 168 ms); 21 products of FP16 digits take 4.7 ms at the tensor cores' measured
-// rate, and this kernel 9.4 ms (1000 discs at p = 12: 5.2 -> 0.37 ms).
+// rate, and this kernel 8.2 ms (1000 discs at p = 12: 5.2 -> 0.33 ms).
 //
-// Exactness: a level <= 3 collects at most 4 products of 4(2p+1) <= 124 digit pairs, below 4 x 124 x 2^14
-// = 2^22.96 per source: two sources (a drain group) stay below 2^24.  Levels 4, 5, 6 could leave the
-// exact range by one bit only if every digit had its largest value; their unit is then 2^-16 of what
-// is left out anyway.  Drained levels are summed in 64-bit integers, so a CTA's sum does not depend
-// on any order.
-//
-// A CTA owns 128 targets and a range of sources, two sources at a time: warps 0-3 and 4-7 each form
-// the W rows of one of the two (thread = target; the fixed-point sequence of pair_fixed.cuh) and
-// store its digits into the stage ring in the tensor cores' K-major layout of 8 x 16-byte core
-// matrices (thread = row: consecutive threads write consecutive 16-byte pieces); warp 17 copies the X
+// A CTA owns 128 targets and a range of sources.  Two warpgroups form the W rows of every second
+// source each (thread = target; the fixed-point sequence of pair_fixed.cuh), eight orders at a time
+// into the stage ring (consecutive threads write consecutive 16-byte pieces); warp 17 copies the X
 // digits of the same orders (packed once per application); warp 16 issues the MMAs; warps 8-15 drain
-// the accumulators after every two sources.
+// the accumulators into 64-bit integers, so a CTA's sum does not depend on any order.  When: before a
+// round (two sources) whose X digits could carry a sum of the levels 0..4 past 2^24, from the bound
+// that the packing kernel left for each source; the decaying coefficients of scattering problems let
+// several rounds pass.  (One round alone stays below it in the levels 0..3 for any digits.)
+// The ring holds three stages of two MMA steps: six stages of one step took 10.0 instead of 9.1 ms
+// (5000 discs, the translation's part of the operator), a third warpgroup brought nothing.
 #include <algorithm>
 #include <cmath>
 #include <mutex>
@@ -38,14 +36,22 @@
 #include "digits_tc.cuh"
 #include "lsms_internal.h"
 #include "lsms_ops.h"
+#include "near_f64.cuh"
 #include "pair_fixed.cuh"
 
 namespace {
 
 constexpr int TABLE_BYTES = 256 * 16;
+constexpr int kExact = 1 << 24;                // FP32 sums of integers are exact up to here
 constexpr int MAX_SOURCES = 1024;             // per CTA: the 64-bit sums keep 10 bits for them
+constexpr int GROUPS = 2;                     // warpgroups forming W
+constexpr int GEN_WARPS = 4 * GROUPS;
+constexpr int MMA_WARP = GEN_WARPS + DRAIN_WARPS;
+constexpr int THREADS = (MMA_WARP + 2) * 32;
+constexpr size_t smem_bytes(int npad) {
+  return (size_t)STAGES * stage_bytes(npad) + TABLE_BYTES + MAX_SOURCES / GROUPS * sizeof(int) + 256;
+}
 
-constexpr size_t smem_bytes(int npad) { return (size_t)STAGES * stage_bytes(npad) + TABLE_BYTES + 256; }
 inline int k_steps(int p) { return (4 * (2 * p + 1) + 15) / 16; }   // K = 16 steps of one source
 
 // Largest |Re|, |Im| of each right-hand side as the bits of a non-negative double (NaN and Inf
@@ -60,16 +66,20 @@ __global__ void k_absmax(const double* __restrict__ x, long long per, unsigned l
   if ((threadIdx.x & 31) == 0 && m) atomicMax(out + blockIdx.y, m);
 }
 // Digits of X for the sources src0 .. src0 + gridDim.x - 1 of right-hand side r0 + blockIdx.y:
-// per source [K group][plane][column][8 K values] FP16, K = 4 s + (A, B, C, D), column 2 q + (Re, Im).
+// per source [K group][plane][column][8 K values] FP16, K = 4 s + (A, B, C, D), column 2 q + (Re, Im); and
+// bound[source]: what the source adds to any element of the levels 0..4 at most, 128 sum |X digits|.
 __global__ void __launch_bounds__(256)
 k_pack_digits(const double2* __restrict__ xs, int n, int p, int src0, int r0, int npad, int kgs,
-              const unsigned long long* __restrict__ maxbits, unsigned char* __restrict__ img) {
+              const unsigned long long* __restrict__ maxbits, unsigned char* __restrict__ img,
+              int* __restrict__ bound) {
   __shared__ long long re[128], im[128];          // beta_{nu +- s} at 48 + order, zero outside -p..p
+  __shared__ int l1[64];                          // sum of |digit| of planes 0..4 per column
   const int P = 2 * p + 1, r = r0 + blockIdx.y;
   const unsigned long long mb = maxbits[r];
   if (mb == 0 || mb >= kInfBits) return;          // the product does not read the image then
   const int sh = 46 - scale_exponent(mb);
   const double2* b = xs + ((size_t)r * n + src0 + blockIdx.x) * P;
+  if (threadIdx.x < 64) l1[threadIdx.x] = 0;
   if (threadIdx.x < 128) {
     const int o = (int)threadIdx.x - 48 + p;
     double2 v = make_double2(0.0, 0.0);
@@ -102,6 +112,7 @@ k_pack_digits(const double2* __restrict__ xs, int n, int p, int src0, int r0, in
           a = pi + mi; bb = pr - mr; cc = pr + mr; d = -pi + mi;
         }
         if (s == 0) bb = d = 0;
+        if (s & 2) { a = -a; bb = -bb; cc = -cc; d = -d; }   // the sequence's signs + + - -
       }
       uint32_t u[PL], v[PL];
       digit_pairs(a << 16, bb << 16, u);
@@ -112,9 +123,25 @@ k_pack_digits(const double2* __restrict__ xs, int n, int p, int src0, int r0, in
         w[j][2 * h + 1] = v[j];
       }
     }
+    int sum = 0;
 #pragma unroll
-    for (int j = 0; j < PL; ++j)
+    for (int j = 0; j < PL; ++j) {
       dst[((size_t)kg * PL + j) * npad + col] = make_uint4(w[j][0], w[j][1], w[j][2], w[j][3]);
+      if (j <= 4) {
+        __half2 h = __float2half2_rn(0.0f);       // four digits of at most 128 in a half: exact
+#pragma unroll
+        for (int i = 0; i < 4; ++i) h = __hadd2(h, __habs2(*reinterpret_cast<const __half2*>(&w[j][i])));
+        sum += (int)__low2float(h) + (int)__high2float(h);
+      }
+    }
+    atomicAdd(&l1[col], sum);
+  }
+  __syncthreads();
+  if (threadIdx.x < 32) {
+    int m = max(l1[threadIdx.x], l1[threadIdx.x + 32]);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
+    if (threadIdx.x == 0) bound[(size_t)blockIdx.y * gridDim.x + blockIdx.x] = 128 * m;
   }
 }
 
@@ -123,13 +150,15 @@ k_pack_digits(const double2* __restrict__ xs, int n, int p, int src0, int r0, in
 template <int NPAD, int LMAX>
 __global__ void __launch_bounds__(THREADS, 1)
 k_translate_digits(const double* __restrict__ cx, const double* __restrict__ cy, int n, int p, PairConsts pc,
-                   const longlong2* __restrict__ table, const unsigned char* __restrict__ img, int src0, int nsrc,
+                   const longlong2* __restrict__ table, const unsigned char* __restrict__ img,
+                   const int* __restrict__ bound, int src0, int nsrc,
                    int per_cta, int r0, const unsigned long long* __restrict__ maxbits, int row0, int nrows,
                    double2* __restrict__ alpha, int* __restrict__ err) {
   extern __shared__ __align__(128) unsigned char smem[];
   constexpr int STAGE = stage_bytes(NPAD);
   longlong2* stab = (longlong2*)(smem + STAGES * STAGE);
-  uint64_t* bars = (uint64_t*)(smem + STAGES * STAGE + TABLE_BYTES);   // full[3], empty[3], acc_full, acc_empty
+  int* round_bound = (int*)(smem + STAGES * STAGE + TABLE_BYTES);      // [rounds]
+  uint64_t* bars = (uint64_t*)(round_bound + MAX_SOURCES / GROUPS);   // full[S], empty[S], acc_full, acc_empty
   uint32_t* tmem_slot = (uint32_t*)(bars + 2 * STAGES + 2);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int P = 2 * p + 1, r = r0 + blockIdx.z;
@@ -148,12 +177,12 @@ k_translate_digits(const double* __restrict__ cx, const double* __restrict__ cy,
     return;
   }
   const int steps = (4 * P + 15) / 16;             // K = 16 steps of a source
-  const int chunks = (steps + 1) / 2;
-  const int pairs = (s_end - s_begin + 1) / 2;     // drain groups
+  const int rounds = (s_end - s_begin + GROUPS - 1) / GROUPS;
+  const int chunks = (steps + 1) / 2;              // stages of a source
   const uint32_t full0 = smem_u32(bars), empty0 = full0 + 8 * STAGES, accf = full0 + 16 * STAGES, acce = accf + 8;
   if (threadIdx.x == 0) {
     for (int s = 0; s < STAGES; ++s) {
-      mbar_init(full0 + 8 * s, 5);                 // four generating warps and the copy
+      mbar_init(full0 + 8 * s, 5);                 // four forming warps and the copy
       mbar_init(empty0 + 8 * s, 1);
     }
     mbar_init(accf, 1);
@@ -161,8 +190,13 @@ k_translate_digits(const double* __restrict__ cx, const double* __restrict__ cy,
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (threadIdx.x < 256) stab[threadIdx.x] = table[threadIdx.x];
+  for (int q = threadIdx.x; q < rounds; q += THREADS) {
+    int w = 0;
+    for (int m = s_begin + GROUPS * q; m < min(s_end, s_begin + GROUPS * (q + 1)); ++m) w += bound[(size_t)blockIdx.z * nsrc + m];
+    round_bound[q] = w;
+  }
   __syncwarp();
-  if (warp == GEN_WARPS + DRAIN_WARPS) tmem_alloc(smem_u32(tmem_slot), 512);
+  if (warp == MMA_WARP) tmem_alloc(smem_u32(tmem_slot), 512);
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
@@ -170,14 +204,14 @@ k_translate_digits(const double* __restrict__ cx, const double* __restrict__ cy,
   const uint32_t sbase = smem_u32(smem);
 
   if (warp < GEN_WARPS) {
-    // ---- digits of W: group g takes every second source, thread = target row
+    // ---- digits of W: warpgroup g takes every third source, thread = target row
     const int g = warp >> 2, row = threadIdx.x & (ROWS - 1);
     const int l = row0 + blockIdx.x * ROWS + row;
     const bool lvalid = l < row0 + nrows;
     const double xl = lvalid ? cx[l] : 0.0, yl = lvalid ? cy[l] : 0.0;
     bool ok = true;
-    for (int q = 0; q < pairs && ok; ++q) {
-      const int m = s_begin + 2 * q + g;
+    for (int q = 0; q < rounds && ok; ++q) {
+      const int m = s_begin + GROUPS * q + g;
       PairSeed o;
       o.j0 = o.y0 = o.j1 = o.y1 = o.c = o.s = o.w = 0;
       if (lvalid && m < s_end && src0 + m != l) {
@@ -185,32 +219,27 @@ k_translate_digits(const double* __restrict__ cx, const double* __restrict__ cy,
         const double r2 = fma(dx, dx, dy * dy);
         if (!pair_is_near(r2, pc)) pair_seed(dx, dy, r2, pc, stab, o);
       }
-      // order 0; the step from it gives order 1 (J_{-1} = -J_1)
       PairState a;
-      a.j = o.j0; a.jm = -o.j1; a.y = o.y0; a.ym = -o.y1;
-      a.c = 1LL << 62; a.s = 0; a.f = 0;
+      PairStep step;
+      pair_start(o, a, step);
       for (int c = 0; c < chunks; ++c) {
-        const int t = (q * chunks + c) * 2 + g;
-        const int st = t % STAGES, round = t / STAGES;
-        if (round > 0 && !mbar_wait(empty0 + 8 * st, (round - 1) & 1)) {
+        const int t = (q * chunks + c) * GROUPS + g;
+        const int st = t % STAGES, lap = t / STAGES;
+        if (lap > 0 && !mbar_wait(empty0 + 8 * st, (lap - 1) & 1)) {
           ok = false;
           break;
         }
         unsigned char* base = smem + st * STAGE + row * 16;
-        const int kgs = min(KG, 2 * steps - KG * c);
 #pragma unroll 1
-        for (int kg = 0; kg < kgs; ++kg) {
+        for (int kg = 0; kg < KG && KG * c + kg < 2 * steps; ++kg) {
           uint32_t u[PL], v[PL], w[PL], z[PL];
-          int64_t pr[4];
-          if (2 * (KG * c + kg) <= 2 * p) {
-            pair_products(a, pr);
-            digit_pairs(pr[0], pr[1], u);
-            digit_pairs(pr[2], pr[3], v);
-            pair_step(a, o);
-            pair_products(a, pr);
-            digit_pairs(pr[0], pr[1], w);
-            digit_pairs(pr[2], pr[3], z);
-            pair_step(a, o);
+          if (KG * c + kg <= p) {                  // orders 2 (KG c + kg) and the next
+            int64_t pr[8];
+            pair_two_orders(a, step, (int64_t)kDigitBias, pr);
+            biased_digit_pairs(pr[0], pr[1], u);
+            biased_digit_pairs(pr[2], pr[3], v);
+            biased_digit_pairs(pr[4], pr[5], w);
+            biased_digit_pairs(pr[6], pr[7], z);
           } else {
 #pragma unroll
             for (int j = 0; j < PL; ++j) u[j] = v[j] = w[j] = z[j] = 0;
@@ -225,7 +254,7 @@ k_translate_digits(const double* __restrict__ cx, const double* __restrict__ cy,
       }
     }
     if (!ok && lane == 0) atomicExch(err, 11);
-  } else if (warp < GEN_WARPS + DRAIN_WARPS) {
+  } else if (warp < MMA_WARP) {
     // ---- drain: warp d owns lanes 32 (d mod 4) .. + 31 and half of the columns
     const int d = warp - GEN_WARPS, quad = warp & 3, half = d >> 2;
     constexpr int HC = NPAD / 2;
@@ -234,8 +263,11 @@ k_translate_digits(const double* __restrict__ cx, const double* __restrict__ cy,
     for (int i = 0; i < HC; ++i) acc[i] = 0;
     const uint32_t tb = tmem + ((uint32_t)(32 * quad) << 16) + half * HC;
     bool ok = true;
-    for (int q = 0; q < pairs; ++q) {
-      ok = __all_sync(0xffffffffu, mbar_wait(accf, q & 1));
+    for (int q = 0, group = 0; q < rounds; ++group) {
+      int sum = 0;
+      do sum += round_bound[q++];
+      while (q < rounds && sum + round_bound[q] <= kExact);      // the issuing warp's groups
+      ok = __all_sync(0xffffffffu, mbar_wait(accf, group & 1));
       if (!ok) break;
       tc_fence_after();
       drain_levels<NPAD, LMAX>(tb, acc);
@@ -245,68 +277,72 @@ k_translate_digits(const double* __restrict__ cx, const double* __restrict__ cy,
     }
     if (ok) {
       const int row = blockIdx.x * ROWS + 32 * quad + lane;
-      const int ex = scale_exponent(mb) - 49;      // unit of acc
-      const double s1 = scalbn(1.0, ex / 2), s2 = scalbn(1.0, ex - ex / 2);
+      const int ex = scale_exponent(mb) - 48;      // unit of acc
       if (row < nrows) {
 #pragma unroll
         for (int i = 0; i < HC; ++i) {
           const int col = half * HC + i;
           if (col < 2 * P)
-            atomicAdd((double*)(ar + (size_t)row * P) + col, __ll2double_rn(acc[i]) * s1 * s2);
+            atomicAdd((double*)(ar + (size_t)row * P) + col, fixed_to_double(acc[i], ex));
         }
       }
     } else if (lane == 0) {
       atomicExch(err, 12);
     }
-  } else if (warp == GEN_WARPS + DRAIN_WARPS) {
-    // ---- MMA issue
-    if (lane == 0) {
+  } else {
+    if (warp == MMA_WARP && lane == 0) {
+      // ---- MMA issue
       bool ok = true;
-      for (int q = 0; q < pairs && ok; ++q) {
-        if (q > 0 && !mbar_wait(acce, (q - 1) & 1)) {
-          ok = false;
-          break;
+      int t = 0, group = 0, sum = 0;
+      for (int q = 0; q < rounds && ok; ++q) {
+        const int w = round_bound[q];
+        const bool start = q == 0 || sum + w > kExact;           // a round stays below it by itself
+        sum = start ? w : sum + w;
+        if (start && q > 0) {
+          mma_commit(accf);
+          if (!mbar_wait(acce, group & 1)) {
+            ok = false;
+            break;
+          }
+          ++group;
+          tc_fence_after();
         }
-        tc_fence_after();
-        for (int c2 = 0; c2 < 2 * chunks; ++c2) {
-          const int t = q * 2 * chunks + c2;
-          const int st = t % STAGES, round = t / STAGES;
-          if (!mbar_wait(full0 + 8 * st, round & 1)) {
+        for (int c = 0; c < GROUPS * chunks; ++c, ++t) {
+          const int st = t % STAGES, lap = t / STAGES;
+          if (!mbar_wait(full0 + 8 * st, lap & 1)) {
             ok = false;
             break;
           }
           tc_fence_after();
-          const uint32_t sa = sbase + st * STAGE, sb = sa + A_BYTES;
-          const int ksteps = min(2, steps - 2 * (c2 >> 1));
-          for (int ks = 0; ks < ksteps; ++ks) issue_step<NPAD, LMAX>(tmem, sa, sb, ks, c2 == 0 && ks == 0);
+          const uint32_t sa = sbase + st * STAGE;
+          const int ksteps = min(2, steps - 2 * (c / GROUPS));
+          for (int ks = 0; ks < ksteps; ++ks)
+            issue_step<NPAD, LMAX>(tmem, sa, sa + A_BYTES, ks, start && c == 0 && ks == 0);
           mma_commit(empty0 + 8 * st);
         }
-        if (ok) mma_commit(accf);
       }
+      if (ok) mma_commit(accf);
       if (!ok) atomicExch(err, 13);
-    }
-    __syncwarp();
-  } else {
-    // ---- copies of the X digits
-    if (lane == 0) {
+    } else if (warp == MMA_WARP + 1 && lane == 0) {
+      // ---- copies of the X digits
       bool ok = true;
-      const size_t src_bytes = (size_t)2 * steps * b_kg_bytes(NPAD);
+      constexpr uint32_t STEP = 2 * b_kg_bytes(NPAD);
+      const size_t src_bytes = (size_t)steps * STEP;
       const unsigned char* ir = img + (size_t)blockIdx.z * nsrc * src_bytes;
       int t = 0;
-      for (int q = 0; q < pairs && ok; ++q)
-        for (int c2 = 0; c2 < 2 * chunks; ++c2, ++t) {
-          const int st = t % STAGES, round = t / STAGES;
-          if (round > 0 && !mbar_wait(empty0 + 8 * st, (round - 1) & 1)) {
-            ok = false;
-            break;
+      for (int q = 0; q < rounds && ok; ++q)
+        for (int c = 0; c < chunks && ok; ++c)
+          for (int g = 0; g < GROUPS; ++g, ++t) {
+            const int st = t % STAGES, lap = t / STAGES;
+            if (lap > 0 && !mbar_wait(empty0 + 8 * st, (lap - 1) & 1)) {
+              ok = false;
+              break;
+            }
+            const int m = min(s_begin + GROUPS * q + g, s_end - 1);
+            const uint32_t bytes = min(2, steps - 2 * c) * STEP;
+            mbar_expect_tx(full0 + 8 * st, bytes);
+            bulk_load(sbase + st * STAGE + A_BYTES, ir + m * src_bytes + (size_t)c * 2 * STEP, bytes, full0 + 8 * st);
           }
-          const int c = c2 >> 1, m = min(s_begin + 2 * q + (c2 & 1), s_end - 1);
-          const int kgs = min(KG, 2 * steps - KG * c);
-          const uint32_t bytes = (uint32_t)kgs * b_kg_bytes(NPAD);
-          mbar_expect_tx(full0 + 8 * st, bytes);
-          bulk_load(sbase + st * STAGE + A_BYTES, ir + m * src_bytes + (size_t)c * KG * b_kg_bytes(NPAD), bytes,
-                    full0 + 8 * st);
-        }
       // copies still in flight end before the CTA does
       for (int s = max(0, t - STAGES); s < t && !ok; ++s) mbar_wait(full0 + 8 * (s % STAGES), (s / STAGES) & 1);
       if (!ok) atomicExch(err, 14);
@@ -316,7 +352,7 @@ k_translate_digits(const double* __restrict__ cx, const double* __restrict__ cy,
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  if (warp == GEN_WARPS + DRAIN_WARPS) tmem_dealloc(tmem, 512);
+  if (warp == MMA_WARP) tmem_dealloc(tmem, 512);
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -352,57 +388,23 @@ __global__ void k_near_sequences(const double* __restrict__ cx, const double* __
   }
 }
 
-// alpha^l += sum over l's listed sources: one warp per (target, right-hand side), lane = output order.
-// The sequences are read where they lie (a window of P consecutive values per source order, in L1
-// after the first; the lists of 5000 discs at p = 14 take 63 MB, in L2 between applications), so the
-// kernel needs no shared memory and enough warps share an SM to keep its FP64 pipe busy: four
-// independent FMAs per order and warp.  5000 discs: 2.80 ms with the sequences formed anew in
-// shared memory (one CTA per SM) -> 0.51 ms
-// (its 8 M warp FMAs take 0.44 ms of the pipe).
-__global__ void __launch_bounds__(128)
-k_translate_near_f64(int n, int p, int row0, int nrows, const int* __restrict__ ptr, const int* __restrict__ idx,
-                     const double2* __restrict__ seq, const double2* __restrict__ xs, double2* __restrict__ alpha) {
-  const int P = 2 * p + 1, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int l = row0 + blockIdx.x * 4 + warp, r = blockIdx.y;
-  if (l >= row0 + nrows) return;
-  const int e1 = ptr[l + 1];
-  const double2* xr = xs + (size_t)r * n * P;
-  const int nu = min(lane, P - 1);                       // idle lanes repeat the last order
-  double rr = 0.0, ii = 0.0, ri = 0.0, ir = 0.0;
-  for (int e = ptr[l]; e < e1; ++e) {
-    const double2* h = seq + (size_t)e * (4 * p + 1) + 2 * p - nu;
-    const double2* b = xr + (size_t)idx[e] * P;
-#pragma unroll 4
-    for (int q = 0; q < P; ++q) {
-      const double2 hv = __ldg(h + q), bv = __ldg(b + q);
-      rr = fma(hv.x, bv.x, rr);
-      ii = fma(hv.y, bv.y, ii);
-      ri = fma(hv.x, bv.y, ri);
-      ir = fma(hv.y, bv.x, ir);
-    }
-  }
-  if (lane < P) {
-    double2* o = alpha + ((size_t)r * nrows + (l - row0)) * P + lane;
-    *o = make_double2(o->x + (rr - ii), o->y + (ri + ir));
-  }
-}
-
 template <int NPAD, int LMAX>
 void launch_digits(dim3 grid, cudaStream_t st, const lsms_ctx* c, const PairConsts& pc, const unsigned char* img,
-                   int src0, int nsrc, int per_cta, int r0, const unsigned long long* maxbits, int row0, int nrows,
-                   double2* alpha, int* err) {
+                   const int* bound, int src0, int nsrc, int per_cta, int r0, const unsigned long long* maxbits,
+                   int row0, int nrows, double2* alpha, int* err) {
   static std::once_flag attr;
   std::call_once(attr, [] {
     cudaFuncSetAttribute(k_translate_digits<NPAD, LMAX>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                          (int)smem_bytes(NPAD));
   });
   k_translate_digits<NPAD, LMAX><<<grid, THREADS, smem_bytes(NPAD), st>>>(
-      c->d_cx, c->d_cy, c->n, c->p, pc, (const longlong2*)c->f64tc.d_table, img, src0, nsrc, per_cta, r0, maxbits,
-      row0, nrows, alpha, err);
+      c->d_cx, c->d_cy, c->n, c->p, pc, (const longlong2*)c->f64tc.d_table, img, bound, src0, nsrc, per_cta, r0,
+      maxbits, row0, nrows, alpha, err);
 }
 
 constexpr size_t kImageBytes = (size_t)256 << 20;   // digits of X held at once
 constexpr int kMinDiscs = 96;
+constexpr double kStoreBytes = 64e6;
 
 }  // namespace
 
@@ -416,22 +418,36 @@ void f64tc_free(lsms_ctx* c) {
 
 // Tables of the layout: `ptr`, `idx` list per target the sources within (1 + 1e-6) of the near
 // distance (host arrays).  Layouts of fewer than kMinDiscs discs (not one full tile of rows) or of
-// mostly near pairs (summed on the FP64 pipe either way) keep k_translate_f64 and its symmetric form.
+// mostly near pairs (summed on the FP64 pipe either way) store the sequences of all their pairs if
+// these take at most kStoreBytes (16 discs: 75 us with the sequences formed anew -> 11 us);
+// larger ones keep k_translate_f64 and its symmetric form.
 int f64tc_setup(lsms_ctx* c, const std::vector<int>& ptr, const std::vector<int>& idx) {
   f64tc_free(c);
   F64Tc& f = c->f64tc;
   const int n = c->n;
-  if (n < kMinDiscs || (double)idx.size() > 0.5 * n * (double)(n - 1) || !tc_err_flag(c)) return LSMS_OK;
+  if (n <= 0 || !tc_err_flag(c)) return LSMS_OK;
+  const bool digits = n >= kMinDiscs && (double)idx.size() <= 0.5 * n * (double)(n - 1);
+  const bool store = !digits && (double)n * (n - 1) * (4 * c->p + 1) * sizeof(double2) <= kStoreBytes;
+  if (!digits && !store) return LSMS_OK;
+  std::vector<int> all_ptr, all_idx;
+  if (store) {
+    all_ptr.resize(n + 1);
+    for (int l = 0; l <= n; ++l) all_ptr[l] = l * (n - 1);
+    for (int l = 0; l < n; ++l)
+      for (int m = 0; m < n; ++m)
+        if (m != l) all_idx.push_back(m);
+  }
+  const std::vector<int>&lp = store ? all_ptr : ptr, &li = store ? all_idx : idx;
   const long double pi = 3.14159265358979323846264338327950288L;
   std::vector<longlong2> tab(256);
   for (int i = 0; i < 256; ++i) {
     const long double a = 2 * pi * i / 256 - pi / 4, one = 4611686018427387904.0L;
     tab[i] = make_longlong2((long long)rintl(cosl(a) * one), (long long)rintl(sinl(a) * one));
   }
-  const size_t nnz = idx.size(), ne = nnz > 0 ? nnz : 1;
+  const size_t nnz = li.size(), ne = nnz > 0 ? nnz : 1;
   std::vector<int> tgt(nnz);
   for (int l = 0; l < n; ++l)
-    for (int e = ptr[l]; e < ptr[l + 1]; ++e) tgt[e] = l;
+    for (int e = lp[l]; e < lp[l + 1]; ++e) tgt[e] = l;
   if (cudaMalloc(&f.d_table, TABLE_BYTES) != cudaSuccess ||
       cudaMalloc((void**)&f.d_ptr, (n + 1) * sizeof(int)) != cudaSuccess ||
       cudaMalloc((void**)&f.d_idx, 2 * ne * sizeof(int)) != cudaSuccess) {
@@ -440,13 +456,14 @@ int f64tc_setup(lsms_ctx* c, const std::vector<int>& ptr, const std::vector<int>
     return ctx_fail(c, LSMS_ERR_OOM, "cudaMalloc failed for the near pairs of the FP64 translation");
   }
   cudaMemcpy(f.d_table, tab.data(), TABLE_BYTES, cudaMemcpyHostToDevice);
-  cudaMemcpy(f.d_ptr, ptr.data(), (n + 1) * sizeof(int), cudaMemcpyHostToDevice);
+  cudaMemcpy(f.d_ptr, lp.data(), (n + 1) * sizeof(int), cudaMemcpyHostToDevice);
   if (nnz) {
-    cudaMemcpy(f.d_idx, idx.data(), nnz * sizeof(int), cudaMemcpyHostToDevice);
+    cudaMemcpy(f.d_idx, li.data(), nnz * sizeof(int), cudaMemcpyHostToDevice);
     cudaMemcpy(f.d_idx + nnz, tgt.data(), nnz * sizeof(int), cudaMemcpyHostToDevice);
   }
   f.nnz = (int)nnz;
   f.ready = true;
+  f.digits = digits;
   return check_cuda(c, "f64tc_setup");
 }
 
@@ -467,7 +484,8 @@ int f64tc_sequences(lsms_ctx* c) {
     return ctx_fail(c, LSMS_ERR_OOM, "cudaMalloc failed for the near sequences of the FP64 translation");
   }
   k_near_sequences<<<(f.nnz + 127) / 128, 128, 0, c->stream>>>(c->d_cx, c->d_cy, f.d_idx + f.nnz, f.d_idx, f.nnz,
-                                                                c->p, c->k2, pair_consts(c->k2, pair_z_near(c->p)),
+                                                                c->p, c->k2,
+                                                                pair_consts(c->k2, f.digits ? pair_z_near(c->p) : HUGE_VAL),
                                                                 (double2*)f.d_seq);
   cudaStreamSynchronize(c->stream);
   return check_cuda(c, "f64tc_sequences");
@@ -477,22 +495,32 @@ int f64tc_sequences(lsms_ctx* c) {
 int translate_f64_tc(lsms_ctx* c, int nrhs, const double2* xs, double2* alpha, cudaStream_t st, int row0, int nrows) {
   F64Tc& f = c->f64tc;
   const int n = c->n, p = c->p, P = c->P, npad = pad_columns(p), steps = k_steps(p);
+  cudaMemsetAsync(alpha, 0, (size_t)nrhs * nrows * P * sizeof(double2), st);
+  if (!f.digits) {
+    // about 8 warps per SM
+    if (f.nnz > 0) {
+      const int splits = (int)std::max<long long>(1, std::min<long long>(n - 1, 152LL * 8 / std::max(1LL, (long long)nrows * nrhs)));
+      launch_near_f64(n, p, nullptr, row0, nrows, splits, f.d_ptr, f.d_idx, (const double2*)f.d_seq, xs, nrhs, alpha, st);
+    }
+    return check_cuda(c, "translate_f64_tc");
+  }
   const size_t src_bytes = (size_t)2 * steps * b_kg_bytes(npad);
   // the image holds whole right-hand sides if several fit, else a run of sources of one
-  const int cap = (int)std::max<size_t>(2, kImageBytes / src_bytes);
+  const int cap = (int)std::max<size_t>(1, kImageBytes / src_bytes);
   const int rb = std::max(1, std::min(nrhs, cap / n));
   int runs = (n + cap - 1) / cap;
-  const int run = (((n + runs - 1) / runs) + 1) / 2 * 2;
+  const int run = (n + runs - 1) / runs;
   runs = (n + run - 1) / run;
   const size_t img_bytes = (size_t)rb * std::min(run, n) * src_bytes;
   const size_t max_bytes = ((size_t)nrhs * 8 + 255) & ~size_t(255);
   int rc;
-  if ((rc = ensure(c, f.ws, max_bytes + img_bytes))) return rc;
+  const size_t bound_bytes = ((size_t)rb * std::min(run, n) * sizeof(int) + 255) & ~size_t(255);
+  if ((rc = ensure(c, f.ws, max_bytes + bound_bytes + img_bytes))) return rc;
   unsigned long long* maxbits = (unsigned long long*)f.ws.ptr;
-  unsigned char* img = (unsigned char*)f.ws.ptr + max_bytes;
+  int* bound = (int*)((unsigned char*)f.ws.ptr + max_bytes);
+  unsigned char* img = (unsigned char*)f.ws.ptr + max_bytes + bound_bytes;
   int* err = tc_err_flag(c);
   cudaMemsetAsync(maxbits, 0, (size_t)nrhs * 8, st);
-  cudaMemsetAsync(alpha, 0, (size_t)nrhs * nrows * P * sizeof(double2), st);
   const long long per = 2LL * n * P;
   k_absmax<<<dim3((int)std::min<long long>((per + 1023) / 1024, 152), nrhs), 256, 0, st>>>((const double*)xs, per,
                                                                                           maxbits);
@@ -502,28 +530,28 @@ int translate_f64_tc(lsms_ctx* c, int nrhs, const double2* xs, double2* alpha, c
     const int nr = std::min(rb, nrhs - r0);
     for (int s0 = 0; s0 < n; s0 += run) {
       const int ns = std::min(run, n - s0);
-      k_pack_digits<<<dim3(ns, nr), 256, 0, st>>>(xs, n, p, s0, r0, npad, 2 * steps, maxbits, img);
-      // source ranges: the fewest rounds of 152 CTAs times the pairs of a CTA, plus about two pairs
-      // of time per CTA for its start and end
+      k_pack_digits<<<dim3(ns, nr), 256, 0, st>>>(xs, n, p, s0, r0, npad, 2 * steps, maxbits, img, bound);
+      // source ranges: the fewest waves of 152 CTAs times the rounds of two sources of a CTA, plus
+      // about two rounds of time per CTA for its start and end
       int best = 1;
       double cost = 1e300;
-      const int max_split = std::min((ns + 1) / 2, std::max(1, 65535));
-      for (int sp = (ns + MAX_SOURCES - 1) / MAX_SOURCES; sp <= max_split && sp <= 152 * 8; ++sp) {
-        const double rounds = std::ceil((double)tiles * sp * nr / 152.0);
-        const double cc = rounds * (2.0 + std::ceil(std::ceil((double)ns / sp) / 2.0));
+      const int max_split = std::min((ns + GROUPS - 1) / GROUPS, 152 * 8);
+      for (int sp = (ns + MAX_SOURCES - 1) / MAX_SOURCES; sp <= max_split; ++sp) {
+        const double waves = std::ceil((double)tiles * sp * nr / 152.0);
+        const double cc = waves * (2.0 + std::ceil(std::ceil((double)ns / sp) / GROUPS));
         if (cc < cost * 0.999) {
           cost = cc;
           best = sp;
         }
       }
-      const int per_cta = (((ns + best - 1) / best) + 1) / 2 * 2;
+      const int per_cta = (((ns + best - 1) / best) + GROUPS - 1) / GROUPS * GROUPS;
       dim3 grid(tiles, (ns + per_cta - 1) / per_cta, nr);
       // seven levels for the short layouts, whose phases are the most accurate: there the six levels'
       // 1.3e-15 of a term would show beside the 1e-16 k rho of its phase
       const bool more = n < 1024;
 #define LSMS_DG(NP)                                                                                       \
-  (more ? launch_digits<NP, 6>(grid, st, c, pc, img, s0, ns, per_cta, r0, maxbits, row0, nrows, alpha, err)           \
-        : launch_digits<NP, 5>(grid, st, c, pc, img, s0, ns, per_cta, r0, maxbits, row0, nrows, alpha, err))
+  (more ? launch_digits<NP, 6>(grid, st, c, pc, img, bound, s0, ns, per_cta, r0, maxbits, row0, nrows, alpha, err)           \
+        : launch_digits<NP, 5>(grid, st, c, pc, img, bound, s0, ns, per_cta, r0, maxbits, row0, nrows, alpha, err))
       if (npad == 32) LSMS_DG(32);
       else if (npad == 48) LSMS_DG(48);
       else LSMS_DG(64);
@@ -531,7 +559,6 @@ int translate_f64_tc(lsms_ctx* c, int nrhs, const double2* xs, double2* alpha, c
     }
   }
   if (f.nnz > 0)
-    k_translate_near_f64<<<dim3((nrows + 3) / 4, nrhs), 128, 0, st>>>(n, p, row0, nrows, f.d_ptr, f.d_idx,
-                                                                      (const double2*)f.d_seq, xs, alpha);
+    launch_near_f64(n, p, nullptr, row0, nrows, 1, f.d_ptr, f.d_idx, (const double2*)f.d_seq, xs, nrhs, alpha, st);
   return check_cuda(c, "translate_f64_tc");
 }

@@ -1,5 +1,5 @@
 // The fixed-point pair sequence of csrc/pair_fixed.cuh on the host: reads "k p dx dy" (hexadecimal
-// floats), prints the four products of every order s = 0..2p as integers with 65 fractional bits.
+// floats), prints the four products of every order s = 0..2p as integers with 64 fractional bits.
 #include <cstdio>
 #include <vector>
 
@@ -26,13 +26,15 @@ int main() {
     PairSeed o;
     pair_seed(dx, dy, r2, q, tab.data(), o);
     PairState a;
-    a.j = o.j0; a.jm = -o.j1; a.y = o.y0; a.ym = -o.y1;
-    a.c = 1LL << 62; a.s = 0; a.f = 0;
-    for (int s = 0; s <= 2 * p; ++s) {
-      int64_t v[4];
-      pair_products(a, v);
-      printf("%lld %lld %lld %lld\n", (long long)v[0], (long long)v[1], (long long)v[2], (long long)v[3]);
-      pair_step(a, o);
+    PairStep t;
+    pair_start(o, a, t);
+    for (int s = 0; s <= 2 * p; s += 2) {
+      int64_t v[8];
+      pair_two_orders(a, t, 0, v);
+      const long long sign = s & 2 ? -1 : 1;     // the sequence's signs + + - -
+      for (int h = 0; h < 2 && s + h <= 2 * p; ++h)
+        printf("%lld %lld %lld %lld\n", sign * (long long)v[4 * h], sign * (long long)v[4 * h + 1],
+               sign * (long long)v[4 * h + 2], sign * (long long)v[4 * h + 3]);
     }
   }
   return 0;

@@ -49,7 +49,7 @@ def test_sequence(program, p):
             phi = mp.atan2(mp.mpf(dy), mp.mpf(dx))
             tol = 1e-15 + 4 * 1.1e-16 * float(z) * math.sqrt(2 / (math.pi * float(z)))
             for s in range(2 * p + 1):
-                got = [mp.mpf(int(t)) / mp.mpf(2) ** 65 for t in next(rows).split()]
+                got = [mp.mpf(int(t)) / mp.mpf(2) ** 64 for t in next(rows).split()]
                 h, c, sn = mp.hankel1(s, z), mp.cos(s * phi), mp.sin(s * phi)
                 for g, e in zip(got, (h.real * c, h.real * sn, h.imag * c, h.imag * sn)):
                     assert abs(g - e) <= tol, (p, s, float(z))
