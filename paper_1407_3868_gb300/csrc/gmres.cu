@@ -68,7 +68,7 @@ struct GmState {
   int reorth;     // 1: the current Arnoldi step needs a second Gram-Schmidt pass
 };
 
-constexpr int DOT_T = 2048;    // elements of w staged per CTA
+constexpr int DOT_T = 2048;    // elements of w staged per CTA, at most
 constexpr int DOT_GY = 8;      // groups of 8 vectors in the grid; a CTA loops over every 8th group
 constexpr int GIVENS_MAX = 4096;
 
@@ -77,13 +77,14 @@ constexpr int GIVENS_MAX = 4096;
 // captured graph follows the Arnoldi step).  V slots are ldv apart; system b occupies elements
 // off[b] .. off[b + 1] of a slot (systems may differ in length: the layouts of a batch).  With a
 // gate the kernel does nothing unless system b needs a second Gram-Schmidt pass.
-// A CTA stages a chunk of DOT_T elements of w in shared memory; each warp takes one basis vector
+// A CTA stages a chunk of `chunk` elements of w in shared memory; each warp takes one basis vector
 // at a time (vectors blockIdx.y * 8 + warp, stepping gridDim.y * 8) with 8 loads in flight per lane
-// and reduces it with shuffles only, so the multi-dot streams the basis at memory speed.
+// and reduces it with shuffles only, so the multi-dot streams the basis at memory speed.  Short
+// systems take shorter chunks (dot_chunk), so that their few elements spread over the SMs' FP64 pipes.
 template <typename T>
 __global__ void __launch_bounds__(256)
 k_mdot(const vec2<T>* __restrict__ V, long long ldv, int nv0, const int* __restrict__ kp,
-       int self_norm, const double2* __restrict__ w, const long long* __restrict__ off,
+       int self_norm, const double2* __restrict__ w, const long long* __restrict__ off, int chunk,
        double2* __restrict__ out, int out_stride, const GmState* __restrict__ gate) {
   using V2 = vec2<T>;
   constexpr int U = 8;
@@ -92,14 +93,14 @@ k_mdot(const vec2<T>* __restrict__ V, long long ldv, int nv0, const int* __restr
   const int nv = nv0 + (kp ? *kp : 0);
   const int ntot = nv + (self_norm ? 1 : 0);
   const long long L = off[b + 1] - off[b];
-  const long long c0 = blockIdx.x * (long long)DOT_T;
+  const long long c0 = blockIdx.x * (long long)chunk;
   if (c0 >= L || (int)blockIdx.y * 8 >= ntot) return;
-  const int cnt = (int)min((long long)DOT_T, L - c0);
+  const int cnt = (int)min((long long)chunk, L - c0);
   V += off[b] + c0;
   w += off[b] + c0;
   out += (long long)b * out_stride;
   __shared__ V2 ws[DOT_T];
-  for (int i = threadIdx.x; i < DOT_T; i += blockDim.x) {
+  for (int i = threadIdx.x; i < (cnt + 32 * U - 1) / (32 * U) * (32 * U); i += blockDim.x) {
     const double2 u = i < cnt ? w[i] : make_double2(0.0, 0.0);
     ws[i] = mk2<T>(u.x, u.y);
   }
@@ -109,7 +110,7 @@ k_mdot(const vec2<T>* __restrict__ V, long long ldv, int nv0, const int* __restr
     T ax = 0, ay = 0, bx = 0, by = 0;
     if (i < nv) {
       const V2* vi = V + (long long)i * ldv;
-      for (int t = lane; t < DOT_T; t += 32 * U) {
+      for (int t = lane; t < cnt; t += 32 * U) {
         V2 v[U];
 #pragma unroll
         for (int u = 0; u < U; ++u) {
@@ -139,19 +140,35 @@ k_mdot(const vec2<T>* __restrict__ V, long long ldv, int nv0, const int* __restr
   }
 }
 
+// After the first Gram-Schmidt pass of a system: h1[0..k] = V^H w, h1[k+1] = ||w||^2.  The first pass
+// removes ||h1||^2 from ||w||^2; if more than about half of it goes (||w'|| < 0.7 ||w||), cancellation
+// may have left w' not orthogonal enough and a second pass runs.  One warp.
+__device__ __forceinline__ void gm_prep(int k, const double2* __restrict__ h1, GmState* __restrict__ st) {
+  double s = 0.0;
+  for (int i = threadIdx.x; i <= k; i += 32) s += h1[i].x * h1[i].x + h1[i].y * h1[i].y;
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+  if (threadIdx.x == 0) {
+    const double a = h1[k + 1].x;
+    st->reorth = (a - s < 0.49 * a) ? 1 : 0;
+  }
+}
+
 // System b = blockIdx.y:  w[b][t] += sign sum_{i < nv_b} V[i][b][t] h[b][i] over the system's
 // elements off[b] .. off[b + 1].  nv_b = nv, or nv_arr[b] when given; with a gate only when system b
-// needs a second pass.
+// needs a second pass.  prep (the first Gram-Schmidt pass): the first CTA of a system decides whether
+// it needs one (gm_prep).  Blocks of 64 threads where that spreads a short system over more SMs.
 template <typename T>
 __global__ void __launch_bounds__(256)
 k_maxpy(const vec2<T>* __restrict__ V, long long ldv, int nv, const int* __restrict__ nv_arr,
         const int* __restrict__ kp, const double2* __restrict__ h, int h_stride,
         double2* __restrict__ w, const long long* __restrict__ off, double sign,
-        const GmState* __restrict__ gate) {
+        const GmState* __restrict__ gate, GmState* __restrict__ prep) {
   using V2 = vec2<T>;
   const int b = blockIdx.y;
   if (gate && !gate[b].reorth) return;
   const long long L = off[b + 1] - off[b];
+  if (prep && blockIdx.x == 0 && threadIdx.x < 32) gm_prep(*kp, h + (long long)b * h_stride, prep + b);
   if (blockIdx.x * (long long)blockDim.x >= L) return;
   if (nv_arr) nv = nv_arr[b];
   if (kp) nv += *kp;
@@ -164,9 +181,9 @@ k_maxpy(const vec2<T>* __restrict__ V, long long ldv, int nv, const int* __restr
   for (int i0 = 0; i0 < nv; i0 += 256) {
     const int c = min(256, nv - i0);
     __syncthreads();
-    if (threadIdx.x < c) {
-      const double2 u = h[i0 + threadIdx.x];
-      hs[threadIdx.x] = mk2<T>(u.x, u.y);
+    for (int i = threadIdx.x; i < c; i += blockDim.x) {
+      const double2 u = h[i0 + i];
+      hs[i] = mk2<T>(u.x, u.y);
     }
     __syncthreads();
     if (t < L) {
@@ -200,26 +217,12 @@ k_maxpy(const vec2<T>* __restrict__ V, long long ldv, int nv, const int* __restr
   }
 }
 
-// After the first Gram-Schmidt pass of system b = blockIdx.x: h1[0..k] = V^H w, h1[k+1] = ||w||^2.
-// The first pass removes ||h1||^2 from ||w||^2; if more than about half of it goes
-// (||w'|| < 0.7 ||w||), cancellation may have left w' not orthogonal enough and a second pass runs.
-__global__ void __launch_bounds__(32) k_gm_prep(const int* __restrict__ kp, const double2* __restrict__ h1,
-                                                int stride, GmState* __restrict__ st) {
-  const int k = *kp;
-  h1 += (long long)blockIdx.x * stride;
-  double s = 0.0;
-  for (int i = threadIdx.x; i <= k; i += 32) s += h1[i].x * h1[i].x + h1[i].y * h1[i].y;
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-  if (threadIdx.x == 0) {
-    const double a = h1[k + 1].x;
-    st[blockIdx.x].reorth = (a - s < 0.49 * a) ? 1 : 0;
-  }
-}
-
 // Column k of system b = blockIdx.x: H[0..k][k] = h1 + h2, H[k+1][k] = ||w_final||; apply the
-// previous Givens rotations, form the new one, update g and the residual estimate.  The lanes
-// stage the column and the rotations in shared memory, lane 0 sweeps them.
+// previous Givens rotations, form the new one, update g and the residual estimate.  One warp.
+// The rotations run down the column as a_{i+1} = -s_i a_i + c_i col[i+1] (s_i real, |s_i| <= 1), new
+// col[i] = conj(c_i) a_i + s_i col[i+1]: an affine recurrence, so each lane composes a run of maps, a
+// scan over the lanes gives every run its first a, and a second sweep finishes the runs: k / 32 + 5
+// dependent steps instead of k (a dependent FP64 operation takes tens of cycles here).
 __global__ void __launch_bounds__(32)
 k_gm_column(const int* __restrict__ kp, const double2* __restrict__ h1, const double2* __restrict__ h2,
             int stride, double2* __restrict__ H, long long hstride, int ldh, double2* __restrict__ cs,
@@ -249,26 +252,53 @@ k_gm_column(const int* __restrict__ kp, const double2* __restrict__ h1, const do
   for (int i = lane; i <= k; i += 32) s2 += hl[i].x * hl[i].x + hl[i].y * hl[i].y;
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) s2 += __shfl_xor_sync(0xffffffffu, s2, o);
+  const double hn = sqrt(fmax(hl[k + 1].x - s2, 0.0));
+  __syncwarp();
+  const int per = (k + 31) / 32, i0 = min(k, lane * per), i1 = min(k, i0 + per);
+  // a -> am a + ab over the lane's run
+  double am = 1.0;
+  double2 ab = make_double2(0.0, 0.0);
+  for (int i = i0; i < i1; ++i) {
+    const double si = -s_s[i].x;
+    const double2 m = cmul(c_s[i], col[i + 1]);
+    am *= si;
+    ab = make_double2(fma(si, ab.x, m.x), fma(si, ab.y, m.y));
+  }
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {    // inclusive: the runs of lanes 0 .. lane
+    const double pm = __shfl_up_sync(0xffffffffu, am, o);
+    const double px = __shfl_up_sync(0xffffffffu, ab.x, o), py = __shfl_up_sync(0xffffffffu, ab.y, o);
+    if (lane >= o) {
+      ab = make_double2(fma(am, px, ab.x), fma(am, py, ab.y));
+      am *= pm;
+    }
+  }
+  const double2 a0 = col[0];
+  const double2 full = make_double2(fma(am, a0.x, ab.x), fma(am, a0.y, ab.y));   // a behind this run
+  double2 a;
+  a.x = __shfl_up_sync(0xffffffffu, full.x, 1);
+  a.y = __shfl_up_sync(0xffffffffu, full.y, 1);
+  if (lane == 0) a = a0;
+  double2 last = make_double2(__shfl_sync(0xffffffffu, full.x, 31), __shfl_sync(0xffffffffu, full.y, 31));
+  if (k == 0) last = a0;
+  const double2 next = i1 < k && i1 > i0 ? col[i1] : make_double2(0.0, 0.0);     // before a neighbour writes it
+  __syncwarp();
+  for (int i = i0; i < i1; ++i) {
+    const double2 bb = i + 1 < i1 || i + 1 == k ? col[i + 1] : next;
+    const double2 ci = c_s[i];
+    const double si = s_s[i].x;
+    const double2 t = cjmul(ci, a), m = cmul(ci, bb);
+    col[i] = make_double2(fma(si, bb.x, t.x), fma(si, bb.y, t.y));
+    a = make_double2(fma(-si, a.x, m.x), fma(-si, a.y, m.y));
+  }
   __syncwarp();
   if (lane == 0) {
-    const double hn = sqrt(fmax(hl[k + 1].x - s2, 0.0));
     s->hn = hn;
     s->inv = hn > 0.0 ? 1.0 / hn : 0.0;
-    col[k + 1] = make_double2(hn, 0.0);
-    for (int i = 0; i < k; ++i) {
-      const double2 a = col[i], bb = col[i + 1];
-      const double2 ci = c_s[i], si = s_s[i];
-      // [conj(c) conj(s); -s c] [a; b]
-      const double2 t = make_double2(cjmul(ci, a).x + cjmul(si, bb).x, cjmul(ci, a).y + cjmul(si, bb).y);
-      const double2 u = make_double2(-cmul(si, a).x + cmul(ci, bb).x, -cmul(si, a).y + cmul(ci, bb).y);
-      col[i] = t;
-      col[i + 1] = u;
-    }
-    const double2 a = col[k];
-    const double r = hypot(hypot(a.x, a.y), hn);
+    const double r = hypot(hypot(last.x, last.y), hn);
     double2 c, sg;
     if (r > 0.0) {
-      c = make_double2(a.x / r, a.y / r);
+      c = make_double2(last.x / r, last.y / r);
       sg = make_double2(hn / r, 0.0);
     } else {
       c = make_double2(1.0, 0.0);
@@ -290,31 +320,30 @@ k_gm_column(const int* __restrict__ kp, const double2* __restrict__ h1, const do
   for (int i = lane; i <= k + 1; i += 32) Hc[i] = col[i];
 }
 
-// Back substitution of system b = blockIdx.x: H[0..k_b)[0..k_b) y = g, one warp.
-__global__ void k_gm_backsolve(const int* __restrict__ kk, const double2* __restrict__ H,
-                               long long hstride, int ldh, const double2* __restrict__ g, int stride,
-                               double2* __restrict__ y) {
+// Back substitution of system b = blockIdx.x: H[0..k_b)[0..k_b) y = g, one warp, by columns: once y_i is
+// known the lanes take H's column i (contiguous) times y_i out of the remaining right-hand side in y.
+__global__ void __launch_bounds__(32)
+k_gm_backsolve(const int* __restrict__ kk, const double2* __restrict__ H, long long hstride, int ldh,
+               const double2* __restrict__ g, int stride, double2* __restrict__ y) {
   const int b = blockIdx.x;
   const int k = kk[b];
   H += (long long)b * hstride;
   g += (long long)b * stride;
   y += (long long)b * stride;
   const int lane = threadIdx.x;
+  for (int i = lane; i < k; i += 32) y[i] = g[i];
+  __syncwarp();
   for (int i = k - 1; i >= 0; --i) {
-    double2 s = make_double2(0.0, 0.0);
-    for (int j = i + 1 + lane; j < k; j += 32) {
-      const double2 c = cmul(H[(long long)j * ldh + i], y[j]);
-      s.x += c.x;
-      s.y += c.y;
+    const double2 num = y[i], d = H[(long long)i * ldh + i];
+    const double dd = d.x * d.x + d.y * d.y;
+    const double2 v = dd > 0.0 ? make_double2((num.x * d.x + num.y * d.y) / dd, (num.y * d.x - num.x * d.y) / dd)
+                               : make_double2(0.0, 0.0);
+    __syncwarp();
+    for (int j = lane; j < i; j += 32) {
+      const double2 t = cmul(H[(long long)i * ldh + j], v), o = y[j];
+      y[j] = make_double2(o.x - t.x, o.y - t.y);
     }
-    s = warp_sum(s);
-    if (lane == 0) {
-      const double2 num = make_double2(g[i].x - s.x, g[i].y - s.y);
-      const double2 d = H[(long long)i * ldh + i];
-      const double dd = d.x * d.x + d.y * d.y;
-      y[i] = dd > 0.0 ? make_double2((num.x * d.x + num.y * d.y) / dd, (num.y * d.x - num.x * d.y) / dd)
-                      : make_double2(0.0, 0.0);
-    }
+    if (lane == 0) y[i] = v;
     __syncwarp();
   }
 }
@@ -335,7 +364,7 @@ __global__ void k_scale_by(vec2<T>* __restrict__ dst, const double2* __restrict_
   }
 }
 
-// X[b] = V[k][b] (the operator's fixed input buffer)
+// X = V[k] (the operator's fixed input buffer, first step)
 template <typename T>
 __global__ void k_copy_slot(double2* __restrict__ X, const vec2<T>* __restrict__ V, long long slot,
                             const int* __restrict__ kp) {
@@ -345,21 +374,31 @@ __global__ void k_copy_slot(double2* __restrict__ X, const vec2<T>* __restrict__
     X[t] = to_d2(src[t]);
 }
 
-// V[k + 1][b] = W[b] * st[b].inv   (system b = blockIdx.y)
+// V[k + 1][b] = W[b] * st[b].inv (system b = blockIdx.y), the same into X, the operator's fixed input
+// of the next step, rounded as the basis is; the first CTA of a system zeroes the dot products of that step.
 template <typename T>
 __global__ void k_scale_into_slot(vec2<T>* __restrict__ V, long long slot, const double2* __restrict__ W,
                                   const GmState* __restrict__ st, const long long* __restrict__ off,
-                                  const int* __restrict__ kp) {
-  const int b = blockIdx.y;
+                                  const int* __restrict__ kp, double2* __restrict__ X, double2* __restrict__ h1,
+                                  double2* __restrict__ h2, int stride) {
+  const int b = blockIdx.y, k = *kp;
   const double s = st[b].inv;
   const long long L = off[b + 1] - off[b];
-  vec2<T>* dst = V + (long long)(*kp + 1) * slot + off[b];
+  vec2<T>* dst = V + (long long)(k + 1) * slot + off[b];
   const double2* src = W + off[b];
+  X += off[b];
   for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < L;
        t += (long long)gridDim.x * blockDim.x) {
     const double2 v = src[t];
-    dst[t] = mk2<T>(v.x * s, v.y * s);
+    const vec2<T> u = mk2<T>(v.x * s, v.y * s);
+    dst[t] = u;
+    X[t] = to_d2(u);
   }
+  if (blockIdx.x == 0)
+    for (int i = threadIdx.x; i < min(stride, k + 4); i += blockDim.x) {
+      h1[(long long)b * stride + i] = make_double2(0.0, 0.0);
+      h2[(long long)b * stride + i] = make_double2(0.0, 0.0);
+    }
 }
 
 // ring[k mod ring_slots][b] = st[b] (host-mapped memory), then k += 1.  One block.
@@ -372,13 +411,12 @@ __global__ void k_gm_snapshot(const GmState* __restrict__ st, int nb, GmState* _
   if (threadIdx.x == 0) *kp = k + 1;
 }
 
-// The stopping test of the graph-resident loop, after the step counter has counted this Arnoldi
-// step (k steps done): a system that met its tolerance, broke down (hn = 0) or saw a non-finite
+// The stopping test of the graph-resident loop; it counts this Arnoldi step (k steps done): a system that met its tolerance, broke down (hn = 0) or saw a non-finite
 // value keeps k as its iteration count; the loop's condition becomes 0 when no system is left, a
 // non-finite value appeared or k reached maxiter.  hist (one system): its residual after each step.
 // One block.
 __global__ void k_gm_decide(const GmState* __restrict__ st, int nb, const double* __restrict__ tol,
-                            int* __restrict__ kdone, double* __restrict__ res, const int* __restrict__ kp,
+                            int* __restrict__ kdone, double* __restrict__ res, int* __restrict__ kp,
                             int maxiter, int* __restrict__ nonfinite, int* __restrict__ guard,
                             double* __restrict__ hist, int hist_cap, cudaGraphConditionalHandle cond) {
   __shared__ int active, bad;
@@ -387,7 +425,7 @@ __global__ void k_gm_decide(const GmState* __restrict__ st, int nb, const double
     bad = 0;
   }
   __syncthreads();
-  const int k = *kp;
+  const int k = *kp + 1;                          // steps done, this one included
   const int runs = *guard + 1;                    // executions of this test: bounds the loop by itself
   for (int b = threadIdx.x; b < nb; b += blockDim.x) {
     if (kdone[b] >= 0) continue;
@@ -401,6 +439,7 @@ __global__ void k_gm_decide(const GmState* __restrict__ st, int nb, const double
   if (threadIdx.x == 0) {
     if (hist && k >= 1 && k <= hist_cap) hist[k - 1] = st[0].res;
     if (bad) *nonfinite = 1;
+    *kp = k;
     *guard = runs;
     cudaGraphSetConditional(cond, (active > 0 && !bad && k < maxiter && runs < maxiter) ? 1u : 0u);
   }
@@ -476,21 +515,30 @@ inline int grid_for(long long total, int block) {
   return (int)g;
 }
 
+// Elements of w per CTA of k_mdot (a multiple of the 256 that a warp loads at once): as many CTAs as
+// SMs where the systems are long enough; 2048 is where the atomic sums stop mattering.
+inline int dot_chunk(long long total) {
+  return total <= 152 * 256 ? 256 : total <= 152 * 512 ? 512 : total <= 152 * 1024 ? 1024 : DOT_T;
+}
+inline int axpy_block(long long total) { return total <= 152 * 256 ? 64 : 256; }
+
 // out[b * out_stride + i] = V_b[i]^H w_b, i < nv, for the systems of s
 template <typename T>
 void mdot(const vec2<T>* V, long long ldv, int nv, const double2* w, const GmSys& s, double2* out,
           int out_stride, cudaStream_t st) {
   for (int b = 0; b < s.nb; ++b)
     cudaMemsetAsync(out + (long long)b * out_stride, 0, (size_t)nv * sizeof(double2), st);
-  dim3 grid((unsigned)((s.maxlen + DOT_T - 1) / DOT_T), (unsigned)std::min(DOT_GY, (nv + 7) / 8), (unsigned)s.nb);
-  k_mdot<T><<<grid, 256, 0, st>>>(V, ldv, nv, nullptr, 0, w, s.d_off, out, out_stride, nullptr);
+  const int chunk = dot_chunk(s.maxlen * s.nb);
+  dim3 grid((unsigned)((s.maxlen + chunk - 1) / chunk), (unsigned)std::min(DOT_GY, (nv + 7) / 8), (unsigned)s.nb);
+  k_mdot<T><<<grid, 256, 0, st>>>(V, ldv, nv, nullptr, 0, w, s.d_off, chunk, out, out_stride, nullptr);
 }
 
 template <typename T>
 void maxpy(const vec2<T>* V, long long ldv, int nv, const int* nv_arr, const double2* h, int h_stride,
            double2* w, const GmSys& s, double sign, cudaStream_t st) {
-  dim3 grid((unsigned)((s.maxlen + 255) / 256), (unsigned)s.nb);
-  k_maxpy<T><<<grid, 256, 0, st>>>(V, ldv, nv, nv_arr, nullptr, h, h_stride, w, s.d_off, sign, nullptr);
+  const int blk = axpy_block(s.maxlen * s.nb);
+  dim3 grid((unsigned)((s.maxlen + blk - 1) / blk), (unsigned)s.nb);
+  k_maxpy<T><<<grid, blk, 0, st>>>(V, ldv, nv, nv_arr, nullptr, h, h_stride, w, s.d_off, sign, nullptr, nullptr);
 }
 
 // Device scratch of one batched GMRES run.
@@ -560,31 +608,31 @@ int ensure_ring(lsms_ctx* c, int nb) {
   return LSMS_OK;
 }
 
-// One Arnoldi step of every system, with the step index read on the device (capturable).
+// One Arnoldi step of every system, with the step index read on the device (capturable): X holds basis
+// vector k, the dot products are zero on entry; k_gm_decide (the device loop) or k_gm_snapshot (the
+// host loop, `ring`) counts the step.
 template <typename T>
-int enqueue_iteration(lsms_ctx* c, const GmPtrs& g, const GmSys& s, int maxiter, int flags,
+int enqueue_iteration(lsms_ctx* c, const GmPtrs& g, const GmSys& s, int maxiter, int flags, bool ring,
                       cudaStream_t st) {
   const long long slot = s.slot;
   const int nb = s.nb;
   vec2<T>* V = (vec2<T>*)g.V;
   int rc;
-  k_copy_slot<T><<<grid_for(slot, 256), 256, 0, st>>>(g.X, V, slot, g.dk);
   if ((rc = apply_device(c, s.apply_nrhs, g.X, g.W, flags, st))) return rc;
-  const dim3 gd((unsigned)((s.maxlen + DOT_T - 1) / DOT_T), (unsigned)std::min(DOT_GY, (maxiter + 2 + 7) / 8),
+  const int chunk = dot_chunk(s.maxlen * nb), blk = axpy_block(s.maxlen * nb);
+  const dim3 gd((unsigned)((s.maxlen + chunk - 1) / chunk), (unsigned)std::min(DOT_GY, (maxiter + 2 + 7) / 8),
                 (unsigned)nb);
-  const dim3 ga((unsigned)((s.maxlen + 255) / 256), (unsigned)nb);
+  const dim3 ga((unsigned)((s.maxlen + blk - 1) / blk), (unsigned)nb);
   // classical Gram-Schmidt; the second pass runs only when the first cancels much of w
-  cudaMemsetAsync(g.h1, 0, (size_t)nb * g.stride * sizeof(double2), st);
-  k_mdot<T><<<gd, 256, 0, st>>>(V, slot, 1, g.dk, 1, g.W, s.d_off, g.h1, g.stride, nullptr);   // V^H w, ||w||^2
-  k_gm_prep<<<nb, 32, 0, st>>>(g.dk, g.h1, g.stride, g.st);
-  k_maxpy<T><<<ga, 256, 0, st>>>(V, slot, 1, nullptr, g.dk, g.h1, g.stride, g.W, s.d_off, -1.0, nullptr);
-  cudaMemsetAsync(g.h2, 0, (size_t)nb * g.stride * sizeof(double2), st);
-  k_mdot<T><<<gd, 256, 0, st>>>(V, slot, 1, g.dk, 1, g.W, s.d_off, g.h2, g.stride, g.st);
-  k_maxpy<T><<<ga, 256, 0, st>>>(V, slot, 1, nullptr, g.dk, g.h2, g.stride, g.W, s.d_off, -1.0, g.st);
+  k_mdot<T><<<gd, 256, 0, st>>>(V, slot, 1, g.dk, 1, g.W, s.d_off, chunk, g.h1, g.stride, nullptr);   // V^H w, ||w||^2
+  k_maxpy<T><<<ga, blk, 0, st>>>(V, slot, 1, nullptr, g.dk, g.h1, g.stride, g.W, s.d_off, -1.0, nullptr, g.st);
+  k_mdot<T><<<gd, 256, 0, st>>>(V, slot, 1, g.dk, 1, g.W, s.d_off, chunk, g.h2, g.stride, g.st);
+  k_maxpy<T><<<ga, blk, 0, st>>>(V, slot, 1, nullptr, g.dk, g.h2, g.stride, g.W, s.d_off, -1.0, g.st, nullptr);
   k_gm_column<<<nb, 32, (size_t)(3 * maxiter + 2) * sizeof(double2), st>>>(
       g.dk, g.h1, g.h2, g.stride, g.H, g.hstride, g.ldh, g.cs, g.sn, g.g, g.st);
-  k_scale_into_slot<T><<<dim3(grid_for(s.maxlen, 256), nb), 256, 0, st>>>(V, slot, g.W, g.st, s.d_off, g.dk);
-  k_gm_snapshot<<<1, 256, 0, st>>>(g.st, nb, (GmState*)c->gm_ring_dev, RING, g.dk);
+  k_scale_into_slot<T><<<dim3(grid_for(s.maxlen, 256), nb), 256, 0, st>>>(V, slot, g.W, g.st, s.d_off, g.dk, g.X,
+                                                                        g.h1, g.h2, g.stride);
+  if (ring) k_gm_snapshot<<<1, 256, 0, st>>>(g.st, nb, (GmState*)c->gm_ring_dev, RING, g.dk);
   return check_cuda(c, "gmres iteration");
 }
 
@@ -669,7 +717,7 @@ int gmres_device_loop(lsms_ctx* c, const GmPtrs& g, const GmSys& s, const double
         cudaGraph_t body = cp.conditional.phGraph_out[0];
         if (cudaStreamBeginCaptureToGraph(stream, body, nullptr, nullptr, 0, cudaStreamCaptureModeThreadLocal) ==
             cudaSuccess) {
-          int erc = enqueue_iteration<T>(c, g, s, maxiter, flags, stream);
+          int erc = enqueue_iteration<T>(c, g, s, maxiter, flags, false, stream);
           if (erc == LSMS_OK)
             k_gm_decide<<<1, 256, 0, stream>>>(g.st, nb, d_tol, d_kdone, d_res, g.dk, maxiter, d_bad, d_guard,
                                                 hcap ? d_hist : nullptr, hcap, cond);
@@ -743,6 +791,8 @@ int gmres_batch_t(lsms_ctx* c, const GmSys& s, const double2* rhs, double2* x, b
   k_gm_start<<<nb, 1, 0, stream>>>(g.nrm, g.st, g.g, g.stride);
   k_scale_by<T><<<dim3(grid_for(s.maxlen, 256), nb), 256, 0, stream>>>(V, r0, g.st, s.d_off);
   cudaMemsetAsync(g.dk, 0, sizeof(int), stream);
+  cudaMemsetAsync(g.h1, 0, (size_t)2 * nb * g.stride * sizeof(double2), stream);   // h1 and h2
+  k_copy_slot<T><<<grid_for(slot, 256), 256, 0, stream>>>(g.X, V, slot, g.dk);
   cudaStreamSynchronize(stream);
   if ((rc = check_cuda(c, "gmres start"))) return rc;
   std::vector<GmState> s0(nb);
@@ -783,7 +833,7 @@ int gmres_batch_t(lsms_ctx* c, const GmSys& s, const double2* rhs, double2* x, b
     c->timing = 0;
     cudaGraph_t graph = nullptr;
     if (cudaStreamBeginCapture(stream, cudaStreamCaptureModeThreadLocal) == cudaSuccess) {
-      const int erc = enqueue_iteration<T>(c, g, s, maxiter, flags, stream);
+      const int erc = enqueue_iteration<T>(c, g, s, maxiter, flags, true, stream);
       const cudaError_t e = cudaStreamEndCapture(stream, &graph);
       if (erc == LSMS_OK && e == cudaSuccess && graph &&
           cudaGraphInstantiate(&exec, graph, 0) != cudaSuccess)
@@ -816,7 +866,7 @@ int gmres_batch_t(lsms_ctx* c, const GmSys& s, const double2* rhs, double2* x, b
         cudaGraphExecDestroy(exec);
         return check_cuda(c, "cudaGraphLaunch");
       }
-    } else if ((rc = enqueue_iteration<T>(c, g, s, maxiter, flags, stream))) {
+    } else if ((rc = enqueue_iteration<T>(c, g, s, maxiter, flags, true, stream))) {
       return rc;
     }
     cudaEventRecord(c->gm_ev[k % RING], stream);
