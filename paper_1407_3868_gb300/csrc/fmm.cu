@@ -29,12 +29,14 @@
 
 #include "c64.cuh"
 #include "ff_hankel.cuh"
+#include "near_f64.cuh"
 #include "near_pairs.cuh"
 #include "lsms_internal.h"
 #include "lsms_ops.h"
 
 namespace {
 
+constexpr size_t kSeq64Bytes = (size_t)8 << 30;   // FP64 near sequences stored up to here
 constexpr int FW = 4;     // target discs (warps) per CTA of the near-field kernel
 constexpr int FCH = 32;   // source discs per staged chunk
 constexpr int FHS = 65;   // pair sequence stride (4p + 1 <= 61)
@@ -76,29 +78,37 @@ __global__ void k_fmm_shift_table(const double* __restrict__ cx, const double* _
   }
 }
 
-// The mixed near field's pair sequences: row k of seq = h[s + 2p] = H_s(k rho) e^{i s phi}, s =
-// -2p..2p (then one zero), for list entry k (target perm[t], source csrc[k]); built in FP64 (CUDA
-// J0, Y0, J1, Y1, forward recurrence, angular powers) and stored in FP32.  One thread per target.
+// The near field's pair sequences: row k of seq = h[s + 2p] = H_s(k rho) e^{i s phi}, s = -2p..2p (then
+// one zero), for list entry k (target perm[t], source csrc[k]); built in FP64 (CUDA J0, Y0, J1, Y1,
+// forward recurrence, angular powers) and stored in FP32, and in FP64 (rows of 4p + 1) where seq64 is
+// given.  A warp per target, a lane per pair.
 __global__ void k_fmm_pair_seq(const double* __restrict__ cx, const double* __restrict__ cy,
                                const int* __restrict__ perm, const int* __restrict__ cptr,
-                               const int* __restrict__ csrc, int n, int p, double k, float2* __restrict__ seq) {
-  const int t = blockIdx.x * blockDim.x + threadIdx.x;
+                               const int* __restrict__ csrc, int n, int p, double k, float2* __restrict__ seq,
+                               double2* __restrict__ seq64) {
+  const int t = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   if (t >= n) return;
   const int l = perm[t], RS = 4 * p + 2, c0 = 2 * p;
-  for (int e = cptr[t]; e < cptr[t + 1]; ++e) {
+  for (int e = cptr[t] + (threadIdx.x & 31); e < cptr[t + 1]; e += 32) {
     const int m = csrc[e];
     const double dx = cx[l] - cx[m], dy = cy[l] - cy[m];
     const double rho = hypot(dx, dy), z = k * rho;
     const double2 e1 = make_double2(dx / rho, dy / rho);
     float2* h = seq + (size_t)e * RS;
+    double2* h64 = seq64 ? seq64 + (size_t)e * (4 * p + 1) : nullptr;
     double2 hm = make_double2(j0(z), y0(z)), hq = make_double2(j1(z), y1(z)), eq = e1;
     h[c0] = make_float2((float)hm.x, (float)hm.y);
+    if (h64) h64[c0] = hm;
     for (int q = 1; q <= 2 * p; ++q) {
       const double2 v = cmul(hq, eq);
-      const double2 u = cmul(hq, make_double2(eq.x, -eq.y));
-      const double sg = (q & 1) ? -1.0 : 1.0;
+      double2 u = cmul(hq, make_double2(eq.x, -eq.y));
+      if (q & 1) u = make_double2(-u.x, -u.y);
       h[c0 + q] = make_float2((float)v.x, (float)v.y);
-      h[c0 - q] = make_float2((float)(sg * u.x), (float)(sg * u.y));
+      h[c0 - q] = make_float2((float)u.x, (float)u.y);
+      if (h64) {
+        h64[c0 + q] = v;
+        h64[c0 - q] = u;
+      }
       if (q < 2 * p) {
         const double f = 2.0 * q / z;
         const double2 hn = make_double2(f * hq.x - hm.x, f * hq.y - hm.y);
@@ -702,7 +712,7 @@ void fmm_free(lsms_ctx* c) {
   FmmState& f = c->fmm;
   void* ptrs[] = {f.d_perm,  f.d_bstart, f.d_dbox,   f.d_sbox,   f.d_scx,  f.d_scy,   f.d_tab,   f.d_khat,
                   f.d_grid,  f.d_bq,     f.d_acc,    f.d_hd,     f.d_twn,  f.d_tw2,   f.d_cptr,  f.d_csrc,
-                  f.d_cseq,  f.ws.ptr,
+                  f.d_cseq,  f.d_cseq64, f.ws.ptr,
                   f.d_tab32, f.d_khat32, f.d_grid32, f.d_bq32,   f.d_acc32, f.d_hd32, f.d_twn32, f.d_tw232};
   for (void* q : ptrs)
     if (q) cudaFree(q);
@@ -808,8 +818,15 @@ int fmm_setup(lsms_ctx* c) {
   cudaMemcpy(f.d_cptr, cptr.data(), (n + 1) * sizeof(int), cudaMemcpyHostToDevice);
   if (!csrc.empty()) cudaMemcpy(f.d_csrc, csrc.data(), csrc.size() * sizeof(int), cudaMemcpyHostToDevice);
   cudaStream_t st = c->stream;
-  k_fmm_pair_seq<<<(n + 127) / 128, 128, 0, st>>>(c->d_cx, c->d_cy, f.d_perm, f.d_cptr, f.d_csrc, n, p, c->k2,
-                                                  f.d_cseq);
+  // FP64 near field: the stored sequences (430 MB for 20,000 discs at p = 14) if they are few and fit;
+  // otherwise k_fmm_near forms them anew in every application
+  const size_t seq64 = csrc.size() * (size_t)(4 * p + 1) * sizeof(double2);
+  if (seq64 > 0 && seq64 <= kSeq64Bytes && cudaMalloc((void**)&f.d_cseq64, seq64) != cudaSuccess) {
+    cudaGetLastError();
+    f.d_cseq64 = nullptr;
+  }
+  k_fmm_pair_seq<<<(n + 3) / 4, 128, 0, st>>>(c->d_cx, c->d_cy, f.d_perm, f.d_cptr, f.d_csrc, n, p, c->k2, f.d_cseq,
+                                              f.d_cseq64);
   if (!f.far) {                    // near field only
     cudaStreamSynchronize(st);
     f.ready = true;
@@ -891,6 +908,13 @@ int fmm_translate(lsms_ctx* c, int nrhs, const double2* xs, double2* alpha, bool
     if (timed) cudaEventRecord(f.ev[1], st);
     k_fmm_d2f<<<blocks_for(len, 256), 256, 0, st>>>(xs, x32, len);
     launch_pair_seq(p, nrhs, st, f.d_perm, f.d_cptr, f.d_csrc, f.d_cseq, n, x32, alpha);
+    if (timed) cudaEventRecord(f.ev[2], st);
+    f.timed = timed;
+    return LSMS_OK;
+  }
+  if (f.d_cseq64) {
+    if (timed) cudaEventRecord(f.ev[1], st);
+    launch_near_f64(n, p, f.d_perm, 0, n, 1, f.d_cptr, f.d_csrc, f.d_cseq64, xs, nrhs, alpha, st);
     if (timed) cudaEventRecord(f.ev[2], st);
     f.timed = timed;
     return LSMS_OK;
