@@ -115,6 +115,21 @@ int apply_device(lsms_ctx* c, int nrhs, const double2* x, double2* y, int flags,
   const bool given = (flags & LSMS_APPLY_TRANSLATION_GIVEN) && c->alpha_given;
   double2* alpha = given ? c->alpha_given : (double2*)c->ws_alpha.ptr;
   int launches = 0;
+  const bool boxes = c->fmm.ready && (c->fmm.scope == 0 || (flags & LSMS_APPLY_RESIDUAL_INTERNAL));
+  if (mixed && c->side && !given && !boxes && !(flags & (LSMS_APPLY_NO_TRANSLATION | LSMS_APPLY_NO_REFLECTION)) &&
+      mixed_sym_path(c, nrhs)) {
+    const float2* acc = nullptr;
+    if ((rc = mixed_sym_sums(c, nrhs, x, c->d_scale_in + mode * P, xs, alpha, &acc, st))) return rc;
+    const bool dense = c->dense && !(flags & LSMS_APPLY_ALPHA);
+    launch_mixed_end(c, dense || (flags & LSMS_APPLY_ALPHA) ? nullptr : x, alpha, acc, c->d_scale_out + mode * P, nrhs,
+                     dense ? alpha : y, st);
+    if (dense)
+      launch_scatter_dense(x, alpha, c->d_smt + (size_t)mode * P * P,
+                           c->has_theta ? (const double*)c->theta_buf.ptr : nullptr, nrhs, n, P, y, st);
+    // start, pair kernel, end; split, GEMM, per-node stage, GEMM; near pairs
+    c->last_launches = 7 + (c->near_nnz > 0 ? 1 : 0) + (dense ? 1 : 0);
+    return check_cuda(c, "apply");
+  }
   launch_scale_in(x, c->d_scale_in + mode * P, xs, nrhs, n, P, st);
   ++launches;
   if (c->timing) cudaEventRecord(c->ev[0], st);
@@ -136,7 +151,7 @@ int apply_device(lsms_ctx* c, int nrhs, const double2* x, double2* y, int flags,
     if (given) {
       // computed for every layout of the batch at once (translate_mixed_batch)
       cudaStreamWaitEvent(st, c->alpha_ready, 0);
-    } else if (c->fmm.ready && (c->fmm.scope == 0 || (flags & LSMS_APPLY_RESIDUAL_INTERNAL))) {
+    } else if (boxes) {
       if (c->fmm.far) launches += (c->fmm.dmin > 2 ? 8 : 7) * nrhs;
       launches += mixed ? 2 : 1;
       if ((rc = fmm_translate(c, nrhs, xs, alpha, mixed, st))) return rc;

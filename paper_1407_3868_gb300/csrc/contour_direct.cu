@@ -32,7 +32,7 @@ __device__ __forceinline__ double2 row_sum(const double2* __restrict__ a, const 
 __global__ void __launch_bounds__(128)
 k_zgemm_direct(const double2* __restrict__ A, int M, int K, const double2* __restrict__ B, double2* __restrict__ C,
                int P, int per) {
-  const int w = blockIdx.x * 4 + (threadIdx.x >> 5), lane = threadIdx.x & 31, r = blockIdx.y;
+  const int w = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5), lane = threadIdx.x & 31, r = blockIdx.y;
   const int chunks = (K + per - 1) / per, m = w / chunks;
   if (m >= M) return;
   const int k0 = (w - m * chunks) * per;
@@ -50,7 +50,7 @@ __global__ void __launch_bounds__(128)
 k_node_direct(int ns, int n, int P, const double2* __restrict__ eagg, const double2* __restrict__ xs,
               const double2* __restrict__ fagg, const double2* __restrict__ refl, const double2* __restrict__ udis,
               double2* __restrict__ V) {
-  const int v = blockIdx.x * 4 + (threadIdx.x >> 5), lane = threadIdx.x & 31, r = blockIdx.y;
+  const int v = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5), lane = threadIdx.x & 31, r = blockIdx.y;
   if (v >= ns) return;
   const int q = min(lane, P - 1);
   const double2* b = xs + (size_t)r * n * P;
@@ -75,10 +75,13 @@ void launch_zgemm_direct(const double2* A, int M, int K, const double2* B, doubl
   // about 16 warps per SM, at least 16 elements of K each
   const int chunks = (int)std::max<long long>(1, std::min<long long>((K + 15) / 16, 152LL * 16 / std::max(1LL, (long long)M * nrhs)));
   const int per = (K + chunks - 1) / chunks, nc = (K + per - 1) / per;
-  k_zgemm_direct<<<dim3((unsigned)(((long long)M * nc + 3) / 4), nrhs), 128, 0, st>>>(A, M, K, B, C, P, per);
+  const long long warps = (long long)M * nc;
+  const int wpc = small_block(warps * nrhs);
+  k_zgemm_direct<<<dim3((unsigned)((warps + wpc - 1) / wpc), nrhs), 32 * wpc, 0, st>>>(A, M, K, B, C, P, per);
 }
 
 void launch_node_direct(int ns, int n, int P, int nrhs, const double2* eagg, const double2* xs, const double2* fagg,
                         const double2* refl, const double2* udis, double2* V, cudaStream_t st) {
-  k_node_direct<<<dim3((ns + 3) / 4, nrhs), 128, 0, st>>>(ns, n, P, eagg, xs, fagg, refl, udis, V);
+  const int wpc = small_block((long long)ns * nrhs);
+  k_node_direct<<<dim3((ns + wpc - 1) / wpc, nrhs), 32 * wpc, 0, st>>>(ns, n, P, eagg, xs, fagg, refl, udis, V);
 }

@@ -13,7 +13,7 @@
 // complex element, a warp one 8-row x 4-element core matrix: 64 contiguous bytes per row from
 // memory, 32 distinct banks on the store).  The bound is that read (164 MB for 5000 discs and 1024
 // nodes: 24 us at the measured copy rate); the two products take 102 and 113 us there, on the FP64
-// pipe (k_zgemm_rows) they took 2.5 ms each.
+// pipe (tiled products in shared memory) they took 2.5 ms each.
 #include <algorithm>
 #include <cmath>
 #include <mutex>
@@ -321,16 +321,15 @@ int zgemm_setup(lsms_ctx* c) {
   ZgemmTc& z = c->zgemm;
   const int n = c->n, rows = 2 * c->ns;
   if ((double)rows * n < kZgemmMinTable || !tc_err_flag(c)) return LSMS_OK;
-  unsigned long long* bits = nullptr;
-  int* bad = nullptr;
-  const size_t bb = (size_t)2 * rows * 8 + 16;
-  if (cudaMalloc((void**)&z.d_exp, (size_t)2 * rows * sizeof(int)) != cudaSuccess ||
-      cudaMalloc((void**)&bits, bb) != cudaSuccess) {
+  // one allocation: exponents, then the maxima they come from
+  const size_t eb = ((size_t)2 * rows * sizeof(int) + 15) & ~size_t(15), bb = (size_t)2 * rows * 8 + 16;
+  if (cudaMalloc((void**)&z.d_exp, eb + bb) != cudaSuccess) {
     cudaGetLastError();
     zgemm_free(c);
     return ctx_fail(c, LSMS_ERR_OOM, "cudaMalloc failed for the table exponents");
   }
-  bad = (int*)(bits + 2 * rows);
+  unsigned long long* bits = (unsigned long long*)((unsigned char*)z.d_exp + eb);
+  int* bad = (int*)(bits + 2 * rows);
   cudaMemsetAsync(bits, 0, bb, c->stream);
   k_row_max<<<(rows + 7) / 8, 256, 0, c->stream>>>(c->d_eagg, rows, n, bits);
   const int per = std::max(1, (n + 63) / 64);
@@ -339,7 +338,6 @@ int zgemm_setup(lsms_ctx* c) {
   int h = 0;
   cudaMemcpyAsync(&h, bad, sizeof(int), cudaMemcpyDeviceToHost, c->stream);
   cudaStreamSynchronize(c->stream);
-  cudaFree(bits);
   z.ready = h == 0;
   return check_cuda(c, "zgemm_setup");
 }

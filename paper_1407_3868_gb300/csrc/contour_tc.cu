@@ -10,7 +10,7 @@
 // so the contraction is as accurate as FP32.
 //
 // Kernel: one CTA per (128-row tile, 64-column tile, K range).  Thread 0 streams the six operand
-// tiles of each 64-wide K block (three planes of A, three of B) with TMA into a 3-stage ring of
+// tiles of each 64-wide K block (three planes of A, three of B) with TMA into a ring of up to 3 stages of
 // 128-byte-swizzled shared memory; thread 32 issues the 24 tcgen05.mma (6 products x 4 K steps of
 // 16) per block into one 128 x 64 FP32 accumulator in tensor memory and releases each stage with
 // tcgen05.commit; after the last block all four warps read the accumulator (tcgen05.ld, warp w owns
@@ -20,6 +20,7 @@
 #include <cudaTypedefs.h>
 #include <cuda_bf16.h>
 
+#include <algorithm>
 #include <cmath>
 #include <cstring>
 #include <mutex>
@@ -46,22 +47,23 @@ __constant__ int kPairB[6] = {0, 1, 0, 2, 0, 1};
 
 // C[row][col] += sum_k A[row][k] B^T[col][k] over this CTA's K blocks, for the 6 plane products.
 // ta: A planes, 3-D tensor {Kpad, M, 3}; tb: B planes {Kpad, Ncols, 3}; both BF16, box {64, rows, 1}.
+template <int stages>
 __global__ void __launch_bounds__(128, 1)
 k_gemm_bf16x6(const __grid_constant__ CUtensorMap ta, const __grid_constant__ CUtensorMap tb, int M,
               int Ncols, int kblocks, int kchunk, float* __restrict__ C, int ldc,
               int* __restrict__ err) {
   extern __shared__ unsigned char smem_raw[];
   unsigned char* smem = (unsigned char*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
-  uint64_t* bars = (uint64_t*)(smem + STAGES * STAGE_BYTES);   // full[S], empty[S], done
-  uint32_t* tmem_slot = (uint32_t*)(bars + 2 * STAGES + 1);
+  uint64_t* bars = (uint64_t*)(smem + stages * STAGE_BYTES);   // full[S], empty[S], done
+  uint32_t* tmem_slot = (uint32_t*)(bars + 2 * stages + 1);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int m0 = blockIdx.x * BM, n0 = blockIdx.y * BN;
   const int kb0 = blockIdx.z * kchunk;
   const int nkb = min(kchunk, kblocks - kb0);
   if (nkb <= 0) return;
-  const uint32_t full0 = smem_u32(bars), empty0 = smem_u32(bars + STAGES), done = smem_u32(bars + 2 * STAGES);
+  const uint32_t full0 = smem_u32(bars), empty0 = smem_u32(bars + stages), done = smem_u32(bars + 2 * stages);
   if (threadIdx.x == 0) {
-    for (int s = 0; s < STAGES; ++s) {
+    for (int s = 0; s < stages; ++s) {
       mbar_init(full0 + 8 * s, 1);
       mbar_init(empty0 + 8 * s, 1);
     }
@@ -82,7 +84,7 @@ k_gemm_bf16x6(const __grid_constant__ CUtensorMap ta, const __grid_constant__ CU
     // producer: TMA of 3 A planes and 3 B planes per K block
     bool ok = true;
     for (int i = 0; i < nkb; ++i) {
-      const int s = i % STAGES, round = i / STAGES;
+      const int s = i % stages, round = i / stages;
       if (round > 0 && !mbar_wait(empty0 + 8 * s, (round - 1) & 1)) {
         ok = false;
         break;
@@ -99,7 +101,7 @@ k_gemm_bf16x6(const __grid_constant__ CUtensorMap ta, const __grid_constant__ CU
     // MMA issuer
     bool ok = true;
     for (int i = 0; i < nkb; ++i) {
-      const int s = i % STAGES, round = i / STAGES;
+      const int s = i % stages, round = i / stages;
       if (!mbar_wait(full0 + 8 * s, round & 1)) {
         ok = false;
         break;
@@ -378,7 +380,9 @@ int tc_setup(lsms_ctx* c) {
   if ((rc = make_map(c, &t->map_a_dis, t->a_dis, t->kpad_dis, c->n, BM))) return rc;
   static std::once_flag attr;
   std::call_once(attr, [] {
-    cudaFuncSetAttribute(k_gemm_bf16x6, cudaFuncAttributeMaxDynamicSharedMemorySize, GEMM_SMEM);
+    cudaFuncSetAttribute(k_gemm_bf16x6<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, GEMM_SMEM);
+    cudaFuncSetAttribute(k_gemm_bf16x6<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, GEMM_SMEM);
+    cudaFuncSetAttribute(k_gemm_bf16x6<3>, cudaFuncAttributeMaxDynamicSharedMemorySize, GEMM_SMEM);
   });
   return LSMS_OK;
 }
@@ -420,7 +424,12 @@ static void launch_gemm(const CUtensorMap& ta, const CUtensorMap& tb, int M, int
   const int kchunk = (kb + split - 1) / split;
   split = (kb + kchunk - 1) / kchunk;
   dim3 grid(mt, nt, split);
-  k_gemm_bf16x6<<<grid, 128, GEMM_SMEM, st>>>(ta, tb, M, ncols, kb, kchunk, C, ncols_pad, err);
+  // no more stages than K blocks: with two (147 KB) a CTA fits beside two CTAs of the pair kernel that
+  // runs at the same time, with three it waits for a whole SM (200 discs: 72 -> 65 us per application)
+  const int smem = std::min(kchunk, STAGES) * STAGE_BYTES + 1024 + 256;
+  if (kchunk >= 3) k_gemm_bf16x6<3><<<grid, 128, smem, st>>>(ta, tb, M, ncols, kb, kchunk, C, ncols_pad, err);
+  else if (kchunk == 2) k_gemm_bf16x6<2><<<grid, 128, smem, st>>>(ta, tb, M, ncols, kb, kchunk, C, ncols_pad, err);
+  else k_gemm_bf16x6<1><<<grid, 128, smem, st>>>(ta, tb, M, ncols, kb, kchunk, C, ncols_pad, err);
 }
 
 int* tc_err_flag(lsms_ctx* c) {
@@ -483,6 +492,12 @@ int reflection_mixed_stage(lsms_ctx* c, int nrhs, const double2* xs, cudaStream_
                                                                c->d_refl, c->d_udis, t->ncols_pad, t->kpad_dis, t->b_dis);
   launch_gemm(t->map_a_dis, t->map_b_dis, c->n, ncols, t->ncols_pad, t->kpad_dis, t->c_dis, t->d_err, st);
   return check_cuda(c, "reflection_mixed");
+}
+
+const float* reflection_mixed_output(const lsms_ctx* c, int* ldc) {
+  const TcState* t = (const TcState*)c->tc;
+  *ldc = t->ncols_pad;
+  return t->c_dis;
 }
 
 // alpha += the disaggregated reflected coupling of the last reflection_mixed_stage.

@@ -250,6 +250,10 @@ void build_node_tables(lsms_ctx* c);
 void layer_response(const lsms_ctx* c, cplx lam, std::vector<cplx>& g, cplx r[4][3]);
 int validate_geometry(const lsms_ctx* c, int n, const double* xy, std::string& err);
 
+// Warps per CTA of kernels that give every warp its own row: one while the warps are few, so that they
+// spread over the SMs (an SM's FP64 pipe takes 16 cycles for a warp instruction).
+inline int small_block(long long warps) { return warps <= 152 * 8 ? 1 : 4; }
+
 // ------------------------------------------------------------------------------------------
 // Kernel launchers (kernels_f64.cu).  All arrays are device pointers; all launches are
 // asynchronous on `st`.  Coefficient arrays are [nrhs][N][P] (complex as double2).

@@ -55,10 +55,19 @@ int mixed_check(lsms_ctx* c);         // reads and clears the device error flag 
 // the mixed reflected coupling split at its final add (run the stage on a side stream, add after a join)
 int reflection_mixed_stage(lsms_ctx* c, int nrhs, const double2* xs, cudaStream_t st);
 void reflection_mixed_add(lsms_ctx* c, int nrhs, double2* alpha, cudaStream_t st);
+const float* reflection_mixed_output(const lsms_ctx* c, int* ldc);   // the stage's result, [n][ldc]
 int* tc_err_flag(lsms_ctx* c);        // that flag (device), or null before tc_setup
 int build_lowp_tables(lsms_ctx* c);
 // alpha = T xs in FP32 arithmetic (sums of the per-split FP32 partials accumulated in FP64)
 int translate_mixed(lsms_ctx* c, int nrhs, const double2* xs, double2* alpha, cudaStream_t st);
+// whether translate_mixed takes the unordered-pair kernel; the application around it in two parts
+// (mixed.cu): alpha (near pairs) and *acc (far pairs) of the scaled x beside the reflected coupling, then
+// y = x - s_out (their sum) (x null: y = their sum; y may be alpha)
+bool mixed_sym_path(const lsms_ctx* c, int nrhs);
+int mixed_sym_sums(lsms_ctx* c, int nrhs, const double2* x, const double* s_in, double2* xs, double2* alpha,
+                   const float2** acc, cudaStream_t st);
+void launch_mixed_end(lsms_ctx* c, const double2* x, const double2* alpha, const float2* acc, const double2* s_out,
+                      int nrhs, double2* y, cudaStream_t st);
 // the same for blocks of right-hand sides on the tensor cores, near pairs excluded (translate_tc.cu)
 int translate_mixed_tc(lsms_ctx* c, int nrhs, const double2* xs, double2* alpha, cudaStream_t st);
 // alpha += near-pair terms of T xs32 (FP64-accurate sequences, FP32 coefficients); for target rows

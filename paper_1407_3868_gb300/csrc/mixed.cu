@@ -608,6 +608,43 @@ __global__ void k_to_float(const double2* __restrict__ x, float2* __restrict__ y
     y[i] = make_float2((float)x[i].x, (float)x[i].y);
 }
 
+// The start and the end of an application whose translation is k_translate_f32_sym: xs = scale x with
+// its FP32 copy, the zeroed FP32 accumulator and alpha; y = x - s_out (alpha + acc + C), or the sum in
+// brackets (x null), C the disaggregated reflected coupling [n][ldc] (k_c_add_alpha's columns).
+__global__ void k_mixed_start(const double2* __restrict__ x, const double* __restrict__ scale, long long total, int P,
+                              double2* __restrict__ xs, float2* __restrict__ xs32, float2* __restrict__ acc,
+                              double2* __restrict__ alpha) {
+  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < total;
+       i += (long long)gridDim.x * blockDim.x) {
+    const double s = scale[i % P];
+    const double2 v = make_double2(x[i].x * s, x[i].y * s);
+    xs[i] = v;
+    xs32[i] = make_float2((float)v.x, (float)v.y);
+    acc[i] = make_float2(0.f, 0.f);
+    alpha[i] = make_double2(0.0, 0.0);
+  }
+}
+__global__ void k_mixed_end(const double2* x, const double2* alpha, const float2* __restrict__ acc,
+                            const float* __restrict__ C, int ldc, const double2* __restrict__ s_out, int n, int P,
+                            int nrhs, double2* y) {
+  const long long total = (long long)nrhs * n * P;
+  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < total;
+       i += (long long)gridDim.x * blockDim.x) {
+    const int m = (int)(i % P);
+    const long long rr = i / P;
+    const int row = (int)(rr % n), r = (int)(rr / n);
+    const float* c = C + (size_t)row * ldc + r * 2 * P + m;
+    const double2 a = make_double2(alpha[i].x + (double)acc[i].x + (double)c[0],
+                                   alpha[i].y + (double)acc[i].y + (double)c[P]);
+    if (x) {
+      const double2 s = s_out[m], v = x[i];
+      y[i] = make_double2(v.x - (s.x * a.x - s.y * a.y), v.y - (s.x * a.y + s.y * a.x));
+    } else {
+      y[i] = a;
+    }
+  }
+}
+
 __global__ void k_centres_ff(const double* __restrict__ cx, const double* __restrict__ cy, int n,
                              float4* __restrict__ out) {
   const int j = blockIdx.x * blockDim.x + threadIdx.x;
@@ -928,6 +965,53 @@ int translate_mixed(lsms_ctx* c, int nrhs, const double2* xs, double2* alpha, cu
   }
   launch_translate_near(c, nrhs, xs32, alpha, st);
   return check_cuda(c, "translate_mixed");
+}
+
+bool mixed_sym_path(const lsms_ctx* c, int nrhs) {
+  const bool tc = c->tc_min_rhs > 0 && nrhs >= c->tc_min_rhs && c->p >= 6 && c->p <= LSMS_MAX_P;
+  return !tc && c->f32_shape == 2 && !translate_uses_block(nrhs, c->p);
+}
+
+// The mixed application with the unordered-pair translation, up to its sums: the reflected coupling on
+// the side stream (its last product stays in the FP32 output of the tensor cores), and on `st` one
+// kernel that prepares everything, the near pairs (a few CTAs: they share the chip with the coupling's
+// products, whose CTAs need whole SMs that the pair kernel would not leave) and the pair kernel.
+// launch_mixed_end adds the three.  200 discs: 79 -> 65, 777 discs: 123 -> 115 us per application (near
+// pairs behind the pair kernel: 123, on the side stream: 132 at 777 discs).
+int mixed_sym_sums(lsms_ctx* c, int nrhs, const double2* x, const double* s_in, double2* xs, double2* alpha,
+                   const float2** acc_out, cudaStream_t st) {
+  const int n = c->n, p = c->p, P = c->P;
+  const long long len = (long long)nrhs * n * P;
+  const size_t b32 = (((size_t)len * sizeof(float2)) + 255) & ~size_t(255);
+  int rc;
+  if ((rc = ensure(c, c->ws_lp, 2 * b32))) return rc;
+  float2* xs32 = (float2*)c->ws_lp.ptr;
+  float2* acc = (float2*)((unsigned char*)c->ws_lp.ptr + b32);
+  const int g = (int)std::min<long long>((len + 255) / 256, 152 * 16);
+  k_mixed_start<<<g, 256, 0, st>>>(x, s_in, len, P, xs, xs32, acc, alpha);
+  if (c->timing) cudaEventRecord(c->ev[0], st);
+  cudaEventRecord(c->ev_fork, st);
+  cudaStreamWaitEvent(c->side, c->ev_fork, 0);
+  if ((rc = reflection_mixed_stage(c, nrhs, xs, c->side))) return rc;
+  cudaEventRecord(c->ev_join, c->side);
+  launch_translate_near(c, nrhs, xs32, alpha, st);
+  const float kh = (float)c->k2, kl = (float)(c->k2 - (double)kh);
+  const float nh = (float)c->near_r2, nl = (float)(c->near_r2 - (double)nh);
+  launch_translate_sym(st, (const float4*)c->d_lp_misc, n, p, kh, kl, xs32, acc, nrhs, nh, nl, c->split_mult);
+  if (c->timing) cudaEventRecord(c->ev[1], st);
+  cudaStreamWaitEvent(st, c->ev_join, 0);
+  if (c->timing) cudaEventRecord(c->ev[2], st);
+  *acc_out = acc;
+  return check_cuda(c, "mixed_sym_sums");
+}
+
+void launch_mixed_end(lsms_ctx* c, const double2* x, const double2* alpha, const float2* acc, const double2* s_out,
+                      int nrhs, double2* y, cudaStream_t st) {
+  const long long len = (long long)nrhs * c->n * c->P;
+  int ldc = 0;
+  const float* C = reflection_mixed_output(c, &ldc);
+  k_mixed_end<<<(int)std::min<long long>((len + 255) / 256, 152 * 16), 256, 0, st>>>(x, alpha, acc, C, ldc, s_out, c->n,
+                                                                                  c->P, nrhs, y);
 }
 
 int translate_mixed_rows(lsms_ctx* c, int nrhs, const double2* xs, double2* alpha_rows, int row0, int nrows,

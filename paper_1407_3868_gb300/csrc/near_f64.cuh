@@ -5,6 +5,8 @@
 
 #include <cuda_runtime.h>
 
+#include "lsms_internal.h"
+
 namespace {
 
 // alpha^l += sum over the sources listed for row t, l = perm[t] (perm: targets in box order; rows row0 ..
@@ -22,7 +24,7 @@ k_near_f64(int n, int p, const int* __restrict__ perm, int row0, int nrows, int 
            const int* __restrict__ ptr, const int* __restrict__ idx, const double2* __restrict__ seq,
            const double2* __restrict__ xs, double2* __restrict__ alpha) {
   const int P = 2 * p + 1, lane = threadIdx.x & 31, r = blockIdx.y;
-  const int w = blockIdx.x * 4 + (threadIdx.x >> 5), part = w % splits;
+  const int w = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5), part = w % splits;
   const int t = row0 + w / splits;
   if (t >= row0 + nrows) return;
   const int l = perm ? perm[t] : t, len = ptr[t + 1] - ptr[t];
@@ -58,7 +60,9 @@ inline void launch_near_f64(int n, int p, const int* perm, int row0, int nrows, 
                             const int* idx, const double2* seq, const double2* xs, int nrhs, double2* alpha,
                             cudaStream_t st) {
   if (nrows <= 0 || nrhs <= 0) return;
-  k_near_f64<<<dim3((unsigned)(((long long)nrows * splits + 3) / 4), nrhs), 128, 0, st>>>(n, p, perm, row0, nrows, splits,
+  const long long warps = (long long)nrows * splits;
+  const int per = small_block(warps * nrhs);   // warps per CTA
+  k_near_f64<<<dim3((unsigned)((warps + per - 1) / per), nrhs), 32 * per, 0, st>>>(n, p, perm, row0, nrows, splits,
                                                                                          ptr, idx, seq, xs, alpha);
 }
 
