@@ -326,7 +326,7 @@ int zgemm_setup(lsms_ctx* c) {
   if (cudaMalloc((void**)&z.d_exp, eb + bb) != cudaSuccess) {
     cudaGetLastError();
     zgemm_free(c);
-    return ctx_fail(c, LSMS_ERR_OOM, "cudaMalloc failed for the table exponents");
+    return LSMS_OK;                                // the FP64 pipe then (launch_zgemm_direct)
   }
   unsigned long long* bits = (unsigned long long*)((unsigned char*)z.d_exp + eb);
   int* bad = (int*)(bits + 2 * rows);
@@ -356,8 +356,11 @@ int zgemm_f64(lsms_ctx* c, bool agg, int nrhs, const double2* B, double2* C, cud
   const size_t sb = (size_t)KG * b_kg_bytes(npad);
   const int rb = (int)std::max<size_t>(1, std::min<size_t>(nrhs, kImageBytes / (max_stages * sb)));
   const size_t mbytes = ((size_t)nrhs * 32 * 8 + 255) & ~size_t(255);
-  int rc;
-  if ((rc = ensure(c, z.ws, mbytes + (size_t)rb * max_stages * sb))) return rc;
+  if (ensure(c, z.ws, mbytes + (size_t)rb * max_stages * sb)) {   // no memory for the image
+    c->err.clear();
+    launch_zgemm_direct(A, M, K, B, C, P, nrhs, st);
+    return check_cuda(c, "zgemm_f64");
+  }
   unsigned long long* maxbits = (unsigned long long*)z.ws.ptr;
   unsigned char* img = (unsigned char*)z.ws.ptr + mbytes;
   const int* kexp = agg ? nullptr : z.d_exp + 2 * c->ns;

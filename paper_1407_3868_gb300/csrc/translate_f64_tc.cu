@@ -406,6 +406,7 @@ void launch_digits(dim3 grid, cudaStream_t st, const lsms_ctx* c, const PairCons
 constexpr size_t kImageBytes = (size_t)256 << 20;   // digits of X held at once
 constexpr int kMinDiscs = 96;
 constexpr double kStoreBytes = 64e6;
+constexpr double kNearBytes = 8e9;                  // near sequences beside the digits
 
 }  // namespace
 
@@ -421,14 +422,17 @@ void f64tc_free(lsms_ctx* c) {
 // distance (host arrays).  Layouts of fewer than kMinDiscs discs (not one full tile of rows) or of
 // mostly near pairs (summed on the FP64 pipe either way) store the sequences of all their pairs if
 // these take at most kStoreBytes (16 discs: 75 us with the sequences formed anew -> 11 us);
-// larger ones keep k_translate_f64 and its symmetric form.
+// larger ones, and layouts for whose tables there is no memory, keep k_translate_f64 and its symmetric
+// form.
 int f64tc_setup(lsms_ctx* c, const std::vector<int>& ptr, const std::vector<int>& idx) {
   f64tc_free(c);
   F64Tc& f = c->f64tc;
   const int n = c->n;
   if (n <= 0 || !tc_err_flag(c)) return LSMS_OK;
-  const bool digits = n >= kMinDiscs && (double)idx.size() <= 0.5 * n * (double)(n - 1);
-  const bool store = !digits && (double)n * (n - 1) * (4 * c->p + 1) * sizeof(double2) <= kStoreBytes;
+  const double seq_bytes = (4 * c->p + 1) * (double)sizeof(double2);
+  const bool digits = n >= kMinDiscs && (double)idx.size() <= 0.5 * n * (double)(n - 1) &&
+                      (double)idx.size() * seq_bytes <= kNearBytes;
+  const bool store = !digits && (double)n * (n - 1) * seq_bytes <= kStoreBytes;
   if (!digits && !store) return LSMS_OK;
   std::vector<int> all_ptr, all_idx;
   if (store) {
@@ -454,7 +458,7 @@ int f64tc_setup(lsms_ctx* c, const std::vector<int>& ptr, const std::vector<int>
   if (cudaMalloc(&f.d_table, bytes) != cudaSuccess) {
     cudaGetLastError();
     f64tc_free(c);
-    return ctx_fail(c, LSMS_ERR_OOM, "cudaMalloc failed for the near pairs of the FP64 translation");
+    return LSMS_OK;
   }
   f.d_ptr = (int*)((unsigned char*)f.d_table + TABLE_BYTES);
   f.d_idx = f.d_ptr + n + 1;
@@ -485,8 +489,8 @@ int f64tc_sequences(lsms_ctx* c) {
   }
   if (cudaMalloc(&f.d_seq, (size_t)f.nnz * (4 * c->p + 1) * sizeof(double2)) != cudaSuccess) {
     cudaGetLastError();
-    f.d_seq = nullptr;
-    return ctx_fail(c, LSMS_ERR_OOM, "cudaMalloc failed for the near sequences of the FP64 translation");
+    f64tc_free(c);
+    return LSMS_OK;
   }
   k_near_sequences<<<(f.nnz + 127) / 128, 128, 0, c->stream>>>(c->d_cx, c->d_cy, f.d_idx + f.nnz, f.d_idx, f.nnz,
                                                                 c->p, c->k2,
@@ -518,9 +522,12 @@ int translate_f64_tc(lsms_ctx* c, int nrhs, const double2* xs, double2* alpha, c
   runs = (n + run - 1) / run;
   const size_t img_bytes = (size_t)rb * std::min(run, n) * src_bytes;
   const size_t max_bytes = ((size_t)nrhs * 8 + 255) & ~size_t(255);
-  int rc;
   const size_t bound_bytes = ((size_t)rb * std::min(run, n) * sizeof(int) + 255) & ~size_t(255);
-  if ((rc = ensure(c, f.ws, max_bytes + bound_bytes + img_bytes))) return rc;
+  if (ensure(c, f.ws, max_bytes + bound_bytes + img_bytes)) {   // no memory for the image: the FP64 pipe
+    c->err.clear();
+    launch_translate_f64(c->d_cx, c->d_cy, n, p, c->k2, xs, alpha, nrhs, st, row0, nrows);
+    return check_cuda(c, "translate_f64");
+  }
   unsigned long long* maxbits = (unsigned long long*)f.ws.ptr;
   int* bound = (int*)((unsigned char*)f.ws.ptr + max_bytes);
   unsigned char* img = (unsigned char*)f.ws.ptr + max_bytes + bound_bytes;
