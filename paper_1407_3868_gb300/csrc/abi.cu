@@ -75,7 +75,7 @@ int need_particles(lsms_ctx* c) {
 int translate_f64(lsms_ctx* c, int nrhs, const double2* xs, double2* alpha, cudaStream_t st, int row0, int nrows) {
   if (nrows < 0) nrows = c->n - row0;
   if (c->n == 0 || nrhs == 0 || nrows <= 0) return LSMS_OK;
-  if (c->f64tc.ready) return translate_f64_tc(c, nrhs, xs, alpha, st, row0, nrows);
+  if (f64tc_usable(c)) return translate_f64_tc(c, nrhs, xs, alpha, st, row0, nrows);
   launch_translate_f64(c->d_cx, c->d_cy, c->n, c->p, c->k2, xs, alpha, nrhs, st, row0, nrows);
   return LSMS_OK;
 }
@@ -439,6 +439,7 @@ extern "C" int lsms_set_particles(lsms_ctx* c, int n, const double* xy) {
   std::vector<double> xs(n);
   for (int j = 0; j < n; ++j) xs[j] = c->cx[j] - c->xc;
   tc_free(c);
+  fmm_free(c);                               // the previous layout's, also where this call fails below
   f64tc_free(c);
   zgemm_free(c);
   void* old[] = {c->d_cx, c->d_cy, c->d_eagg, c->d_edis, c->d_eagg_lp, c->d_edis_lp, c->d_lp_misc};
@@ -467,12 +468,7 @@ extern "C" int lsms_set_particles(lsms_ctx* c, int n, const double* xy) {
     if ((rc = check_cuda(c, "set_particles"))) return rc;
     if ((rc = build_lowp_tables(c))) return rc;
   }
-  if (c->fmm.box_width > 0.0) {
-    if ((rc = fmm_setup(c))) return rc;
-  } else {
-    fmm_free(c);
-  }
-  return f64tc_sequences(c);
+  return fmm_update(c);
 }
 
 // ---------------------------------------------------------------------------------------------

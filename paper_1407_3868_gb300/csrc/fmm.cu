@@ -878,6 +878,16 @@ int fmm_setup(lsms_ctx* c) {
   return check_cuda(c, "set_fmm");
 }
 
+// Box tables for the current layout and width (none at width 0), then the FP64 near sequences of the
+// translation over all pairs, which every translation uses again when the boxes are refused.
+int fmm_update(lsms_ctx* c) {
+  const int rc = fmm_setup(c);
+  const std::string msg = c->err;
+  const int rs = f64tc_sequences(c);
+  if (rc) c->err = msg;
+  return rc ? rc : rs;
+}
+
 // alpha = T xs for nrhs right-hand sides through the box method.  Launches: per right-hand side
 // M2M, five transform passes, the direct offsets and L2L, plus the near-field launches.
 int fmm_translate(lsms_ctx* c, int nrhs, const double2* xs, double2* alpha, bool mixed, cudaStream_t st) {
@@ -948,11 +958,7 @@ extern "C" int lsms_set_fmm(lsms_ctx* c, double box_width, int order) {
     const int rc = lsms_set_fmm(k, box_width, order);
     if (rc) return ctx_fail(c, rc, std::string("set_fmm: ") + k->err);
   }
-  if (c->kids.empty() && c->n >= 0) {
-    const int rc = fmm_setup(c);
-    return rc ? rc : f64tc_sequences(c);
-  }
-  return LSMS_OK;
+  return c->kids.empty() && c->n >= 0 ? fmm_update(c) : LSMS_OK;
 }
 
 extern "C" int lsms_set_fmm_scope(lsms_ctx* c, int scope) {

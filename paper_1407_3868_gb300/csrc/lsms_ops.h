@@ -16,6 +16,7 @@ int ensure(lsms_ctx* c, DevBuf& b, size_t bytes);
 bool solve_small(std::vector<cplx>& a, int n, std::vector<cplx>& b, int nrhs);
 // box-compressed translation (fmm.cu)
 int fmm_setup(lsms_ctx* c);
+int fmm_update(lsms_ctx* c);           // after a change of the layout or of the boxes
 void fmm_free(lsms_ctx* c);
 // mixed: the near field in FP32 (adjacent boxes) plus the FP32 near-pair kernel; else all FP64
 int fmm_translate(lsms_ctx* c, int nrhs, const double2* xs, double2* alpha, bool mixed, cudaStream_t st);
@@ -24,6 +25,7 @@ int fmm_translate(lsms_ctx* c, int nrhs, const double2* xs, double2* alpha, bool
 int f64tc_setup(lsms_ctx* c, const std::vector<int>& ptr, const std::vector<int>& idx);
 void f64tc_free(lsms_ctx* c);
 int f64tc_sequences(lsms_ctx* c);     // after a change of the layout or of the box translation
+bool f64tc_usable(const lsms_ctx* c);  // the tables are there, the listed pairs' sequences among them
 int translate_f64_tc(lsms_ctx* c, int nrhs, const double2* xs, double2* alpha, cudaStream_t st, int row0, int nrows);
 // rows row0 .. row0 + nrows - 1 (nrows < 0: to the last disc) of alpha = T xs in FP64, by whichever
 // path the layout takes

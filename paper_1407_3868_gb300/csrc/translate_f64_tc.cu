@@ -500,6 +500,8 @@ int f64tc_sequences(lsms_ctx* c) {
   return check_cuda(c, "f64tc_sequences");
 }
 
+bool f64tc_usable(const lsms_ctx* c) { return c->f64tc.ready && (c->f64tc.nnz == 0 || c->f64tc.d_seq); }
+
 // alpha = rows row0 .. row0 + nrows - 1 of T xs, [nrhs][nrows][P].
 int translate_f64_tc(lsms_ctx* c, int nrhs, const double2* xs, double2* alpha, cudaStream_t st, int row0, int nrows) {
   F64Tc& f = c->f64tc;
