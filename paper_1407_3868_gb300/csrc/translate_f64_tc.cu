@@ -205,7 +205,7 @@ k_translate_digits(const double* __restrict__ cx, const double* __restrict__ cy,
   const uint32_t sbase = smem_u32(smem);
 
   if (warp < GEN_WARPS) {
-    // ---- digits of W: warpgroup g takes every third source, thread = target row
+    // ---- digits of W: warpgroup g takes every second source (GROUPS = 2), thread = target row
     const int g = warp >> 2, row = threadIdx.x & (ROWS - 1);
     const int l = row0 + blockIdx.x * ROWS + row;
     const bool lvalid = l < row0 + nrows;
@@ -226,7 +226,8 @@ k_translate_digits(const double* __restrict__ cx, const double* __restrict__ cy,
       for (int c = 0; c < chunks; ++c) {
         const int t = (q * chunks + c) * GROUPS + g;
         const int st = t % STAGES, lap = t / STAGES;
-        if (lap > 0 && !mbar_wait(empty0 + 8 * st, (lap - 1) & 1)) {
+        // all lanes give up together: the others would wait for this one at the warp's barrier below
+        if (lap > 0 && !__all_sync(0xffffffffu, mbar_wait(empty0 + 8 * st, (lap - 1) & 1))) {
           ok = false;
           break;
         }
