@@ -574,7 +574,7 @@ extern "C" int lsms_aggregate(lsms_ctx* c, int nrhs, const double* beta, double*
   if ((rc = check_cuda(c, "aggregate"))) return rc;
   std::vector<cplx> pq((size_t)nrhs * 2 * ns);
   if ((rc = copy_out(c, (double*)pq.data(), c->ws_pq.ptr, pq.size()))) return rc;
-  if (precision == LSMS_MIXED && (rc = mixed_check(c))) return rc;
+  if ((rc = mixed_check(c))) return rc;
   // the device works in x - xc; densities in absolute x carry exp(-i lambda xc)
   const std::vector<cplx> ph = shift_phase(c, -1.0);
   cplx* pp = reinterpret_cast<cplx*>(p_plus);
@@ -645,7 +645,7 @@ extern "C" int lsms_disaggregate(lsms_ctx* c, int nrhs, const double* s_plus, co
   }
   if ((rc = check_cuda(c, "disaggregate"))) return rc;
   if ((rc = copy_out(c, alpha, c->ws_alpha.ptr, len))) return rc;
-  return precision == LSMS_MIXED ? mixed_check(c) : LSMS_OK;
+  return mixed_check(c);
 }
 
 // a_inc of line sources on the device: [nsrc][N][P] into `out`.
@@ -680,7 +680,8 @@ extern "C" int lsms_incident(lsms_ctx* c, int nsrc, const double* src_xy, double
   cudaMemcpyAsync(c->ws_aux.ptr, src_xy, (size_t)nsrc * 2 * sizeof(double), cudaMemcpyHostToDevice, c->stream);
   if ((rc = ensure(c, c->ws_alpha, len * sizeof(double2)))) return rc;
   if ((rc = incident_device(c, nsrc, (const double*)c->ws_aux.ptr, (double2*)c->ws_alpha.ptr, c->stream))) return rc;
-  return copy_out(c, a_inc, c->ws_alpha.ptr, len);
+  if ((rc = copy_out(c, a_inc, c->ws_alpha.ptr, len))) return rc;
+  return mixed_check(c);
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -720,7 +721,8 @@ extern "C" int lsms_eval_field(lsms_ctx* c, int src_index, int ntgt, const doubl
   launch_field(ns, ntgt, d_tgt, c->xc, c->d_lam, c->d_g1, c->d_field, pq, d_src, c->k1, which, d_out,
                c->stream);
   if ((rc = check_cuda(c, "eval_field"))) return rc;
-  return copy_out(c, out, d_out, ntgt);
+  if ((rc = copy_out(c, out, d_out, ntgt))) return rc;
+  return mixed_check(c);
 }
 
 // ---------------------------------------------------------------------------------------------

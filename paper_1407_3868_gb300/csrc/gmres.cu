@@ -1081,6 +1081,8 @@ extern "C" int lsms_solve(lsms_ctx* c, int nsrc, const double* src_xy, double to
   if (status != LSMS_OK && status != LSMS_ERR_NOT_CONVERGED) return status;
   launch_diag_scale(xs, c->d_scale_in + c->P, beta, LT, c->P, st);   // beta = D^{-1} b
   if ((rc = check_cuda(c, "solve"))) return rc;
+  cudaStreamSynchronize(st);
+  if ((rc = mixed_check(c))) return rc;                  // the last residual's products
   if (info) {
     int mi = 0;
     double mr = 0.0, m64 = 0.0;

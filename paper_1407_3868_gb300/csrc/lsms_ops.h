@@ -53,7 +53,9 @@ int incident_device(lsms_ctx* c, int nsrc, const double* d_src, double2* out, cu
 // mixed-precision contour contractions on the tensor cores (contour_tc.cu)
 int tc_setup(lsms_ctx* c);            // BF16 planes of the layout's tables (after set_particles)
 void tc_free(lsms_ctx* c);
-int mixed_check(lsms_ctx* c);         // reads and clears the device error flag of the TC kernels
+// reads and clears the device error flag (a wait of a tensor-core kernel ran out, FP64 or mixed): the last
+// step of every call that waits for its kernels
+int mixed_check(lsms_ctx* c);
 // the mixed reflected coupling split at its final add (run the stage on a side stream, add after a join)
 int reflection_mixed_stage(lsms_ctx* c, int nrhs, const double2* xs, cudaStream_t st);
 void reflection_mixed_add(lsms_ctx* c, int nrhs, double2* alpha, cudaStream_t st);
