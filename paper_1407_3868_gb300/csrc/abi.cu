@@ -567,7 +567,8 @@ extern "C" int lsms_aggregate(lsms_ctx* c, int nrhs, const double* beta, double*
   if (precision == LSMS_MIXED) {
     if ((rc = aggregate_mixed(c, nrhs, (const double2*)c->ws_x.ptr, G, c->stream))) return rc;
   } else {
-    if ((rc = zgemm_f64(c, true, nrhs, (const double2*)c->ws_x.ptr, G, c->stream))) return rc;
+    // the caller sees single nodes: sums that keep each of them to its own size (contour_f64_tc.cu)
+    launch_zgemm_direct(c->d_eagg, 2 * ns, c->n, (const double2*)c->ws_x.ptr, G, P, nrhs, c->stream);
   }
   launch_node_stage(ns, P, nrhs, G, c->d_fagg, nullptr, nullptr, nullptr, (double2*)c->ws_pq.ptr,
                     nullptr, nullptr, c->stream);
@@ -640,8 +641,8 @@ extern "C" int lsms_disaggregate(lsms_ctx* c, int nrhs, const double* s_plus, co
   cudaMemsetAsync(c->ws_alpha.ptr, 0, len * sizeof(double2), c->stream);
   if (precision == LSMS_MIXED) {
     if ((rc = disaggregate_mixed(c, nrhs, (const double2*)c->ws_v.ptr, (double2*)c->ws_alpha.ptr, c->stream))) return rc;
-  } else {
-    if ((rc = zgemm_f64(c, false, nrhs, (const double2*)c->ws_v.ptr, (double2*)c->ws_alpha.ptr, c->stream))) return rc;
+  } else {                                   // densities of any shape over the nodes: as in lsms_aggregate
+    launch_zgemm_direct(c->d_edis, c->n, 2 * ns, (const double2*)c->ws_v.ptr, (double2*)c->ws_alpha.ptr, P, nrhs, c->stream);
   }
   if ((rc = check_cuda(c, "disaggregate"))) return rc;
   if ((rc = copy_out(c, alpha, c->ws_alpha.ptr, len))) return rc;

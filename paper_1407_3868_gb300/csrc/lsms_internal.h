@@ -95,7 +95,13 @@ struct F64Tc {
 // FP64 contour contractions on the tensor cores (contour_f64_tc.cu).
 struct ZgemmTc {
   bool ready = false;
-  int* d_exp = nullptr;             // [2ns] row exponents of E_agg, [2ns] column exponents of E_dis
+  int classes = 0;                  // of discs, by depth
+  int stages = 0, tiles = 0;        // K stages of the aggregate, row tiles of the disaggregate
+  int* d_exp = nullptr;             // [classes][2ns] exponents of E_agg's rows, the same of E_dis's columns
+  int* d_kidx = nullptr;            // the discs class by class, padded with -1 to whole stages; behind d_exp, as
+  int* d_start = nullptr;           // [classes + 1] where each begins
+  unsigned char* d_scls = nullptr;  // class of every stage
+  void* d_tiles = nullptr;          // int4 (class, first position, rows, 0)
   DevBuf ws;                        // scales and digit images of the right operand
 };
 

@@ -42,6 +42,10 @@
 
 namespace {
 
+using Tile = DigitTile<6, 4>;
+constexpr int PL = Tile::PL, KG = Tile::KG, A_PLANE = Tile::A_PLANE, A_BYTES = Tile::A_BYTES, STAGES = 3;
+__host__ __device__ constexpr int b_kg_bytes(int npad) { return Tile::b_kg_bytes(npad); }
+__host__ __device__ constexpr int stage_bytes(int npad) { return Tile::stage_bytes(npad); }
 constexpr int TABLE_BYTES = 256 * 16;
 constexpr int kExact = 1 << 24;                // FP32 sums of integers are exact up to here
 constexpr int MAX_SOURCES = 1024;             // per CTA: the 64-bit sums keep 10 bits for them
@@ -51,6 +55,38 @@ constexpr int MMA_WARP = GEN_WARPS + DRAIN_WARPS;
 constexpr int THREADS = (MMA_WARP + 2) * 32;
 constexpr size_t smem_bytes(int npad) {
   return (size_t)STAGES * stage_bytes(npad) + TABLE_BYTES + MAX_SOURCES / GROUPS * sizeof(int) + 256;
+}
+
+// Levels of one accumulated element -> units of level 5 / 64, added to acc.
+template <int LMAX>
+__device__ __forceinline__ void add_levels(int64_t& acc, const uint32_t* f) {
+  int lo = __float2int_rn(__uint_as_float(f[5]));
+  if (LMAX >= 6) lo += (__float2int_rn(__uint_as_float(f[6])) + 128) >> 8;
+  acc = mad_wide((lo + 32) >> 6, 1, acc);
+  acc = mad_wide(__float2int_rn(__uint_as_float(f[4])), 1 << 2, acc);
+  acc = mad_wide(__float2int_rn(__uint_as_float(f[3])), 1 << 10, acc);
+  acc = mad_wide(__float2int_rn(__uint_as_float(f[2])), 1 << 18, acc);
+  acc = mad_wide(__float2int_rn(__uint_as_float(f[1])), 1 << 26, acc);
+  acc = mad_wide(__float2int_rn(__uint_as_float(f[0])) * 16, 1 << 30, acc);
+}
+
+// Add the accumulators of this warp's 32 rows and NPAD / 2 columns (tb: its tensor-memory address) to
+// acc, in units of 2^46 = 64 of level 5.
+template <int NPAD, int LMAX>
+__device__ __forceinline__ void drain_levels(uint32_t tb, int64_t* acc) {
+  constexpr int NL = LMAX + 1;
+#pragma unroll
+  for (int cb = 0; cb < NPAD / 8; ++cb) {
+    uint32_t f[NL][4];
+    load_levels<NPAD, LMAX>(tb + 4 * cb, f);
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      uint32_t e[NL];
+#pragma unroll
+      for (int L = 0; L < NL; ++L) e[L] = f[L][i];
+      add_levels<LMAX>(acc[4 * cb + i], e);
+    }
+  }
 }
 
 inline int k_steps(int p) { return (4 * (2 * p + 1) + 15) / 16; }   // K = 16 steps of one source
@@ -116,8 +152,8 @@ k_pack_digits(const double2* __restrict__ xs, int n, int p, int src0, int r0, in
         if (s & 2) { a = -a; bb = -bb; cc = -cc; d = -d; }   // the sequence's signs + + - -
       }
       uint32_t u[PL], v[PL];
-      digit_pairs(a << 16, bb << 16, u);
-      digit_pairs(cc << 16, d << 16, v);
+      digit_pairs<PL>(a << 16, bb << 16, u);
+      digit_pairs<PL>(cc << 16, d << 16, v);
 #pragma unroll
       for (int j = 0; j < PL; ++j) {
         w[j][2 * h] = u[j];
@@ -237,11 +273,11 @@ k_translate_digits(const double* __restrict__ cx, const double* __restrict__ cy,
           uint32_t u[PL], v[PL], w[PL], z[PL];
           if (KG * c + kg <= p) {                  // orders 2 (KG c + kg) and the next
             int64_t pr[8];
-            pair_two_orders(a, step, (int64_t)kDigitBias, pr);
-            biased_digit_pairs(pr[0], pr[1], u);
-            biased_digit_pairs(pr[2], pr[3], v);
-            biased_digit_pairs(pr[4], pr[5], w);
-            biased_digit_pairs(pr[6], pr[7], z);
+            pair_two_orders(a, step, (int64_t)digit_bias<PL>(), pr);
+            biased_digit_pairs<PL>(pr[0], pr[1], u);
+            biased_digit_pairs<PL>(pr[2], pr[3], v);
+            biased_digit_pairs<PL>(pr[4], pr[5], w);
+            biased_digit_pairs<PL>(pr[6], pr[7], z);
           } else {
 #pragma unroll
             for (int j = 0; j < PL; ++j) u[j] = v[j] = w[j] = z[j] = 0;
@@ -319,7 +355,7 @@ k_translate_digits(const double* __restrict__ cx, const double* __restrict__ cy,
           const uint32_t sa = sbase + st * STAGE;
           const int ksteps = min(2, steps - 2 * (c / GROUPS));
           for (int ks = 0; ks < ksteps; ++ks)
-            issue_step<NPAD, LMAX>(tmem, sa, sa + A_BYTES, ks, start && c == 0 && ks == 0);
+            issue_step<Tile, NPAD, LMAX>(tmem, sa, sa + A_BYTES, ks, start && c == 0 && ks == 0);
           mma_commit(empty0 + 8 * st);
         }
       }
