@@ -9,9 +9,11 @@
 // with X_source the signed sums beta_{nu+s} +- beta_{nu-s}.  W and X are held as 48-bit fixed point
 // numbers (W: 48 fractional bits; X: relative to the largest coefficient of the
 // right-hand side) and cut into six signed 8-bit digits each; the digits are exact in FP16, a product
-// of two has at most 14 bits, so the tensor cores' FP32 sums are exact integers.  Products of digits
-// i of W and j of X with i + j = L add into one accumulator per level L; levels beyond LMAX (5 or 6)
-// are below the 48 bits and left out.  One tcgen05.mma multiplies a digit plane of W with several
+// of two has at most 14 bits, so the tensor cores' FP32 sums are exact integers up to 2^24.  Products of
+// digits i of W and j of X with i + j = L add into one accumulator per level L; levels beyond 5 or 6
+// are below the 48 bits and left out (six_levels).  A row is as accurate as an FP64 sum's where the
+// largest coefficient is a term of it, or one of its size is; k_dominant_row sums the only row that can be
+// without.  One tcgen05.mma multiplies a digit plane of W with several
 // digit planes of X side by side in N: its output columns are consecutive levels.
 //
 // Why: this chip's FP64 pipe (2 FMA per SM and clock) bounds the direct form at 133 ms for 5000 discs
@@ -25,7 +27,8 @@
 // the accumulators into 64-bit integers, so a CTA's sum does not depend on any order.  When: before a
 // round (two sources) whose X digits could carry a sum of the levels 0..4 past 2^24, from the bound
 // that the packing kernel left for each source; the decaying coefficients of scattering problems let
-// several rounds pass.  (One round alone stays below it in the levels 0..3 for any digits.)
+// several rounds pass.  (One round alone stays below it in the levels 0..3 for any digits; in level 4
+// only digits near +-128 nearly throughout could pass it, and be rounded to 2^-46 of the scales.)
 // The ring holds three stages of two MMA steps: six stages of one step took 10.0 instead of 9.1 ms
 // (5000 discs, the translation's part of the operator), a third warpgroup brought nothing.
 #include <algorithm>
@@ -91,32 +94,64 @@ __device__ __forceinline__ void drain_levels(uint32_t tb, int64_t* acc) {
 
 inline int k_steps(int p) { return (4 * (2 * p + 1) + 15) / 16; }   // K = 16 steps of one source
 
-// Largest |Re|, |Im| of each right-hand side as the bits of a non-negative double (NaN and Inf
-// compare above every finite value).
-__global__ void k_absmax(const double* __restrict__ x, long long per, unsigned long long* __restrict__ out) {
-  const double* xr = x + blockIdx.y * per;
+// What the digits of a right-hand side rest on: its largest |Re|, |Im| (the bits of a non-negative double;
+// NaN and Inf compare above every finite value), the number of discs with a coefficient of at least
+// 1/16 of it, and one such disc.
+struct RhsStats {
+  unsigned long long maxbits;
+  int count, disc;
+};
+
+// Largest |Re|, |Im| of every disc (a warp each) and of each right-hand side.
+__global__ void __launch_bounds__(256)
+k_disc_max(const double2* __restrict__ x, int n, int P, unsigned long long* __restrict__ dmax,
+           RhsStats* __restrict__ stats) {
+  __shared__ unsigned long long part[8];
+  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31, r = blockIdx.y, l = blockIdx.x * 8 + w;
   unsigned long long m = 0;
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < per; i += (long long)gridDim.x * blockDim.x)
-    m = max(m, (unsigned long long)__double_as_longlong(xr[i]) & 0x7fffffffffffffffull);
+  if (l < n && lane < P) {
+    const double2 v = x[((size_t)r * n + l) * P + lane];
+    m = max((unsigned long long)__double_as_longlong(v.x) & 0x7fffffffffffffffull,
+            (unsigned long long)__double_as_longlong(v.y) & 0x7fffffffffffffffull);
+  }
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
-  if ((threadIdx.x & 31) == 0 && m) atomicMax(out + blockIdx.y, m);
+  if (lane == 0) {
+    part[w] = m;
+    if (l < n) dmax[(size_t)r * n + l] = m;
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    for (int i = 1; i < 8; ++i) m = max(m, part[i]);
+    if (m) atomicMax(&stats[r].maxbits, m);
+  }
 }
+
 // Digits of X for the sources src0 .. src0 + gridDim.x - 1 of right-hand side r0 + blockIdx.y:
 // per source [K group][plane][column][8 K values] FP16, K = 4 s + (A, B, C, D), column 2 q + (Re, Im); and
-// bound[source]: what the source adds to any element of the levels 0..4 at most, 128 sum |X digits|.
+// bound[source]: what the source adds to any element of the levels 0..4 at most, 128 sum |X digits of the
+// planes 0..4|, or a quarter of the same for level 5, whose sums may pass 2^24 up to 2^26 (rounded to 2^-51
+// of the scales).  The first run of sources (src0 = 0) also counts the right-hand side's large discs.
 __global__ void __launch_bounds__(256)
 k_pack_digits(const double2* __restrict__ xs, int n, int p, int src0, int r0, int npad, int kgs,
-              const unsigned long long* __restrict__ maxbits, unsigned char* __restrict__ img,
-              int* __restrict__ bound) {
+              const unsigned long long* __restrict__ dmax, RhsStats* __restrict__ stats,
+              unsigned char* __restrict__ img, int* __restrict__ bound) {
   __shared__ long long re[128], im[128];          // beta_{nu +- s} at 48 + order, zero outside -p..p
-  __shared__ int l1[64];                          // sum of |digit| of planes 0..4 per column
+  __shared__ int l1[2][64];                       // sum of |digit| of the planes 0..4 and 0..5 per column
   const int P = 2 * p + 1, r = r0 + blockIdx.y;
-  const unsigned long long mb = maxbits[r];
+  const unsigned long long mb = stats[r].maxbits;
   if (mb == 0 || mb >= kInfBits) return;          // the product does not read the image then
+  if (src0 == 0 && threadIdx.x == 0) {
+    const unsigned long long large = mb > (5ull << 52) ? mb - (4ull << 52) : 1;
+    for (int l = blockIdx.x; l < n; l += gridDim.x)
+      if (dmax[(size_t)r * n + l] >= large) {
+        atomicAdd(&stats[r].count, 1);
+        stats[r].disc = l;
+      }
+  }
   const int sh = 46 - scale_exponent(mb);
   const double2* b = xs + ((size_t)r * n + src0 + blockIdx.x) * P;
-  if (threadIdx.x < 64) l1[threadIdx.x] = 0;
+  if (threadIdx.x < 64) l1[0][threadIdx.x] = l1[1][threadIdx.x] = 0;
   if (threadIdx.x < 128) {
     const int o = (int)threadIdx.x - 48 + p;
     double2 v = make_double2(0.0, 0.0);
@@ -160,36 +195,46 @@ k_pack_digits(const double2* __restrict__ xs, int n, int p, int src0, int r0, in
         w[j][2 * h + 1] = v[j];
       }
     }
-    int sum = 0;
+    int sum[2] = {0, 0};
 #pragma unroll
     for (int j = 0; j < PL; ++j) {
       dst[((size_t)kg * PL + j) * npad + col] = make_uint4(w[j][0], w[j][1], w[j][2], w[j][3]);
-      if (j <= 4) {
-        __half2 h = __float2half2_rn(0.0f);       // four digits of at most 128 in a half: exact
+      __half2 h = __float2half2_rn(0.0f);         // four digits of at most 128 in a half: exact
 #pragma unroll
-        for (int i = 0; i < 4; ++i) h = __hadd2(h, __habs2(*reinterpret_cast<const __half2*>(&w[j][i])));
-        sum += (int)__low2float(h) + (int)__high2float(h);
-      }
+      for (int i = 0; i < 4; ++i) h = __hadd2(h, __habs2(*reinterpret_cast<const __half2*>(&w[j][i])));
+      const int d = (int)__low2float(h) + (int)__high2float(h);
+      if (j <= 4) sum[0] += d;
+      sum[1] += d;
     }
-    atomicAdd(&l1[col], sum);
+    atomicAdd(&l1[0][col], sum[0]);
+    atomicAdd(&l1[1][col], sum[1]);
   }
   __syncthreads();
   if (threadIdx.x < 32) {
-    int m = max(l1[threadIdx.x], l1[threadIdx.x + 32]);
+    int m = max(max(l1[0][threadIdx.x], l1[0][threadIdx.x + 32]),
+                max(l1[1][threadIdx.x], l1[1][threadIdx.x + 32]) / 4);
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
     if (threadIdx.x == 0) bound[(size_t)blockIdx.y * gridDim.x + blockIdx.x] = 128 * m;
   }
 }
 
+// Seven levels, or six: what six leave out is 1.3e-15 of the largest coefficient per term.  On right-hand
+// sides whose discs are of one size (a quarter of them within 1/16 of the largest) the operator's
+// translation is then 1.5e-12 off 64-bit sums at 1500 discs, 2.6e-13 with seven levels at 1000, 3.7e-12 and 4.2e-12 in
+// the FP64 pipe's kernels; with one disc 1e4 larger six levels reach 1.4e-11.  Six spare 5 of 26 digit
+// products, which counts where the products bound the kernel, from about 1024 discs on.
+__device__ __forceinline__ bool six_levels(int n, int large_discs) { return n >= 1024 && large_discs >= n / 4; }
+
 // grid: (target tiles, source ranges, right-hand sides); sources src0 + [0, nsrc) of the image; targets
-// row0 .. row0 + nrows - 1, alpha holds those rows.
-template <int NPAD, int LMAX>
+// row0 .. row0 + nrows - 1, alpha holds those rows.  The row of a disc that is the only large one of its
+// right-hand side is left to k_dominant_row.
+template <int NPAD>
 __global__ void __launch_bounds__(THREADS, 1)
 k_translate_digits(const double* __restrict__ cx, const double* __restrict__ cy, int n, int p, PairConsts pc,
                    const longlong2* __restrict__ table, const unsigned char* __restrict__ img,
                    const int* __restrict__ bound, int src0, int nsrc,
-                   int per_cta, int r0, const unsigned long long* __restrict__ maxbits, int row0, int nrows,
+                   int per_cta, int r0, const RhsStats* __restrict__ stats, int row0, int nrows,
                    double2* __restrict__ alpha, int* __restrict__ err) {
   extern __shared__ __align__(128) unsigned char smem[];
   constexpr int STAGE = stage_bytes(NPAD);
@@ -200,7 +245,9 @@ k_translate_digits(const double* __restrict__ cx, const double* __restrict__ cy,
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int P = 2 * p + 1, r = r0 + blockIdx.z;
   const int s_begin = blockIdx.y * per_cta, s_end = min(nsrc, s_begin + per_cta);
-  const unsigned long long mb = maxbits[r];
+  const RhsStats stat = stats[r];
+  const unsigned long long mb = stat.maxbits;
+  const bool six = six_levels(n, stat.count);
   double2* ar = alpha + (size_t)r * nrows * P;
   if (s_begin >= s_end || mb == 0) return;
   if (mb >= kInfBits) {                            // a non-finite coefficient reaches every target
@@ -308,7 +355,8 @@ k_translate_digits(const double* __restrict__ cx, const double* __restrict__ cy,
       ok = __all_sync(0xffffffffu, mbar_wait(accf, group & 1));
       if (!ok) break;
       tc_fence_after();
-      drain_levels<NPAD, LMAX>(tb, acc);
+      if (six) drain_levels<NPAD, 5>(tb, acc);
+      else drain_levels<NPAD, 6>(tb, acc);
       tc_fence_before();
       __syncwarp();
       if (lane == 0) mbar_arrive(acce);
@@ -316,7 +364,7 @@ k_translate_digits(const double* __restrict__ cx, const double* __restrict__ cy,
     if (ok) {
       const int row = blockIdx.x * ROWS + 32 * quad + lane;
       const int ex = scale_exponent(mb) - 48;      // unit of acc
-      if (row < nrows) {
+      if (row < nrows && !(stat.count == 1 && row0 + row == stat.disc)) {
 #pragma unroll
         for (int i = 0; i < HC; ++i) {
           const int col = half * HC + i;
@@ -334,7 +382,7 @@ k_translate_digits(const double* __restrict__ cx, const double* __restrict__ cy,
       int t = 0, group = 0, sum = 0;
       for (int q = 0; q < rounds && ok; ++q) {
         const int w = round_bound[q];
-        const bool start = q == 0 || sum + w > kExact;           // a round stays below it by itself
+        const bool start = q == 0 || sum + w > kExact;
         sum = start ? w : sum + w;
         if (start && q > 0) {
           mma_commit(accf);
@@ -354,8 +402,11 @@ k_translate_digits(const double* __restrict__ cx, const double* __restrict__ cy,
           tc_fence_after();
           const uint32_t sa = sbase + st * STAGE;
           const int ksteps = min(2, steps - 2 * (c / GROUPS));
-          for (int ks = 0; ks < ksteps; ++ks)
-            issue_step<Tile, NPAD, LMAX>(tmem, sa, sa + A_BYTES, ks, start && c == 0 && ks == 0);
+          for (int ks = 0; ks < ksteps; ++ks) {
+            const bool first = start && c == 0 && ks == 0;
+            if (six) issue_step<Tile, NPAD, 5>(tmem, sa, sa + A_BYTES, ks, first);
+            else issue_step<Tile, NPAD, 6>(tmem, sa, sa + A_BYTES, ks, first);
+          }
           mma_commit(empty0 + 8 * st);
         }
       }
@@ -396,20 +447,8 @@ k_translate_digits(const double* __restrict__ cx, const double* __restrict__ cy,
 // ---------------------------------------------------------------------------------------------
 // Near pairs: k rho below pair_z_near (H_{2p} would leave the fixed-point range), from their list.
 // ---------------------------------------------------------------------------------------------
-// The sequences h_s, s = -2p..2p, of every listed pair, once per layout: seq[pair][4p + 1]; zero for
-// the candidates that the digit kernel takes (its own decision, pair_is_near).
-__global__ void k_near_sequences(const double* __restrict__ cx, const double* __restrict__ cy,
-                                 const int* __restrict__ tgt, const int* __restrict__ idx, int nnz, int p, double k,
-                                 PairConsts pc, double2* __restrict__ seq) {
-  const int e = blockIdx.x * blockDim.x + threadIdx.x;
-  if (e >= nnz) return;
-  const int l = tgt[e], m = idx[e];
-  double2* h = seq + (size_t)e * (4 * p + 1) + 2 * p;
-  const double dx = cx[l] - cx[m], dy = cy[l] - cy[m];
-  if (!pair_is_near(fma(dx, dx, dy * dy), pc)) {
-    for (int q = -2 * p; q <= 2 * p; ++q) h[q] = make_double2(0.0, 0.0);
-    return;
-  }
+// h_s, s = -2p..2p, of the pair offset (dx, dy); h points at s = 0.
+__device__ __forceinline__ void pair_sequence(double dx, double dy, double k, int p, double2* h) {
   const double rho = hypot(dx, dy), z = k * rho, iz = 1.0 / z;
   const double2 e1 = make_double2(dx / rho, dy / rho);
   double2 hm = make_double2(j0(z), y0(z)), hq = make_double2(j1(z), y1(z)), eq = e1;
@@ -425,19 +464,70 @@ __global__ void k_near_sequences(const double* __restrict__ cx, const double* __
     eq = cmul(eq, e1);
   }
 }
+// The sequences of every listed pair, once per layout: seq[pair][4p + 1]; zero for the candidates that
+// the digit kernel takes (its own decision, pair_is_near).
+__global__ void k_near_sequences(const double* __restrict__ cx, const double* __restrict__ cy,
+                                 const int* __restrict__ tgt, const int* __restrict__ idx, int nnz, int p, double k,
+                                 PairConsts pc, double2* __restrict__ seq) {
+  const int e = blockIdx.x * blockDim.x + threadIdx.x;
+  if (e >= nnz) return;
+  const int l = tgt[e], m = idx[e];
+  double2* h = seq + (size_t)e * (4 * p + 1) + 2 * p;
+  const double dx = cx[l] - cx[m], dy = cy[l] - cy[m];
+  if (pair_is_near(fma(dx, dx, dy * dy), pc)) {
+    pair_sequence(dx, dy, k, p, h);
+  } else {
+    for (int q = -2 * p; q <= 2 * p; ++q) h[q] = make_double2(0.0, 0.0);
+  }
+}
 
-template <int NPAD, int LMAX>
+// ---------------------------------------------------------------------------------------------
+// The far pairs of the one disc whose coefficients are more than 16 times all others': its own row does not
+// contain it, so the digits, which are cut relative to it, are too coarse there (one disc 1e8 larger: 6e-5
+// of that row at 1500 discs).  Summed in FP64, a warp per 32 sources; without such a disc the CTAs return.
+// ---------------------------------------------------------------------------------------------
+__global__ void __launch_bounds__(32)
+k_dominant_row(const double* __restrict__ cx, const double* __restrict__ cy, int n, int p, double k, PairConsts pc,
+               const double2* __restrict__ xs, const RhsStats* __restrict__ stats, int row0, int nrows,
+               double2* __restrict__ alpha) {
+  __shared__ double2 seq[32][4 * LSMS_MAX_P + 1];
+  const int P = 2 * p + 1, lane = threadIdx.x, r = blockIdx.y;
+  const RhsStats s = stats[r];
+  const int l = s.disc;
+  if (s.count != 1 || s.maxbits >= kInfBits || l < row0 || l >= row0 + nrows) return;
+  const int m0 = blockIdx.x * 32, m = m0 + lane;
+  bool far = false;
+  if (m < n && m != l) {
+    const double dx = cx[l] - cx[m], dy = cy[l] - cy[m];
+    far = !pair_is_near(fma(dx, dx, dy * dy), pc);
+    if (far) pair_sequence(dx, dy, k, p, &seq[lane][2 * p]);
+  }
+  const unsigned mask = __ballot_sync(0xffffffffu, far);
+  __syncwarp();
+  if (lane >= P) return;
+  double2 a = make_double2(0.0, 0.0);
+  for (int i = 0; i < 32; ++i) {
+    if (!(mask >> i & 1)) continue;
+    const double2* b = xs + ((size_t)r * n + m0 + i) * P;
+    for (int q = 0; q < P; ++q) a = cfma(seq[i][2 * p - lane + q], b[q], a);
+  }
+  double2* o = alpha + ((size_t)r * nrows + (l - row0)) * P + lane;
+  atomicAdd(&o->x, a.x);
+  atomicAdd(&o->y, a.y);
+}
+
+template <int NPAD>
 void launch_digits(dim3 grid, cudaStream_t st, const lsms_ctx* c, const PairConsts& pc, const unsigned char* img,
-                   const int* bound, int src0, int nsrc, int per_cta, int r0, const unsigned long long* maxbits,
+                   const int* bound, int src0, int nsrc, int per_cta, int r0, const RhsStats* stats,
                    int row0, int nrows, double2* alpha, int* err) {
   static std::once_flag attr;
   std::call_once(attr, [] {
-    cudaFuncSetAttribute(k_translate_digits<NPAD, LMAX>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    cudaFuncSetAttribute(k_translate_digits<NPAD>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                          (int)smem_bytes(NPAD));
   });
-  k_translate_digits<NPAD, LMAX><<<grid, THREADS, smem_bytes(NPAD), st>>>(
+  k_translate_digits<NPAD><<<grid, THREADS, smem_bytes(NPAD), st>>>(
       c->d_cx, c->d_cy, c->n, c->p, pc, (const longlong2*)c->f64tc.d_table, img, bound, src0, nsrc, per_cta, r0,
-      maxbits, row0, nrows, alpha, err);
+      stats, row0, nrows, alpha, err);
 }
 
 constexpr size_t kImageBytes = (size_t)256 << 20;   // digits of X held at once
@@ -560,28 +650,28 @@ int translate_f64_tc(lsms_ctx* c, int nrhs, const double2* xs, double2* alpha, c
   const int run = (n + runs - 1) / runs;
   runs = (n + run - 1) / run;
   const size_t img_bytes = (size_t)rb * std::min(run, n) * src_bytes;
-  const size_t max_bytes = ((size_t)nrhs * 8 + 255) & ~size_t(255);
+  const size_t stat_bytes = ((size_t)nrhs * sizeof(RhsStats) + 255) & ~size_t(255);
+  const size_t max_bytes = stat_bytes + (((size_t)nrhs * n * 8 + 255) & ~size_t(255));
   const size_t bound_bytes = ((size_t)rb * std::min(run, n) * sizeof(int) + 255) & ~size_t(255);
   if (ensure(c, f.ws, max_bytes + bound_bytes + img_bytes)) {   // no memory for the image: the FP64 pipe
     c->err.clear();
     launch_translate_f64(c->d_cx, c->d_cy, n, p, c->k2, xs, alpha, nrhs, st, row0, nrows);
     return check_cuda(c, "translate_f64");
   }
-  unsigned long long* maxbits = (unsigned long long*)f.ws.ptr;
+  RhsStats* stats = (RhsStats*)f.ws.ptr;
+  unsigned long long* dmax = (unsigned long long*)((unsigned char*)f.ws.ptr + stat_bytes);
   int* bound = (int*)((unsigned char*)f.ws.ptr + max_bytes);
   unsigned char* img = (unsigned char*)f.ws.ptr + max_bytes + bound_bytes;
   int* err = tc_err_flag(c);
-  cudaMemsetAsync(maxbits, 0, (size_t)nrhs * 8, st);
-  const long long per = 2LL * n * P;
-  k_absmax<<<dim3((int)std::min<long long>((per + 1023) / 1024, 152), nrhs), 256, 0, st>>>((const double*)xs, per,
-                                                                                          maxbits);
+  cudaMemsetAsync(stats, 0, (size_t)nrhs * sizeof(RhsStats), st);
+  k_disc_max<<<dim3((n + 7) / 8, nrhs), 256, 0, st>>>(xs, n, P, dmax, stats);
   const PairConsts pc = pair_consts(c->k2, pair_z_near(p));
   const int tiles = (nrows + ROWS - 1) / ROWS;
   for (int r0 = 0; r0 < nrhs; r0 += rb) {
     const int nr = std::min(rb, nrhs - r0);
     for (int s0 = 0; s0 < n; s0 += run) {
       const int ns = std::min(run, n - s0);
-      k_pack_digits<<<dim3(ns, nr), 256, 0, st>>>(xs, n, p, s0, r0, npad, 2 * steps, maxbits, img, bound);
+      k_pack_digits<<<dim3(ns, nr), 256, 0, st>>>(xs, n, p, s0, r0, npad, 2 * steps, dmax, stats, img, bound);
       // source ranges: the fewest waves of 152 CTAs times the rounds of two sources of a CTA, plus
       // about two rounds of time per CTA for its start and end
       int best = 1;
@@ -597,18 +687,15 @@ int translate_f64_tc(lsms_ctx* c, int nrhs, const double2* xs, double2* alpha, c
       }
       const int per_cta = (((ns + best - 1) / best) + GROUPS - 1) / GROUPS * GROUPS;
       dim3 grid(tiles, (ns + per_cta - 1) / per_cta, nr);
-      // seven levels for the short layouts, whose phases are the most accurate: there the six levels'
-      // 1.3e-15 of a term would show beside the 1e-16 k rho of its phase
-      const bool more = n < 1024;
-#define LSMS_DG(NP)                                                                                       \
-  (more ? launch_digits<NP, 6>(grid, st, c, pc, img, bound, s0, ns, per_cta, r0, maxbits, row0, nrows, alpha, err)           \
-        : launch_digits<NP, 5>(grid, st, c, pc, img, bound, s0, ns, per_cta, r0, maxbits, row0, nrows, alpha, err))
+#define LSMS_DG(NP) launch_digits<NP>(grid, st, c, pc, img, bound, s0, ns, per_cta, r0, stats, row0, nrows, alpha, err)
       if (npad == 32) LSMS_DG(32);
       else if (npad == 48) LSMS_DG(48);
       else LSMS_DG(64);
 #undef LSMS_DG
     }
   }
+  k_dominant_row<<<dim3((n + 31) / 32, nrhs), 32, 0, st>>>(c->d_cx, c->d_cy, n, p, c->k2, pc, xs, stats, row0, nrows,
+                                                          alpha);
   // lists cut so that the warps fill the chip (300 discs: 161 -> 107 us the translation, 1000: 478 -> 444)
   const int near_splits = (int)std::max<long long>(1, std::min<long long>(4, 152LL * 24 / std::max(1LL, (long long)nrows * nrhs)));
   if (f.nnz > 0)
