@@ -25,7 +25,7 @@ int upload(lsms_ctx* c, T** dptr, const std::vector<cplx>& v) {
   if (v.empty()) return LSMS_OK;
   if (cudaMalloc((void**)dptr, v.size() * sizeof(cplx)) != cudaSuccess)
     return fail(c, LSMS_ERR_OOM, "cudaMalloc failed for a constant table");
-  if (cudaMemcpy(*dptr, v.data(), v.size() * sizeof(cplx), cudaMemcpyHostToDevice) != cudaSuccess)
+  if (copy_up(c, *dptr, v.data(), v.size() * sizeof(cplx)) != cudaSuccess)
     return fail(c, LSMS_ERR_CUDA, "cudaMemcpy failed for a constant table");
   return LSMS_OK;
 }
@@ -338,9 +338,9 @@ int create_stack(const std::vector<cplx>& kc, const std::vector<double>& ds, int
     return fail(nullptr, rc, m);
   }
   if (cudaMalloc((void**)&c->d_scale_in, s_in.size() * sizeof(double)) != cudaSuccess ||
-      cudaMemcpy(c->d_scale_in, s_in.data(), s_in.size() * sizeof(double), cudaMemcpyHostToDevice) != cudaSuccess ||
+      copy_up(c, c->d_scale_in, s_in.data(), s_in.size() * sizeof(double)) != cudaSuccess ||
       cudaMalloc((void**)&c->d_hscale, c->P * sizeof(double)) != cudaSuccess ||
-      cudaMemcpy(c->d_hscale, c->hscale.data(), c->P * sizeof(double), cudaMemcpyHostToDevice) != cudaSuccess) {
+      copy_up(c, c->d_hscale, c->hscale.data(), c->P * sizeof(double)) != cudaSuccess) {
     lsms_destroy(c);
     return fail(nullptr, LSMS_ERR_CUDA, "upload of the order scales failed");
   }
@@ -348,6 +348,11 @@ int create_stack(const std::vector<cplx>& kc, const std::vector<double>& ds, int
   if (cudaMallocHost((void**)&c->h_pinned, 64 * sizeof(double)) != cudaSuccess) {
     lsms_destroy(c);
     return fail(nullptr, LSMS_ERR_CUDA, "cudaMallocHost failed");
+  }
+  if (cudaStreamSynchronize(c->stream) != cudaSuccess) {
+    cudaGetLastError();
+    lsms_destroy(c);
+    return fail(nullptr, LSMS_ERR_CUDA, "upload of the constant tables failed");
   }
   *out = c;
   return LSMS_OK;
@@ -461,8 +466,8 @@ extern "C" int lsms_set_particles(lsms_ctx* c, int n, const double* xy) {
     return fail(c, LSMS_ERR_OOM, "cudaMalloc failed for the layout tables");
   }
   if (n > 0) {
-    cudaMemcpy(c->d_cx, xs.data(), n * sizeof(double), cudaMemcpyHostToDevice);
-    cudaMemcpy(c->d_cy, c->cy.data(), n * sizeof(double), cudaMemcpyHostToDevice);
+    copy_up(c, c->d_cx, xs.data(), n * sizeof(double));
+    copy_up(c, c->d_cy, c->cy.data(), n * sizeof(double));
     launch_etables(c->d_cx, c->d_cy, n, c->d_lam, c->d_g2, c->ns, c->d, c->d_eagg, c->d_edis, c->stream);
     cudaStreamSynchronize(c->stream);
     if ((rc = check_cuda(c, "set_particles"))) return rc;
@@ -767,7 +772,8 @@ extern "C" int lsms_set_scattering_diagonal(lsms_ctx* c, const double* s) {
     s_out[q] = S[q];
     s_out[P + q] = c->hscale[q] * S[q];
   }
-  if (cudaMemcpy(c->d_scale_out, s_out.data(), s_out.size() * sizeof(cplx), cudaMemcpyHostToDevice) != cudaSuccess)
+  if (copy_up(c, c->d_scale_out, s_out.data(), s_out.size() * sizeof(cplx)) != cudaSuccess ||
+      cudaStreamSynchronize(c->stream) != cudaSuccess)
     return check_cuda(c, "set_scattering_diagonal");
   c->S = S;
   c->custom_diag = s != nullptr;

@@ -444,7 +444,8 @@ int mixed_check(lsms_ctx* c) {
   int h = 0;
   if (cudaMemcpy(&h, t->d_err, sizeof(int), cudaMemcpyDeviceToHost) != cudaSuccess) return check_cuda(c, "mixed_check");
   if (h) {
-    cudaMemset(t->d_err, 0, sizeof(int));
+    cudaMemsetAsync(t->d_err, 0, sizeof(int), c->stream);
+    cudaStreamSynchronize(c->stream);
     return ctx_fail(c, LSMS_ERR_CUDA, "tensor-core contraction timed out waiting on a barrier (code " + std::to_string(h) + ")");
   }
   return LSMS_OK;

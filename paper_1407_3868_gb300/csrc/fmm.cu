@@ -809,14 +809,14 @@ int fmm_setup(lsms_ctx* c) {
     fmm_free(c);
     return ctx_fail(c, LSMS_ERR_OOM, "set_fmm: cudaMalloc failed for the box tables");
   }
-  cudaMemcpy(f.d_perm, perm.data(), n * sizeof(int), cudaMemcpyHostToDevice);
-  cudaMemcpy(f.d_bstart, bstart.data(), (nb + 1) * sizeof(int), cudaMemcpyHostToDevice);
-  cudaMemcpy(f.d_dbox, dbox.data(), n * sizeof(int), cudaMemcpyHostToDevice);
-  cudaMemcpy(f.d_sbox, sbox.data(), n * sizeof(int), cudaMemcpyHostToDevice);
-  cudaMemcpy(f.d_scx, scx.data(), n * sizeof(double), cudaMemcpyHostToDevice);
-  cudaMemcpy(f.d_scy, scy.data(), n * sizeof(double), cudaMemcpyHostToDevice);
-  cudaMemcpy(f.d_cptr, cptr.data(), (n + 1) * sizeof(int), cudaMemcpyHostToDevice);
-  if (!csrc.empty()) cudaMemcpy(f.d_csrc, csrc.data(), csrc.size() * sizeof(int), cudaMemcpyHostToDevice);
+  copy_up(c, f.d_perm, perm.data(), n * sizeof(int));
+  copy_up(c, f.d_bstart, bstart.data(), (nb + 1) * sizeof(int));
+  copy_up(c, f.d_dbox, dbox.data(), n * sizeof(int));
+  copy_up(c, f.d_sbox, sbox.data(), n * sizeof(int));
+  copy_up(c, f.d_scx, scx.data(), n * sizeof(double));
+  copy_up(c, f.d_scy, scy.data(), n * sizeof(double));
+  copy_up(c, f.d_cptr, cptr.data(), (n + 1) * sizeof(int));
+  if (!csrc.empty()) copy_up(c, f.d_csrc, csrc.data(), csrc.size() * sizeof(int));
   cudaStream_t st = c->stream;
   // FP64 near field: the stored sequences (430 MB for 20,000 discs at p = 14) if they are few and fit;
   // otherwise k_fmm_near forms them anew in every application
@@ -884,6 +884,7 @@ int fmm_update(lsms_ctx* c) {
   const int rc = fmm_setup(c);
   const std::string msg = c->err;
   const int rs = f64tc_sequences(c);
+  cudaStreamSynchronize(c->stream);                  // the tables are there for every stream
   if (rc) c->err = msg;
   return rc ? rc : rs;
 }

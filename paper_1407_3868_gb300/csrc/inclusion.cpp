@@ -478,7 +478,8 @@ extern "C" int lsms_set_scattering_matrix(lsms_ctx* c, const double* s) {
       c->d_smt = nullptr;
       return ctx_fail(c, LSMS_ERR_OOM, "set_scattering_matrix: cudaMalloc failed");
     }
-    if (cudaMemcpy(c->d_smt, t.data(), t.size() * sizeof(cplx), cudaMemcpyHostToDevice) != cudaSuccess)
+    if (copy_up(c, c->d_smt, t.data(), t.size() * sizeof(cplx)) != cudaSuccess ||
+        cudaStreamSynchronize(c->stream) != cudaSuccess)
       return check_cuda(c, "set_scattering_matrix");
     c->smat = m;
     c->dense = true;
@@ -512,7 +513,8 @@ extern "C" int lsms_set_orientations(lsms_ctx* c, int n, const double* theta) {
     if (!std::isfinite(theta[j])) return ctx_fail(c, LSMS_ERR_ARG, "set_orientations: non-finite angle");
   int rc;
   if ((rc = ensure(c, c->theta_buf, (size_t)n * sizeof(double)))) return rc;
-  if (cudaMemcpy(c->theta_buf.ptr, theta, (size_t)n * sizeof(double), cudaMemcpyHostToDevice) != cudaSuccess)
+  if (copy_up(c, c->theta_buf.ptr, theta, (size_t)n * sizeof(double)) != cudaSuccess ||
+      cudaStreamSynchronize(c->stream) != cudaSuccess)
     return check_cuda(c, "set_orientations");
   c->has_theta = true;
   return LSMS_OK;

@@ -12,6 +12,12 @@ int ctx_fail(lsms_ctx* c, int code, const std::string& msg);
 int create_stack(const std::vector<cplx>& kc, const std::vector<double>& ds, int layer, double kp,
                  double radius, int p, const lsms_contour* contour, int precision, lsms_ctx** out);
 int ensure(lsms_ctx* c, DevBuf& b, size_t bytes);
+// Host to device in order with the context's stream, which does not wait for the legacy stream of
+// cudaMemcpy.  `src` is free on return (pageable memory is staged); the caller synchronises the stream
+// before other streams may read dst.
+inline cudaError_t copy_up(lsms_ctx* c, void* dst, const void* src, size_t bytes) {
+  return cudaMemcpyAsync(dst, src, bytes, cudaMemcpyHostToDevice, c->stream);
+}
 // Gaussian elimination with partial pivoting, a (n x n) x = b (n x nrhs), row-major; false if singular
 bool solve_small(std::vector<cplx>& a, int n, std::vector<cplx>& b, int nrhs);
 // box-compressed translation (fmm.cu)

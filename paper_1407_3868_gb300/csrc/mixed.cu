@@ -870,8 +870,8 @@ static int build_near_pairs(lsms_ctx* c, std::vector<int>& wide_ptr, std::vector
     cudaGetLastError();
     return ctx_fail(c, LSMS_ERR_OOM, "cudaMalloc failed for the near-pair tables");
   }
-  cudaMemcpy(c->d_near_ptr, ptr.data(), (n + 1) * sizeof(int), cudaMemcpyHostToDevice);
-  if (!idx.empty()) cudaMemcpy(c->d_near_idx, idx.data(), idx.size() * sizeof(int), cudaMemcpyHostToDevice);
+  copy_up(c, c->d_near_ptr, ptr.data(), (n + 1) * sizeof(int));
+  if (!idx.empty()) copy_up(c, c->d_near_idx, idx.data(), idx.size() * sizeof(int));
   if (n > 0 && c->near_nnz > 0)
     k_near_h01<<<(n + 127) / 128, 128, 0, c->stream>>>(c->d_cx, c->d_cy, c->d_near_ptr, c->d_near_idx, n, c->k2,
                                                        (float4*)c->d_near_h);
@@ -1133,8 +1133,9 @@ int batch_translation_items(lsms_ctx* c) {
     cudaGetLastError();
     return ctx_fail(c, LSMS_ERR_OOM, "batched translation: cudaMalloc failed for the work items");
   }
-  cudaMemcpy(c->d_bt_items, items.data(), items.size() * sizeof(int4), cudaMemcpyHostToDevice);
-  cudaMemcpy(c->d_bt_lays, lays.data(), nl * sizeof(longlong4), cudaMemcpyHostToDevice);
+  copy_up(c, c->d_bt_items, items.data(), items.size() * sizeof(int4));
+  copy_up(c, c->d_bt_lays, lays.data(), nl * sizeof(longlong4));
+  cudaStreamSynchronize(c->stream);
   c->bt_ncta = (int)items.size();
   c->bt_part = part;
   return check_cuda(c, "batched translation work items");
@@ -1166,12 +1167,12 @@ int batch_translation_setup(lsms_ctx* c) {
     const int n = k->n, kn = std::max(k->near_nnz, 0);
     if (n <= 0) continue;
     std::vector<int> kp(n + 1), ki((size_t)std::max(kn, 1));
-    if (cudaMemcpy((float4*)c->d_bt_cff + off, k->d_lp_misc, n * sizeof(float4), cudaMemcpyDeviceToDevice) !=
-            cudaSuccess ||
+    if (cudaMemcpyAsync((float4*)c->d_bt_cff + off, k->d_lp_misc, n * sizeof(float4), cudaMemcpyDeviceToDevice,
+                        c->stream) != cudaSuccess ||
         cudaMemcpy(kp.data(), k->d_near_ptr, (n + 1) * sizeof(int), cudaMemcpyDeviceToHost) != cudaSuccess ||
         (kn > 0 && (cudaMemcpy(ki.data(), k->d_near_idx, kn * sizeof(int), cudaMemcpyDeviceToHost) != cudaSuccess ||
-                    cudaMemcpy((float4*)c->d_bt_ntab + e0, k->d_near_h, kn * sizeof(float4),
-                               cudaMemcpyDeviceToDevice) != cudaSuccess))) {
+                    cudaMemcpyAsync((float4*)c->d_bt_ntab + e0, k->d_near_h, kn * sizeof(float4),
+                                    cudaMemcpyDeviceToDevice, c->stream) != cudaSuccess))) {
       batch_translation_free(c);
       return check_cuda(c, "set_layouts: batched translation tables");
     }
@@ -1180,8 +1181,8 @@ int batch_translation_setup(lsms_ctx* c) {
     e0 += kn;
   }
   nptr[total] = (int)e0;
-  cudaMemcpy(c->d_bt_nptr, nptr.data(), (total + 1) * sizeof(int), cudaMemcpyHostToDevice);
-  if (nnz > 0) cudaMemcpy(c->d_bt_nidx, nidx.data(), nnz * sizeof(int), cudaMemcpyHostToDevice);
+  copy_up(c, c->d_bt_nptr, nptr.data(), (total + 1) * sizeof(int));
+  if (nnz > 0) copy_up(c, c->d_bt_nidx, nidx.data(), nnz * sizeof(int));
   int rc = batch_translation_items(c);
   if (rc) {
     batch_translation_free(c);

@@ -596,7 +596,7 @@ int f64tc_setup(lsms_ctx* c, const std::vector<int>& ptr, const std::vector<int>
     std::memcpy(host.data() + TABLE_BYTES + (n + 1) * sizeof(int), li.data(), nnz * sizeof(int));
     std::memcpy(host.data() + TABLE_BYTES + (n + 1 + nnz) * sizeof(int), tgt.data(), nnz * sizeof(int));
   }
-  cudaMemcpy(f.d_table, host.data(), bytes, cudaMemcpyHostToDevice);
+  copy_up(c, f.d_table, host.data(), bytes);
   f.nnz = (int)nnz;
   f.ready = true;
   f.digits = digits;
