@@ -45,13 +45,80 @@ std::vector<cplx> shift_phase(const lsms_ctx* c, double sign) {
 // ---------------------------------------------------------------------------------------------
 int ctx_fail(lsms_ctx* c, int code, const std::string& msg) { return fail(c, code, msg); }
 
+static void drop(DevBuf& b) {
+  if (b.ptr) cudaFree(b.ptr);
+  b = DevBuf();
+}
+
+bool is_capturing(cudaStream_t st) {
+  cudaStreamCaptureStatus s = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(st, &s) == cudaSuccess) return s != cudaStreamCaptureStatusNone;
+  cudaGetLastError();                                // the legacy stream beside a capture on another
+  return true;
+}
+
+static size_t optional_bytes(const lsms_ctx* c) {
+  const size_t seq = (size_t)(4 * c->p + 1) * sizeof(double2);
+  size_t b = c->ws_f64tc.bytes + c->ws_zgemm.bytes + (c->f64tc.d_seq ? c->f64tc.nnz * seq : 0) +
+             (c->fmm.d_cseq64 ? c->fmm.pairs * seq : 0);
+  for (const lsms_ctx* k : c->kids) b += optional_bytes(k);
+  return b;
+}
+
+// cudaFree waits for the kernels that use the memory.
+void release_optional(lsms_ctx* c) {
+  for (lsms_ctx* k : c->kids) release_optional(k);
+  if (!c->kids.empty()) batch_clear_graphs(c);
+  if (c->parent) c->parent->graphs_stale = true;
+  drop(c->ws_f64tc);
+  drop(c->ws_zgemm);
+  f64tc_free(c);
+  zgemm_free(c);
+  if (c->fmm.d_cseq64) cudaFree(c->fmm.d_cseq64);
+  c->fmm.d_cseq64 = nullptr;
+}
+
+cudaError_t device_alloc(lsms_ctx* c, void** p, size_t bytes) {
+  *p = nullptr;
+  const size_t held = optional_bytes(c);
+  cudaError_t e = held > 0 && bytes > c->required_limit ? cudaErrorMemoryAllocation : cudaMalloc(p, bytes);
+  if (e == cudaErrorMemoryAllocation && held > 0) {
+    cudaGetLastError();
+    release_optional(c);
+    e = cudaMalloc(p, bytes);
+  }
+  return e;
+}
+
+cudaError_t device_alloc_optional(lsms_ctx* c, void** p, size_t bytes) {
+  *p = nullptr;
+  cudaError_t e = cudaErrorMemoryAllocation;
+  if (bytes <= c->optional_limit && optional_bytes(c) <= c->optional_limit - bytes) e = cudaMalloc(p, bytes);
+  if (e != cudaSuccess) cudaGetLastError();
+  return e;
+}
+
+bool ensure_optional(lsms_ctx* c, DevBuf& b, size_t bytes, cudaStream_t st) {
+  if (bytes <= b.bytes && b.ptr) return true;
+  if (is_capturing(st)) return false;
+  drop(b);
+  if (device_alloc_optional(c, &b.ptr, bytes) != cudaSuccess) return false;
+  b.bytes = bytes;
+  return true;
+}
+
+// For the tests of the fallbacks: see lsms_ctx.
+void memory_limits(lsms_ctx* c, size_t optional, size_t required) {
+  c->optional_limit = optional;
+  c->required_limit = required;
+  for (lsms_ctx* k : c->kids) memory_limits(k, optional, required);
+}
+
 int ensure(lsms_ctx* c, DevBuf& b, size_t bytes) {
   if (bytes <= b.bytes && b.ptr) return LSMS_OK;
-  if (b.ptr) cudaFree(b.ptr);
-  b.ptr = nullptr;
-  b.bytes = 0;
+  drop(b);
   if (bytes == 0) bytes = 16;
-  if (cudaMalloc(&b.ptr, bytes) != cudaSuccess) {
+  if (device_alloc(c, &b.ptr, bytes) != cudaSuccess) {
     cudaGetLastError();
     return fail(c, LSMS_ERR_OOM, "cudaMalloc failed for a workspace of " + std::to_string(bytes) + " bytes");
   }
@@ -75,6 +142,12 @@ int need_particles(lsms_ctx* c) {
 int translate_f64(lsms_ctx* c, int nrhs, const double2* xs, double2* alpha, cudaStream_t st, int row0, int nrows) {
   if (nrows < 0) nrows = c->n - row0;
   if (c->n == 0 || nrhs == 0 || nrows <= 0) return LSMS_OK;
+  // a mixed context stores the near sequences when it first needs them
+  if (c->f64tc.ready && !c->f64tc.used && !f64tc_usable(c) && !is_capturing(st)) {
+    c->f64tc.used = true;
+    const int rc = f64tc_sequences(c);
+    if (rc) return rc;
+  }
   if (f64tc_usable(c)) return translate_f64_tc(c, nrhs, xs, alpha, st, row0, nrows);
   launch_translate_f64(c->d_cx, c->d_cy, c->n, c->p, c->k2, xs, alpha, nrhs, st, row0, nrows);
   return LSMS_OK;
@@ -402,7 +475,7 @@ extern "C" void lsms_destroy(lsms_ctx* c) {
     if (q) cudaFree(q);
   DevBuf* bufs[] = {&c->ws_x, &c->ws_y, &c->ws_xs, &c->ws_alpha, &c->ws_g, &c->ws_v, &c->ws_pq,
                     &c->ws_sig, &c->ws_aux, &c->ws_rows, &c->gm_v, &c->gm_h, &c->gm_small, &c->gm_x, &c->gm_r,
-                    &c->gm_w, &c->sol, &c->ws_lp, &c->ws_tcb, &c->gm_b, &c->gm_mask, &c->gm_off, &c->theta_buf};
+                    &c->gm_w, &c->sol, &c->ws_lp, &c->ws_tcb, &c->ws_f64tc, &c->ws_zgemm, &c->gm_loop, &c->gm_b, &c->gm_mask, &c->gm_off, &c->theta_buf};
   for (DevBuf* b : bufs)
     if (b->ptr) cudaFree(b->ptr);
   tc_free(c);
@@ -459,8 +532,9 @@ extern "C" int lsms_set_particles(lsms_ctx* c, int n, const double* xy) {
   c->has_theta = false;                      // orientations refer to the previous particles
   const size_t nb = (size_t)(n > 0 ? n : 1) * sizeof(double);
   const size_t eb = (size_t)2 * c->ns * (n > 0 ? n : 1) * sizeof(double2);
-  if (cudaMalloc((void**)&c->d_cx, nb) != cudaSuccess || cudaMalloc((void**)&c->d_cy, nb) != cudaSuccess ||
-      cudaMalloc((void**)&c->d_eagg, eb) != cudaSuccess || cudaMalloc((void**)&c->d_edis, eb) != cudaSuccess) {
+  if (device_alloc(c, (void**)&c->d_cx, nb) != cudaSuccess || device_alloc(c, (void**)&c->d_cy, nb) != cudaSuccess ||
+      device_alloc(c, (void**)&c->d_eagg, eb) != cudaSuccess ||
+      device_alloc(c, (void**)&c->d_edis, eb) != cudaSuccess) {
     cudaGetLastError();
     c->n = -1;
     return fail(c, LSMS_ERR_OOM, "cudaMalloc failed for the layout tables");

@@ -24,6 +24,7 @@
 bool is_batch(const lsms_ctx* c) { return c && !c->kids.empty(); }
 
 void batch_clear_graphs(lsms_ctx* c) {
+  c->graphs_stale = false;
   for (auto& g : c->graphs)
     if (g.exec) cudaGraphExecDestroy(g.exec);
   c->graphs.clear();
@@ -62,6 +63,9 @@ extern "C" int lsms_set_layouts(lsms_ctx* c, int n_layouts, const int* counts, c
       batch_free(c);
       return ctx_fail(c, rc, "set_layouts: layout " + std::to_string(l) + ": " + m);
     }
+    k->parent = c;
+    k->optional_limit = c->optional_limit;
+    k->required_limit = c->required_limit;
     k->use_graphs = c->use_graphs;
     k->split_mult = c->split_mult;
     k->f32_shape = c->f32_shape;
@@ -81,6 +85,10 @@ extern "C" int lsms_set_layouts(lsms_ctx* c, int n_layouts, const int* counts, c
     }
     c->kid_off.push_back(off);
     rc = lsms_set_particles(k, counts[l], xy + 2 * off);
+    if (rc == LSMS_ERR_OOM) {                       // what the layouts so far can do without
+      release_optional(c);
+      rc = lsms_set_particles(k, counts[l], xy + 2 * off);
+    }
     if (rc) {
       const std::string m = k->err;
       batch_free(c);
@@ -167,6 +175,7 @@ int batch_apply(lsms_ctx* c, int nrhs, const double2* x, double2* y, int flags, 
   cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
   if (cudaStreamIsCapturing(st, &cap) == cudaSuccess && cap == cudaStreamCaptureStatusActive)
     return fork_join_apply(c, x, y, flags, st);     // recorded into the graph being captured
+  if (c->graphs_stale) batch_clear_graphs(c);
   for (auto& g : c->graphs)
     if (g.x == x && g.y == y && g.flags == flags) {
       if (cudaGraphLaunch(g.exec, st) != cudaSuccess) return check_cuda(c, "batched apply graph");
@@ -175,6 +184,10 @@ int batch_apply(lsms_ctx* c, int nrhs, const double2* x, double2* y, int flags, 
   // first application with these buffers: run it directly (this also sizes every workspace), then
   // capture the same fork/join for the next calls
   int rc = fork_join_apply(c, x, y, flags, st);
+  if (rc == LSMS_ERR_OOM && x != y) {               // once more without what the layouts can do without
+    release_optional(c);
+    rc = fork_join_apply(c, x, y, flags, st);
+  }
   if (rc) return rc;
   if (!c->use_graphs || c->graphs.size() >= 16) return check_cuda(c, "batched apply");
   cudaGraph_t graph = nullptr;
@@ -235,6 +248,16 @@ int batch_solve(lsms_ctx* c, int nsrc, const double* src_xy, double tol, int max
   for (int i = 1; i < nt; ++i) pool.emplace_back(work);
   work();
   for (auto& th : pool) th.join();
+  // layouts that ran out of memory beside the others: by themselves, without what can be done without
+  bool first = true;
+  for (int l = 0; l < nl; ++l) {
+    if (rc[l] != LSMS_ERR_OOM) continue;
+    if (first) release_optional(c);
+    first = false;
+    const long long o = c->kid_off[l] * P * 2;
+    rc[l] = lsms_solve(c->kids[l], 1, nsrc == 1 ? src_xy : src_xy + 2 * l, tol, maxiter, x0 ? x0 + o : nullptr,
+                   beta_out ? beta_out + o : nullptr, &inf[l]);
+  }
   int status = LSMS_OK;
   for (int l = 0; l < nl; ++l) {
     if (rc[l] == LSMS_OK) continue;

@@ -461,7 +461,6 @@ inline size_t aligned(size_t bytes) { return (bytes + 255) & ~size_t(255); }
 void zgemm_free(lsms_ctx* c) {
   ZgemmTc& z = c->zgemm;
   if (z.d_exp) cudaFree(z.d_exp);
-  if (z.ws.ptr) cudaFree(z.ws.ptr);
   z = ZgemmTc();
 }
 
@@ -489,8 +488,7 @@ int zgemm_setup(lsms_ctx* c) {
   const size_t be = aligned(2 * per * sizeof(int)), bl = aligned(list.size() * sizeof(int)), bs = aligned(scls.size()),
                bt = aligned(tiles.size() * sizeof(int4)), bc = aligned(start.size() * sizeof(int));
   const size_t lists = bl + bs + bt + bc, bm = 2 * per * 8 + 16;
-  if (cudaMalloc((void**)&z.d_exp, be + lists + bm) != cudaSuccess) {
-    cudaGetLastError();
+  if (device_alloc_optional(c, (void**)&z.d_exp, be + lists + bm) != cudaSuccess) {
     zgemm_free(c);
     return LSMS_OK;                                // the FP64 pipe then (launch_zgemm_direct)
   }
@@ -544,13 +542,12 @@ int zgemm_f64(lsms_ctx* c, bool agg, int nrhs, const double2* B, double2* C, cud
   const size_t one = sb * std::max(z.stages, z.classes * dis_stages);
   const int rb = (int)std::max<size_t>(1, std::min<size_t>(nrhs, kImageBytes / one));
   const size_t mbytes = aligned((size_t)nrhs * z.classes * 32 * 8);
-  if (ensure(c, z.ws, mbytes + rb * one)) {   // no memory for the images
-    c->err.clear();
+  if (!ensure_optional(c, c->ws_zgemm, mbytes + rb * one, st)) {   // as in translate_f64_tc
     launch_zgemm_direct(l.A, l.M, l.K, B, C, c->P, nrhs, st);
     return check_cuda(c, "zgemm_f64");
   }
-  unsigned long long* maxbits = (unsigned long long*)z.ws.ptr;
-  unsigned char* img = (unsigned char*)z.ws.ptr + mbytes;
+  unsigned long long* maxbits = (unsigned long long*)c->ws_zgemm.ptr;
+  unsigned char* img = (unsigned char*)c->ws_zgemm.ptr + mbytes;
   l.maxbits = maxbits;
   l.img = img;
   l.aexp = z.d_exp + (agg ? 0 : (size_t)z.classes * 2 * c->ns);

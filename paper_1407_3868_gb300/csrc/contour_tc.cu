@@ -363,8 +363,8 @@ int tc_setup(lsms_ctx* c) {
   t->kpad_dis = round_up(4 * c->ns, BK);
   const size_t sa = (size_t)NPL * 2 * c->ns * t->kpad_agg * 2;
   const size_t sd = (size_t)NPL * c->n * t->kpad_dis * 2;
-  if (cudaMalloc((void**)&t->a_agg, sa) != cudaSuccess || cudaMalloc((void**)&t->a_dis, sd) != cudaSuccess ||
-      cudaMalloc((void**)&t->d_err, sizeof(int)) != cudaSuccess) {
+  if (device_alloc(c, (void**)&t->a_agg, sa) != cudaSuccess || device_alloc(c, (void**)&t->a_dis, sd) != cudaSuccess ||
+      device_alloc(c, (void**)&t->d_err, sizeof(int)) != cudaSuccess) {
     cudaGetLastError();
     return ctx_fail(c, LSMS_ERR_OOM, "cudaMalloc failed for the BF16 plane tables");
   }
@@ -400,9 +400,9 @@ static int tc_reserve(lsms_ctx* c, int ncols, cudaStream_t st) {
   t->c_agg = t->c_dis = nullptr;
   t->ncols_pad = 0;
   const size_t sb1 = (size_t)NPL * need * t->kpad_agg * 2, sb2 = (size_t)NPL * need * t->kpad_dis * 2;
-  if (cudaMalloc((void**)&t->b_agg, sb1) != cudaSuccess || cudaMalloc((void**)&t->b_dis, sb2) != cudaSuccess ||
-      cudaMalloc((void**)&t->c_agg, (size_t)2 * t->ns * need * 4) != cudaSuccess ||
-      cudaMalloc((void**)&t->c_dis, (size_t)t->n * need * 4) != cudaSuccess) {
+  if (device_alloc(c, (void**)&t->b_agg, sb1) != cudaSuccess || device_alloc(c, (void**)&t->b_dis, sb2) != cudaSuccess ||
+      device_alloc(c, (void**)&t->c_agg, (size_t)2 * t->ns * need * 4) != cudaSuccess ||
+      device_alloc(c, (void**)&t->c_dis, (size_t)t->n * need * 4) != cudaSuccess) {
     cudaGetLastError();
     return ctx_fail(c, LSMS_ERR_OOM, "cudaMalloc failed for the BF16 operand planes");
   }

@@ -80,7 +80,7 @@ __global__ void k_fmm_shift_table(const double* __restrict__ cx, const double* _
 
 // The near field's pair sequences: row k of seq = h[s + 2p] = H_s(k rho) e^{i s phi}, s = -2p..2p (then
 // one zero), for list entry k (target perm[t], source csrc[k]); built in FP64 (CUDA J0, Y0, J1, Y1,
-// forward recurrence, angular powers) and stored in FP32, and in FP64 (rows of 4p + 1) where seq64 is
+// forward recurrence, angular powers) and stored in FP32 (seq) and in FP64 (seq64, rows of 4p + 1), where
 // given.  A warp per target, a lane per pair.
 __global__ void k_fmm_pair_seq(const double* __restrict__ cx, const double* __restrict__ cy,
                                const int* __restrict__ perm, const int* __restrict__ cptr,
@@ -94,17 +94,19 @@ __global__ void k_fmm_pair_seq(const double* __restrict__ cx, const double* __re
     const double dx = cx[l] - cx[m], dy = cy[l] - cy[m];
     const double rho = hypot(dx, dy), z = k * rho;
     const double2 e1 = make_double2(dx / rho, dy / rho);
-    float2* h = seq + (size_t)e * RS;
+    float2* h = seq ? seq + (size_t)e * RS : nullptr;
     double2* h64 = seq64 ? seq64 + (size_t)e * (4 * p + 1) : nullptr;
     double2 hm = make_double2(j0(z), y0(z)), hq = make_double2(j1(z), y1(z)), eq = e1;
-    h[c0] = make_float2((float)hm.x, (float)hm.y);
+    if (h) h[c0] = make_float2((float)hm.x, (float)hm.y);
     if (h64) h64[c0] = hm;
     for (int q = 1; q <= 2 * p; ++q) {
       const double2 v = cmul(hq, eq);
       double2 u = cmul(hq, make_double2(eq.x, -eq.y));
       if (q & 1) u = make_double2(-u.x, -u.y);
-      h[c0 + q] = make_float2((float)v.x, (float)v.y);
-      h[c0 - q] = make_float2((float)u.x, (float)u.y);
+      if (h) {
+        h[c0 + q] = make_float2((float)v.x, (float)v.y);
+        h[c0 - q] = make_float2((float)u.x, (float)u.y);
+      }
       if (h64) {
         h64[c0 + q] = v;
         h64[c0 - q] = u;
@@ -117,7 +119,7 @@ __global__ void k_fmm_pair_seq(const double* __restrict__ cx, const double* __re
         eq = cmul(eq, e1);
       }
     }
-    h[4 * p + 1] = make_float2(0.f, 0.f);
+    if (h) h[4 * p + 1] = make_float2(0.f, 0.f);
   }
 }
 
@@ -725,6 +727,15 @@ void fmm_free(lsms_ctx* c) {
   f.order_req = order;
 }
 
+// Room for the FP64 near field's stored sequences (430 MB for 20,000 discs at p = 14) if they are few and
+// fit; otherwise k_fmm_near forms them anew in every application.
+static void alloc_seq64(lsms_ctx* c) {
+  FmmState& f = c->fmm;
+  f.seq64_tried = true;
+  const size_t bytes = f.pairs * (size_t)(4 * c->p + 1) * sizeof(double2);
+  if (bytes > 0 && bytes <= kSeq64Bytes) device_alloc_optional(c, (void**)&f.d_cseq64, bytes);
+}
+
 // Box tables of the current layout (host grouping; device shift tables and transformed kernel).
 int fmm_setup(lsms_ctx* c) {
   FmmState& f = c->fmm;
@@ -795,15 +806,15 @@ int fmm_setup(lsms_ctx* c) {
   const size_t ysz = (size_t)f.n1 * W, asz = (size_t)nb * W;
   const size_t tsz = (size_t)n * (2 * f.S + 1);
   const size_t hsz = (size_t)std::max(1, 2 * (f.dmin - 2)) * (4 * f.order + 1);
-  if (cudaMalloc((void**)&f.d_perm, n * sizeof(int)) != cudaSuccess ||
-      cudaMalloc((void**)&f.d_bstart, (nb + 1) * sizeof(int)) != cudaSuccess ||
-      cudaMalloc((void**)&f.d_dbox, n * sizeof(int)) != cudaSuccess ||
-      cudaMalloc((void**)&f.d_sbox, n * sizeof(int)) != cudaSuccess ||
-      cudaMalloc((void**)&f.d_scx, n * sizeof(double)) != cudaSuccess ||
-      cudaMalloc((void**)&f.d_scy, n * sizeof(double)) != cudaSuccess ||
-      cudaMalloc((void**)&f.d_cptr, (n + 1) * sizeof(int)) != cudaSuccess ||
-      cudaMalloc((void**)&f.d_csrc, std::max<size_t>(1, csrc.size()) * sizeof(int)) != cudaSuccess ||
-      cudaMalloc((void**)&f.d_cseq, std::max<size_t>(1, csrc.size()) * (4 * p + 2) * sizeof(float2)) !=
+  if (device_alloc(c, (void**)&f.d_perm, n * sizeof(int)) != cudaSuccess ||
+      device_alloc(c, (void**)&f.d_bstart, (nb + 1) * sizeof(int)) != cudaSuccess ||
+      device_alloc(c, (void**)&f.d_dbox, n * sizeof(int)) != cudaSuccess ||
+      device_alloc(c, (void**)&f.d_sbox, n * sizeof(int)) != cudaSuccess ||
+      device_alloc(c, (void**)&f.d_scx, n * sizeof(double)) != cudaSuccess ||
+      device_alloc(c, (void**)&f.d_scy, n * sizeof(double)) != cudaSuccess ||
+      device_alloc(c, (void**)&f.d_cptr, (n + 1) * sizeof(int)) != cudaSuccess ||
+      device_alloc(c, (void**)&f.d_csrc, std::max<size_t>(1, csrc.size()) * sizeof(int)) != cudaSuccess ||
+      device_alloc(c, (void**)&f.d_cseq, std::max<size_t>(1, csrc.size()) * (4 * p + 2) * sizeof(float2)) !=
           cudaSuccess) {
     cudaGetLastError();
     fmm_free(c);
@@ -818,13 +829,8 @@ int fmm_setup(lsms_ctx* c) {
   copy_up(c, f.d_cptr, cptr.data(), (n + 1) * sizeof(int));
   if (!csrc.empty()) copy_up(c, f.d_csrc, csrc.data(), csrc.size() * sizeof(int));
   cudaStream_t st = c->stream;
-  // FP64 near field: the stored sequences (430 MB for 20,000 discs at p = 14) if they are few and fit;
-  // otherwise k_fmm_near forms them anew in every application
-  const size_t seq64 = csrc.size() * (size_t)(4 * p + 1) * sizeof(double2);
-  if (seq64 > 0 && seq64 <= kSeq64Bytes && cudaMalloc((void**)&f.d_cseq64, seq64) != cudaSuccess) {
-    cudaGetLastError();
-    f.d_cseq64 = nullptr;
-  }
+  f.pairs = csrc.size();
+  if (c->precision != LSMS_MIXED) alloc_seq64(c);
   k_fmm_pair_seq<<<(n + 3) / 4, 128, 0, st>>>(c->d_cx, c->d_cy, f.d_perm, f.d_cptr, f.d_csrc, n, p, c->k2, f.d_cseq,
                                               f.d_cseq64);
   if (!f.far) {                    // near field only
@@ -832,22 +838,22 @@ int fmm_setup(lsms_ctx* c) {
     f.ready = true;
     return check_cuda(c, "set_fmm");
   }
-  if (cudaMalloc((void**)&f.d_tab, tsz * sizeof(double2)) != cudaSuccess ||
-      cudaMalloc((void**)&f.d_khat, gsz * sizeof(double2)) != cudaSuccess ||
-      cudaMalloc((void**)&f.d_grid, ysz * sizeof(double2)) != cudaSuccess ||
-      cudaMalloc((void**)&f.d_bq, asz * sizeof(double2)) != cudaSuccess ||
-      cudaMalloc((void**)&f.d_acc, asz * sizeof(double2)) != cudaSuccess ||
-      cudaMalloc((void**)&f.d_hd, hsz * sizeof(double2)) != cudaSuccess ||
-      cudaMalloc((void**)&f.d_twn, (size_t)f.n1 * sizeof(double2)) != cudaSuccess ||
-      cudaMalloc((void**)&f.d_tw2, (size_t)f.n2 * sizeof(double2)) != cudaSuccess ||
-      cudaMalloc((void**)&f.d_tab32, tsz * sizeof(float2)) != cudaSuccess ||
-      cudaMalloc((void**)&f.d_khat32, gsz * sizeof(float2)) != cudaSuccess ||
-      cudaMalloc((void**)&f.d_grid32, ysz * sizeof(float2)) != cudaSuccess ||
-      cudaMalloc((void**)&f.d_bq32, asz * sizeof(float2)) != cudaSuccess ||
-      cudaMalloc((void**)&f.d_acc32, asz * sizeof(float2)) != cudaSuccess ||
-      cudaMalloc((void**)&f.d_hd32, hsz * sizeof(float2)) != cudaSuccess ||
-      cudaMalloc((void**)&f.d_twn32, (size_t)f.n1 * sizeof(float2)) != cudaSuccess ||
-      cudaMalloc((void**)&f.d_tw232, (size_t)f.n2 * sizeof(float2)) != cudaSuccess) {
+  if (device_alloc(c, (void**)&f.d_tab, tsz * sizeof(double2)) != cudaSuccess ||
+      device_alloc(c, (void**)&f.d_khat, gsz * sizeof(double2)) != cudaSuccess ||
+      device_alloc(c, (void**)&f.d_grid, ysz * sizeof(double2)) != cudaSuccess ||
+      device_alloc(c, (void**)&f.d_bq, asz * sizeof(double2)) != cudaSuccess ||
+      device_alloc(c, (void**)&f.d_acc, asz * sizeof(double2)) != cudaSuccess ||
+      device_alloc(c, (void**)&f.d_hd, hsz * sizeof(double2)) != cudaSuccess ||
+      device_alloc(c, (void**)&f.d_twn, (size_t)f.n1 * sizeof(double2)) != cudaSuccess ||
+      device_alloc(c, (void**)&f.d_tw2, (size_t)f.n2 * sizeof(double2)) != cudaSuccess ||
+      device_alloc(c, (void**)&f.d_tab32, tsz * sizeof(float2)) != cudaSuccess ||
+      device_alloc(c, (void**)&f.d_khat32, gsz * sizeof(float2)) != cudaSuccess ||
+      device_alloc(c, (void**)&f.d_grid32, ysz * sizeof(float2)) != cudaSuccess ||
+      device_alloc(c, (void**)&f.d_bq32, asz * sizeof(float2)) != cudaSuccess ||
+      device_alloc(c, (void**)&f.d_acc32, asz * sizeof(float2)) != cudaSuccess ||
+      device_alloc(c, (void**)&f.d_hd32, hsz * sizeof(float2)) != cudaSuccess ||
+      device_alloc(c, (void**)&f.d_twn32, (size_t)f.n1 * sizeof(float2)) != cudaSuccess ||
+      device_alloc(c, (void**)&f.d_tw232, (size_t)f.n2 * sizeof(float2)) != cudaSuccess) {
     cudaGetLastError();
     fmm_free(c);
     return ctx_fail(c, LSMS_ERR_OOM, "set_fmm: cudaMalloc failed for the box tables");
@@ -922,6 +928,15 @@ int fmm_translate(lsms_ctx* c, int nrhs, const double2* xs, double2* alpha, bool
     if (timed) cudaEventRecord(f.ev[2], st);
     f.timed = timed;
     return LSMS_OK;
+  }
+  // a mixed context stores them with its first FP64 residual
+  if (!f.seq64_tried && !is_capturing(st)) {
+    alloc_seq64(c);
+    if (f.d_cseq64) {
+      k_fmm_pair_seq<<<(n + 3) / 4, 128, 0, st>>>(c->d_cx, c->d_cy, f.d_perm, f.d_cptr, f.d_csrc, n, p, c->k2, nullptr,
+                                                  f.d_cseq64);
+      cudaStreamSynchronize(st);                     // the next call may be on another stream
+    }
   }
   if (f.d_cseq64) {
     if (timed) cudaEventRecord(f.ev[1], st);

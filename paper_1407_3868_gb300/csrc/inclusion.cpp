@@ -473,7 +473,7 @@ extern "C" int lsms_set_scattering_matrix(lsms_ctx* c, const double* s) {
         t[(size_t)q * P + l] = m[(size_t)l * P + q];
         t[(size_t)P * P + (size_t)q * P + l] = c->hscale[l] * m[(size_t)l * P + q];
       }
-    if (!c->d_smt && cudaMalloc((void**)&c->d_smt, t.size() * sizeof(cplx)) != cudaSuccess) {
+    if (!c->d_smt && device_alloc(c, (void**)&c->d_smt, t.size() * sizeof(cplx)) != cudaSuccess) {
       cudaGetLastError();
       c->d_smt = nullptr;
       return ctx_fail(c, LSMS_ERR_OOM, "set_scattering_matrix: cudaMalloc failed");

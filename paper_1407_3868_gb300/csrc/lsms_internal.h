@@ -3,6 +3,8 @@
 
 #include <cuda_runtime.h>
 
+#include <atomic>
+
 #include <complex>
 #include <string>
 #include <vector>
@@ -66,6 +68,8 @@ struct FmmState {
   int* d_csrc = nullptr;            //   target in box order, source disc of each pair
   float2* d_cseq = nullptr;         // [pairs][4p + 2] their Hankel sequences (FP64-built, stored FP32)
   double2* d_cseq64 = nullptr;      // [pairs][4p + 1] the same in FP64 (null: formed anew, k_fmm_near)
+  size_t pairs = 0;
+  bool seq64_tried = false;         // their allocation, once per set of tables
   float2* d_tab32 = nullptr;        // FP32 copies of the shift tables, the transformed kernel, the
   float2* d_khat32 = nullptr;       // work array, the box coefficients and expansions, the
   float2* d_grid32 = nullptr;       // direct-offset kernels and the twiddles (mixed-precision far
@@ -89,7 +93,7 @@ struct F64Tc {
   int* d_idx = nullptr;             // [nnz] sources, then [nnz] targets
   void* d_seq = nullptr;            // double2 [nnz][4p + 1]: their Hankel sequences (f64tc_sequences)
   int nnz = 0;
-  DevBuf ws;                        // scales and digit images of the coefficients
+  bool used = false;                // a mixed context has translated all pairs in FP64
 };
 
 // FP64 contour contractions on the tensor cores (contour_f64_tc.cu).
@@ -102,7 +106,6 @@ struct ZgemmTc {
   int* d_start = nullptr;           // [classes + 1] where each begins
   unsigned char* d_scls = nullptr;  // class of every stage
   void* d_tiles = nullptr;          // int4 (class, first position, rows, 0)
-  DevBuf ws;                        // scales and digit images of the right operand
 };
 
 struct lsms_ctx {
@@ -191,9 +194,16 @@ struct lsms_ctx {
                                     // run on the tensor cores; 0 = never
   int tc_flush = 32;                // source discs summed per FP32 tensor-memory accumulation
   DevBuf ws_tcb;                    // BF16 coefficient images of the tensor-core translation
+  // digit images of the FP64 products and the scales they rest on: memory the context can do without
+  // (release_optional), as the sequences in f64tc and fmm.d_cseq64
+  DevBuf ws_f64tc, ws_zgemm;
+  size_t optional_limit = SIZE_MAX; // bytes of such memory at most, and the largest request that is granted
+  size_t required_limit = SIZE_MAX; //   while some is held (lowered by the tests of the fallbacks)
 
   // a batch of independent layouts (lsms_set_layouts): one child context per layout
   std::vector<lsms_ctx*> kids;
+  lsms_ctx* parent = nullptr;
+  std::atomic<bool> graphs_stale{false};   // a layout gave memory back that the captured graphs refer to
   std::vector<long long> kid_off;   // first disc of every layout, and the total at the end
   struct GraphEntry {
     const void* x;

@@ -12,6 +12,16 @@ int ctx_fail(lsms_ctx* c, int code, const std::string& msg);
 int create_stack(const std::vector<cplx>& kc, const std::vector<double>& ds, int layer, double kp,
                  double radius, int p, const lsms_contour* contour, int precision, lsms_ctx** out);
 int ensure(lsms_ctx* c, DevBuf& b, size_t bytes);
+// Device memory.  When there is none left for a request, the memory that the context and its layouts
+// can do without is given back (release_optional) and the request made again; the optional requests
+// just fail.
+cudaError_t device_alloc(lsms_ctx* c, void** p, size_t bytes);
+cudaError_t device_alloc_optional(lsms_ctx* c, void** p, size_t bytes);
+bool ensure_optional(lsms_ctx* c, DevBuf& b, size_t bytes, cudaStream_t st);   // not while st is captured
+// The tables and images of the FP64 digit products and the FP64 near sequences of the boxes: the FP64 pipe's
+// kernels run from then on (until the next layout).
+void release_optional(lsms_ctx* c);
+bool is_capturing(cudaStream_t st);
 // Host to device in order with the context's stream, which does not wait for the legacy stream of
 // cudaMemcpy.  `src` is free on return (pageable memory is staged); the caller synchronises the stream
 // before other streams may read dst.

@@ -864,9 +864,9 @@ static int build_near_pairs(lsms_ctx* c, std::vector<int>& wide_ptr, std::vector
   }
   c->near_nnz = (int)idx.size();
   const size_t hb = (size_t)(c->near_nnz > 0 ? c->near_nnz : 1) * sizeof(float4);
-  if (cudaMalloc((void**)&c->d_near_ptr, (n + 1) * sizeof(int)) != cudaSuccess ||
-      cudaMalloc((void**)&c->d_near_idx, (idx.empty() ? 1 : idx.size()) * sizeof(int)) != cudaSuccess ||
-      cudaMalloc(&c->d_near_h, hb) != cudaSuccess) {
+  if (device_alloc(c, (void**)&c->d_near_ptr, (n + 1) * sizeof(int)) != cudaSuccess ||
+      device_alloc(c, (void**)&c->d_near_idx, (idx.empty() ? 1 : idx.size()) * sizeof(int)) != cudaSuccess ||
+      device_alloc(c, &c->d_near_h, hb) != cudaSuccess) {
     cudaGetLastError();
     return ctx_fail(c, LSMS_ERR_OOM, "cudaMalloc failed for the near-pair tables");
   }
@@ -882,7 +882,7 @@ static int build_near_pairs(lsms_ctx* c, std::vector<int>& wide_ptr, std::vector
 int build_lowp_tables(lsms_ctx* c) {
   if (c->d_lp_misc) cudaFree(c->d_lp_misc);
   c->d_lp_misc = nullptr;
-  if (cudaMalloc(&c->d_lp_misc, (size_t)(c->n > 0 ? c->n : 1) * sizeof(float4)) != cudaSuccess) {
+  if (device_alloc(c, &c->d_lp_misc, (size_t)(c->n > 0 ? c->n : 1) * sizeof(float4)) != cudaSuccess) {
     cudaGetLastError();
     return ctx_fail(c, LSMS_ERR_OOM, "cudaMalloc failed for the float-float centres");
   }
@@ -1128,8 +1128,8 @@ int batch_translation_items(lsms_ctx* c) {
   if (c->d_bt_items) cudaFree(c->d_bt_items);
   if (c->d_bt_lays) cudaFree(c->d_bt_lays);
   c->d_bt_items = c->d_bt_lays = nullptr;
-  if (cudaMalloc(&c->d_bt_items, std::max<size_t>(1, items.size()) * sizeof(int4)) != cudaSuccess ||
-      cudaMalloc(&c->d_bt_lays, nl * sizeof(longlong4)) != cudaSuccess) {
+  if (device_alloc(c, &c->d_bt_items, std::max<size_t>(1, items.size()) * sizeof(int4)) != cudaSuccess ||
+      device_alloc(c, &c->d_bt_lays, nl * sizeof(longlong4)) != cudaSuccess) {
     cudaGetLastError();
     return ctx_fail(c, LSMS_ERR_OOM, "batched translation: cudaMalloc failed for the work items");
   }
@@ -1151,10 +1151,10 @@ int batch_translation_setup(lsms_ctx* c) {
   long long nnz = 0;
   for (int l = 0; l < nl; ++l) nnz += std::max(c->kids[l]->near_nnz, 0);
   nidx.resize((size_t)std::max<long long>(nnz, 1));
-  if (cudaMalloc(&c->d_bt_cff, total * sizeof(float4)) != cudaSuccess ||
-      cudaMalloc((void**)&c->d_bt_nptr, (total + 1) * sizeof(int)) != cudaSuccess ||
-      cudaMalloc((void**)&c->d_bt_nidx, (size_t)std::max<long long>(nnz, 1) * sizeof(int)) != cudaSuccess ||
-      cudaMalloc(&c->d_bt_ntab, (size_t)std::max<long long>(nnz, 1) * sizeof(float4)) != cudaSuccess ||
+  if (device_alloc(c, &c->d_bt_cff, total * sizeof(float4)) != cudaSuccess ||
+      device_alloc(c, (void**)&c->d_bt_nptr, (total + 1) * sizeof(int)) != cudaSuccess ||
+      device_alloc(c, (void**)&c->d_bt_nidx, (size_t)std::max<long long>(nnz, 1) * sizeof(int)) != cudaSuccess ||
+      device_alloc(c, &c->d_bt_ntab, (size_t)std::max<long long>(nnz, 1) * sizeof(float4)) != cudaSuccess ||
       cudaEventCreateWithFlags(&c->bt_ev, cudaEventDisableTiming) != cudaSuccess) {
     cudaGetLastError();
     batch_translation_free(c);

@@ -539,7 +539,7 @@ constexpr double kNearBytes = 8e9;                  // near sequences beside the
 
 void f64tc_free(lsms_ctx* c) {
   F64Tc& f = c->f64tc;
-  void* ptrs[] = {f.d_table, f.d_seq, f.ws.ptr};   // d_ptr and d_idx lie behind the table
+  void* ptrs[] = {f.d_table, f.d_seq};             // d_ptr and d_idx lie behind the table
   for (void* p : ptrs)
     if (p) cudaFree(p);
   f = F64Tc();
@@ -582,8 +582,7 @@ int f64tc_setup(lsms_ctx* c, const std::vector<int>& ptr, const std::vector<int>
     for (int e = lp[l]; e < lp[l + 1]; ++e) tgt[e] = l;
   // one allocation: table, list pointers, sources, targets
   const size_t bytes = TABLE_BYTES + ((size_t)(n + 1) + 2 * ne) * sizeof(int);
-  if (cudaMalloc(&f.d_table, bytes) != cudaSuccess) {
-    cudaGetLastError();
+  if (device_alloc_optional(c, &f.d_table, bytes) != cudaSuccess) {
     f64tc_free(c);
     return LSMS_OK;
   }
@@ -604,18 +603,19 @@ int f64tc_setup(lsms_ctx* c, const std::vector<int>& ptr, const std::vector<int>
 }
 
 // The stored near sequences (63 MB at 5000 discs, p = 14) exist while all-pairs FP64 translations
-// can run: not while every translation goes through boxes.
+// can run: not while every translation goes through boxes, nor in a mixed context that has had none
+// (its solves come to them with their first FP64 residual).
 int f64tc_sequences(lsms_ctx* c) {
   F64Tc& f = c->f64tc;
-  const bool want = f.ready && f.nnz > 0 && !(c->fmm.ready && c->fmm.scope == LSMS_FMM_ALL);
+  const bool want = f.ready && f.nnz > 0 && (c->precision != LSMS_MIXED || f.used) &&
+                    !(c->fmm.ready && c->fmm.scope == LSMS_FMM_ALL);
   if (want == (f.d_seq != nullptr)) return LSMS_OK;
   if (!want) {
     cudaFree(f.d_seq);
     f.d_seq = nullptr;
     return LSMS_OK;
   }
-  if (cudaMalloc(&f.d_seq, (size_t)f.nnz * (4 * c->p + 1) * sizeof(double2)) != cudaSuccess) {
-    cudaGetLastError();
+  if (device_alloc_optional(c, &f.d_seq, (size_t)f.nnz * (4 * c->p + 1) * sizeof(double2)) != cudaSuccess) {
     f64tc_free(c);
     return LSMS_OK;
   }
@@ -653,15 +653,15 @@ int translate_f64_tc(lsms_ctx* c, int nrhs, const double2* xs, double2* alpha, c
   const size_t stat_bytes = ((size_t)nrhs * sizeof(RhsStats) + 255) & ~size_t(255);
   const size_t max_bytes = stat_bytes + (((size_t)nrhs * n * 8 + 255) & ~size_t(255));
   const size_t bound_bytes = ((size_t)rb * std::min(run, n) * sizeof(int) + 255) & ~size_t(255);
-  if (ensure(c, f.ws, max_bytes + bound_bytes + img_bytes)) {   // no memory for the image: the FP64 pipe
-    c->err.clear();
+  // without memory for the image (or inside a capture that began before there was one): the FP64 pipe
+  if (!ensure_optional(c, c->ws_f64tc, max_bytes + bound_bytes + img_bytes, st)) {
     launch_translate_f64(c->d_cx, c->d_cy, n, p, c->k2, xs, alpha, nrhs, st, row0, nrows);
     return check_cuda(c, "translate_f64");
   }
-  RhsStats* stats = (RhsStats*)f.ws.ptr;
-  unsigned long long* dmax = (unsigned long long*)((unsigned char*)f.ws.ptr + stat_bytes);
-  int* bound = (int*)((unsigned char*)f.ws.ptr + max_bytes);
-  unsigned char* img = (unsigned char*)f.ws.ptr + max_bytes + bound_bytes;
+  RhsStats* stats = (RhsStats*)c->ws_f64tc.ptr;
+  unsigned long long* dmax = (unsigned long long*)((unsigned char*)c->ws_f64tc.ptr + stat_bytes);
+  int* bound = (int*)((unsigned char*)c->ws_f64tc.ptr + max_bytes);
+  unsigned char* img = (unsigned char*)c->ws_f64tc.ptr + max_bytes + bound_bytes;
   int* err = tc_err_flag(c);
   cudaMemsetAsync(stats, 0, (size_t)nrhs * sizeof(RhsStats), st);
   k_disc_max<<<dim3((n + 7) / 8, nrhs), 256, 0, st>>>(xs, n, P, dmax, stats);
