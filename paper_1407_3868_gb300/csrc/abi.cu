@@ -150,6 +150,7 @@ int translate_f64(lsms_ctx* c, int nrhs, const double2* xs, double2* alpha, cuda
   }
   if (f64tc_usable(c)) return translate_f64_tc(c, nrhs, xs, alpha, st, row0, nrows);
   launch_translate_f64(c->d_cx, c->d_cy, c->n, c->p, c->k2, xs, alpha, nrhs, st, row0, nrows);
+  ++c->f64_launches;
   return LSMS_OK;
 }
 
@@ -161,6 +162,7 @@ int reflection_f64(lsms_ctx* c, int nrhs, const double2* xs, double2* alpha, cud
   if ((rc = ensure(c, c->ws_v, (size_t)nrhs * 2 * ns * P * sizeof(double2)))) return rc;
   double2* G = (double2*)c->ws_g.ptr;
   double2* V = (double2*)c->ws_v.ptr;
+  ++c->f64_launches;                                 // the aggregate's kernel or the per-node stage
   if ((double)2 * ns * n < kZgemmMinTable) {
     launch_node_direct(ns, n, P, nrhs, c->d_eagg, xs, c->d_fagg, c->d_refl, c->d_udis, V, st);
     return zgemm_f64(c, false, nrhs, V, alpha, st);
@@ -188,6 +190,7 @@ int apply_device(lsms_ctx* c, int nrhs, const double2* x, double2* y, int flags,
   const bool given = (flags & LSMS_APPLY_TRANSLATION_GIVEN) && c->alpha_given;
   double2* alpha = given ? c->alpha_given : (double2*)c->ws_alpha.ptr;
   int launches = 0;
+  c->f64_launches = 0;
   const bool boxes = c->fmm.ready && (c->fmm.scope == 0 || (flags & LSMS_APPLY_RESIDUAL_INTERNAL));
   if (mixed && c->side && !given && !boxes && !(flags & (LSMS_APPLY_NO_TRANSLATION | LSMS_APPLY_NO_REFLECTION)) &&
       mixed_sym_path(c, nrhs)) {
@@ -219,7 +222,7 @@ int apply_device(lsms_ctx* c, int nrhs, const double2* x, double2* y, int flags,
   if (!(flags & LSMS_APPLY_NO_TRANSLATION)) {
     // box method (fmm.cu): per right-hand side M2M, five transform passes, the direct offsets
     // and L2L; then the near field (FP64: one kernel; mixed: FP32 copy of xs and the pair-list
-    // kernel).  All pairs: FP64 one kernel; mixed: FP32 copy of xs, the translation (+ the
+    // kernel).  All pairs: FP64 as translate_f64 counts; mixed: FP32 copy of xs, the translation (+ the
     // partial-sum reduction, or the packing of the tensor-core operands) and the near pairs
     if (given) {
       // computed for every layout of the batch at once (translate_mixed_batch)
@@ -232,7 +235,6 @@ int apply_device(lsms_ctx* c, int nrhs, const double2* x, double2* y, int flags,
       launches += 3 + (c->near_nnz > 0 ? 1 : 0);
       if ((rc = translate_mixed(c, nrhs, xs, alpha, st))) return rc;
     } else {
-      launches += c->f64tc.digits ? 3 + (c->f64tc.nnz > 0 ? 1 : 0) : 1;
       if ((rc = translate_f64(c, nrhs, xs, alpha, st))) return rc;
     }
   } else {
@@ -248,7 +250,7 @@ int apply_device(lsms_ctx* c, int nrhs, const double2* x, double2* y, int flags,
     } else {
       if ((rc = reflection_f64(c, nrhs, xs, alpha, st))) return rc;
     }
-    launches += mixed ? 5 : 3;   // split, GEMM, per-node stage, GEMM, add / GEMM, stage, GEMM
+    if (mixed) launches += 5;    // split, GEMM, per-node stage, GEMM, add
   }
   if (c->timing) cudaEventRecord(c->ev[2], st);
   if (c->dense && !(flags & LSMS_APPLY_ALPHA))
@@ -257,7 +259,7 @@ int apply_device(lsms_ctx* c, int nrhs, const double2* x, double2* y, int flags,
   else
     launch_combine(x, alpha, c->d_scale_out + mode * P, y, nrhs, n, P, (flags & LSMS_APPLY_ALPHA) ? 1 : 0, st);
   ++launches;
-  c->last_launches = launches;
+  c->last_launches = launches + c->f64_launches;
   return check_cuda(c, "apply");
 }
 

@@ -530,6 +530,7 @@ int zgemm_f64(lsms_ctx* c, bool agg, int nrhs, const double2* B, double2* C, cud
   l.C = C;
   l.M = agg ? 2 * c->ns : c->n;
   l.K = agg ? c->n : 2 * c->ns;
+  ++c->f64_launches;                                 // the direct product or the order maxima
   if (!z.ready) {
     launch_zgemm_direct(l.A, l.M, l.K, B, C, c->P, nrhs, st);
     return LSMS_OK;
@@ -561,6 +562,7 @@ int zgemm_f64(lsms_ctx* c, bool agg, int nrhs, const double2* B, double2* C, cud
   for (l.r0 = 0; l.r0 < nrhs; l.r0 += rb) {
     const int nr = std::min(rb, nrhs - l.r0);
     const int items = l.stages * KG * (npad / 2);
+    c->f64_launches += 2;
     k_pack_columns<<<dim3(std::min((items + 127) / 128, 1024), nr, images), 128, 0, st>>>(
         B, l.K, c->P, l.r0, l.stages, npad, z.classes, z.d_kidx, z.d_scls, kexp, maxbits, img);
     // K ranges: the fewest rounds of 152 CTAs times the stages of a CTA, plus a start and an end worth

@@ -238,6 +238,7 @@ struct lsms_ctx {
   int timing = 0;
   cudaEvent_t ev[4] = {nullptr, nullptr, nullptr, nullptr};
   int last_launches = 0;            // kernels launched by the last operator application
+  int f64_launches = 0;             // those of its FP64 translation and contour products, as they count themselves
 
   // solution of the last lsms_solve (device, unscaled beta), per source
   int n_src = 0;

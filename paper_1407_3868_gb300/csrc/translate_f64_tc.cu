@@ -637,6 +637,7 @@ int translate_f64_tc(lsms_ctx* c, int nrhs, const double2* xs, double2* alpha, c
   if (!f.digits) {
     // about 8 warps per SM
     if (f.nnz > 0) {
+      ++c->f64_launches;
       const int splits = (int)std::max<long long>(1, std::min<long long>(n - 1, 152LL * 8 / std::max(1LL, (long long)nrows * nrhs)));
       launch_near_f64(n, p, nullptr, row0, nrows, splits, f.d_ptr, f.d_idx, (const double2*)f.d_seq, xs, nrhs, alpha, st);
     }
@@ -656,6 +657,7 @@ int translate_f64_tc(lsms_ctx* c, int nrhs, const double2* xs, double2* alpha, c
   // without memory for the image (or inside a capture that began before there was one): the FP64 pipe
   if (!ensure_optional(c, c->ws_f64tc, max_bytes + bound_bytes + img_bytes, st)) {
     launch_translate_f64(c->d_cx, c->d_cy, n, p, c->k2, xs, alpha, nrhs, st, row0, nrows);
+    ++c->f64_launches;
     return check_cuda(c, "translate_f64");
   }
   RhsStats* stats = (RhsStats*)c->ws_f64tc.ptr;
@@ -671,6 +673,7 @@ int translate_f64_tc(lsms_ctx* c, int nrhs, const double2* xs, double2* alpha, c
     const int nr = std::min(rb, nrhs - r0);
     for (int s0 = 0; s0 < n; s0 += run) {
       const int ns = std::min(run, n - s0);
+      c->f64_launches += 2;
       k_pack_digits<<<dim3(ns, nr), 256, 0, st>>>(xs, n, p, s0, r0, npad, 2 * steps, dmax, stats, img, bound);
       // source ranges: the fewest waves of 152 CTAs times the rounds of two sources of a CTA, plus
       // about two rounds of time per CTA for its start and end
@@ -696,6 +699,7 @@ int translate_f64_tc(lsms_ctx* c, int nrhs, const double2* xs, double2* alpha, c
   }
   k_dominant_row<<<dim3((n + 31) / 32, nrhs), 32, 0, st>>>(c->d_cx, c->d_cy, n, p, c->k2, pc, xs, stats, row0, nrows,
                                                           alpha);
+  c->f64_launches += 2 + (f.nnz > 0 ? 1 : 0);          // maxima, the dominant row, near pairs
   // lists cut so that the warps fill the chip (300 discs: 161 -> 107 us the translation, 1000: 478 -> 444)
   const int near_splits = (int)std::max<long long>(1, std::min<long long>(4, 152LL * 24 / std::max(1LL, (long long)nrows * nrhs)));
   if (f.nnz > 0)
