@@ -549,13 +549,18 @@ void f64tc_free(lsms_ctx* c) {
 // distance (host arrays).  Layouts of fewer than kMinDiscs discs (not one full tile of rows) or of
 // mostly near pairs (summed on the FP64 pipe either way) store the sequences of all their pairs if
 // these take at most kStoreBytes (16 discs: 75 us with the sequences formed anew -> 11 us);
-// larger ones, and layouts for whose tables there is no memory, keep k_translate_f64 and its symmetric
-// form.
+// larger ones, layouts for whose tables there is no memory and lengths below 1e-18 or above 1e18 keep
+// k_translate_f64 and its symmetric form.
 int f64tc_setup(lsms_ctx* c, const std::vector<int>& ptr, const std::vector<int>& idx) {
   f64tc_free(c);
   F64Tc& f = c->f64tc;
   const int n = c->n;
   if (n <= 0 || !tc_err_flag(c)) return LSMS_OK;
+  // near and far pairs are told apart by squared distances in FP32, whose range these must not leave (in
+  // any unit of length in use they do not)
+  double reach = c->d;
+  for (int j = 0; j < n; ++j) reach = std::max(reach, 2.0 * std::fabs(c->cx[j] - c->xc));
+  if (!(pair_z_near(c->p) / c->k2 > 1e-18) || !(reach < 1e18)) return LSMS_OK;
   const double seq_bytes = (4 * c->p + 1) * (double)sizeof(double2);
   const bool digits = n >= kMinDiscs && (double)idx.size() <= 0.5 * n * (double)(n - 1) &&
                       (double)idx.size() * seq_bytes <= kNearBytes;
