@@ -470,7 +470,7 @@ extern "C" void lsms_destroy(lsms_ctx* c) {
   if (c->side) cudaStreamSynchronize(c->side);
   batch_free(c);
   void* ptrs[] = {c->d_lam, c->d_g1, c->d_g2, c->d_refl, c->d_inc, c->d_field, c->d_fagg, c->d_udis,
-                  c->d_scale_in, c->d_hscale, c->d_scale_out, c->d_cx, c->d_cy, c->d_eagg, c->d_edis,
+                  c->d_scale_in, c->d_hscale, c->d_scale_out, c->d_cx, c->d_cy, c->d_eagg, c->d_edis, c->d_eorder,
                   c->d_eagg_lp, c->d_edis_lp, c->d_lp_misc, c->d_near_ptr, c->d_near_idx, c->d_near_h,
                   c->d_smt};
   for (void* q : ptrs)
@@ -522,11 +522,13 @@ extern "C" int lsms_set_particles(lsms_ctx* c, int n, const double* xy) {
   fmm_free(c);                               // the previous layout's, also where this call fails below
   f64tc_free(c);
   zgemm_free(c);
-  void* old[] = {c->d_cx, c->d_cy, c->d_eagg, c->d_edis, c->d_eagg_lp, c->d_edis_lp, c->d_lp_misc};
+  void* old[] = {c->d_cx, c->d_cy, c->d_eagg, c->d_edis, c->d_eorder, c->d_eagg_lp, c->d_edis_lp, c->d_lp_misc};
   for (void* q : old)
     if (q) cudaFree(q);
   c->d_cx = c->d_cy = nullptr;
   c->d_eagg = c->d_edis = nullptr;
+  c->d_eorder = nullptr;
+  c->eagg_ld = n;
   c->d_eagg_lp = c->d_edis_lp = nullptr;
   c->d_lp_misc = nullptr;
   c->n = n;
@@ -649,7 +651,7 @@ extern "C" int lsms_aggregate(lsms_ctx* c, int nrhs, const double* beta, double*
     if ((rc = aggregate_mixed(c, nrhs, (const double2*)c->ws_x.ptr, G, c->stream))) return rc;
   } else {
     // the caller sees single nodes: sums that keep each of them to its own size (contour_f64_tc.cu)
-    launch_zgemm_direct(c->d_eagg, 2 * ns, c->n, (const double2*)c->ws_x.ptr, G, P, nrhs, c->stream);
+    aggregate_direct(c, nrhs, (const double2*)c->ws_x.ptr, G, c->stream);
   }
   launch_node_stage(ns, P, nrhs, G, c->d_fagg, nullptr, nullptr, nullptr, (double2*)c->ws_pq.ptr,
                     nullptr, nullptr, c->stream);

@@ -21,10 +21,10 @@
 // and lsms_disaggregate, which show single nodes, sum on the FP64 pipe.
 //
 // The FP64 tables are read once and cut into digits on the way to shared memory (a lane takes one
-// complex element, a warp one 8-row x 4-element core matrix: 32 distinct banks on the store; the
-// aggregate's columns are gathered in order of depth).  The whole reflected coupling of 5000 discs and 1024 nodes
-// takes 0.46 ms (0.27 ms with one scale per row and six digits, 5.1 ms on the FP64 pipe; the tables'
-// two reads are 0.05 ms), of 1000 discs and 512 nodes 125 us (FP64 pipe: 546 us), of 20,000 discs 1.5 ms (20 ms).
+// complex element, a warp one 8-row x 4-element core matrix: 64 contiguous bytes per row from
+// memory, 32 distinct banks on the store; E_agg's columns are stored in order of depth).  The whole reflected coupling of 5000 discs and 1024 nodes
+// takes 0.30 ms (0.27 ms with one scale per row and six digits, 5.1 ms on the FP64 pipe; the tables'
+// two reads are 0.05 ms), of 1000 discs and 512 nodes 116 us (FP64 pipe: 546 us), of 20,000 discs 0.83 ms (20 ms).
 #include <algorithm>
 #include <cmath>
 #include <cstring>
@@ -58,23 +58,30 @@ __device__ __forceinline__ unsigned long long mag_bits(double2 v) {
   return a > b ? a : b;
 }
 
-// Largest |Re|, |Im| of every (class, row) of a [rows][cols] table, one warp each; the class's columns are
-// kidx[start[c]] .. kidx[start[c + 1] - 1], negative entries are padding.
-__global__ void k_row_max(const double2* __restrict__ a, int rows, int cols, const int* __restrict__ kidx,
-                          const int* __restrict__ start, unsigned long long* __restrict__ out) {
+// out[r][e] = a[r][kidx[e]] (zero where that is negative), e < ld: the columns of E_agg in their classes.
+__global__ void k_order_columns(const double2* __restrict__ a, int rows, int cols, const int* __restrict__ kidx, int ld,
+                                double2* __restrict__ out) {
+  const long long total = (long long)rows * ld;
+  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < total; i += (long long)gridDim.x * blockDim.x) {
+    const long long r = i / ld;
+    const int k = kidx[i - r * ld];
+    out[i] = k >= 0 ? a[r * cols + k] : make_double2(0.0, 0.0);
+  }
+}
+// Largest |Re|, |Im| of every (class, row) of that table [rows][ld], one warp each; the class's columns are
+// start[c] .. start[c + 1] - 1.
+__global__ void k_row_max(const double2* __restrict__ a, int rows, int ld, const int* __restrict__ start,
+                          unsigned long long* __restrict__ out) {
   const int r = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31, c = blockIdx.y;
   if (r >= rows) return;
   unsigned long long m = 0;
-  for (int e = start[c] + lane; e < start[c + 1]; e += 32) {
-    const int k = kidx[e];
-    if (k >= 0) m = max(m, mag_bits(a[(size_t)r * cols + k]));
-  }
+  for (int e = start[c] + lane; e < start[c + 1]; e += 32) m = max(m, mag_bits(a[(size_t)r * ld + e]));
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
   if (lane == 0) out[(size_t)c * rows + r] = m;
 }
-// The same of every (class, column), the class's rows listed in the same way; out zeroed, grid.z parts of
-// the class.
+// The same of every (class, column) of E_dis, the class's rows kidx[start[c]] .. kidx[start[c + 1] - 1], negative
+// entries are padding; out zeroed, grid.z parts of the class.
 __global__ void k_col_max(const double2* __restrict__ a, int cols, const int* __restrict__ kidx,
                           const int* __restrict__ start, unsigned long long* __restrict__ out) {
   const int v = blockIdx.x * blockDim.x + threadIdx.x, c = blockIdx.y;
@@ -98,15 +105,16 @@ __global__ void k_exponents(const unsigned long long* __restrict__ bits, int cou
 // Largest |Re|, |Im| of every (right-hand side, class, order) of b [r][K][P], times 2^-kRoom.
 // Aggregate (kexp null): over the class's discs.  Disaggregate: over all nodes, element k times
 // 2^kexp[class][k].
-__global__ void k_order_max(const double2* __restrict__ b, int K, int P, const int* __restrict__ kidx,
+__global__ void __launch_bounds__(256)
+k_order_max(const double2* __restrict__ b, int K, int P, const int* __restrict__ kidx,
                             const int* __restrict__ start, const int* __restrict__ kexp,
                             unsigned long long* __restrict__ out) {
+  __shared__ unsigned long long part[8][32];
   const int q = threadIdx.x & 31, r = blockIdx.y, c = blockIdx.z;
-  if (q >= P) return;
-  const int w = threadIdx.x >> 5, step = gridDim.x * (blockDim.x >> 5);
+  const int w = threadIdx.x >> 5, step = gridDim.x * 8;
   const int e0 = kexp ? 0 : start[c], e1 = kexp ? K : start[c + 1];
   unsigned long long m = 0;
-  for (int e = e0 + blockIdx.x * (blockDim.x >> 5) + w; e < e1; e += step) {
+  for (int e = e0 + blockIdx.x * 8 + w; e < e1 && q < P; e += step) {
     const int k = kexp ? e : kidx[e];
     if (k < 0) continue;
     unsigned long long v = mag_bits(b[((size_t)r * K + k) * P + q]);
@@ -115,6 +123,10 @@ __global__ void k_order_max(const double2* __restrict__ b, int K, int P, const i
           scalbn(__longlong_as_double((long long)v), (kexp ? kexp[(size_t)c * K + k] : 0) - kRoom));
     m = max(m, v);
   }
+  part[w][q] = m;                                  // one update per CTA: the addresses are few
+  __syncthreads();
+  if (w > 0) return;
+  for (int i = 1; i < 8; ++i) m = max(m, part[i][q]);
   if (m) atomicMax(out + ((size_t)r * gridDim.z + c) * 32 + q, m);
 }
 
@@ -192,7 +204,7 @@ __device__ __forceinline__ int group_end(const unsigned char* cls, int t, int nt
   return e;
 }
 
-// C[r][m][q] += sum_k A[m][k] B[r][k][q].  AGG: rows m = the table's, K order kidx, A scaled by
+// C[r][m][q] += sum_k A[m][k] B[r][k][q].  AGG: rows m = the table's, its K columns in their classes, A scaled by
 // 2^-aexp[class of the stage][m].  Else rows m = kidx[tile.y + i], i < tile.z, of class tile.x, K order
 // the nodes', A scaled by 2^-aexp[class][k] (the inverse is in the image).  grid: (row tiles, K ranges,
 // right-hand sides); shared memory fits one CTA per SM.
@@ -259,12 +271,8 @@ k_zgemm_digits(const double2* __restrict__ A, int M, int K, const int* __restric
     }
     auto k_at = [&](int t, int h) {
       const int kp = (t_begin + t) * CK + 4 * h + ke;
-      return AGG ? kidx[kp] : kp < K ? kp : -1;
+      return kp < K ? kp : -1;
     };
-    int kn[2] = {-1, -1};
-    if (g < nt)
-#pragma unroll
-      for (int h = 0; h < 2; ++h) kn[h] = k_at(g, h);
     int cur = -1;
     bool ok = true;
     for (int t = g; t < nt; t += 2) {
@@ -273,11 +281,10 @@ k_zgemm_digits(const double2* __restrict__ A, int M, int K, const int* __restric
       int ek[2];
 #pragma unroll
       for (int h = 0; h < 2; ++h) {
-        const int k = kn[h];
+        const int k = k_at(t, h);
         ek[h] = !AGG && k >= 0 ? aexp[(size_t)tile.x * K + k] : 0;
 #pragma unroll
         for (int j = 0; j < 4; ++j) v[4 * h + j] = m[j] >= 0 && k >= 0 ? __ldg(rp[j] + k) : make_double2(0.0, 0.0);
-        if (t + 2 < nt) kn[h] = k_at(t + 2, h);
       }
       if (AGG && cls[t] != cur) {
         cur = cls[t];
@@ -421,7 +428,7 @@ void launch_digits(const lsms_ctx* c, const Launch& l, int* err) {
   });
   const ZgemmTc& z = c->zgemm;
   k_zgemm_digits<NPAD, AGG><<<l.grid, THREADS, zsmem_bytes(NPAD), l.st>>>(
-      l.A, l.M, l.K, z.d_kidx, z.d_scls, (const int4*)z.d_tiles, z.classes, l.aexp, l.img, l.stages, l.per_cta, c->P,
+      l.A, l.M, l.K, c->d_eorder, z.d_scls, (const int4*)z.d_tiles, z.classes, l.aexp, l.img, l.stages, l.per_cta, c->P,
       l.r0, l.maxbits, l.C, err);
 }
 
@@ -485,30 +492,42 @@ int zgemm_setup(lsms_ctx* c) {
   }
   // one allocation: the exponents of E_agg and E_dis, the lists, then the maxima the exponents come from
   const size_t per = (size_t)classes * rows;
-  const size_t be = aligned(2 * per * sizeof(int)), bl = aligned(list.size() * sizeof(int)), bs = aligned(scls.size()),
-               bt = aligned(tiles.size() * sizeof(int4)), bc = aligned(start.size() * sizeof(int));
-  const size_t lists = bl + bs + bt + bc, bm = 2 * per * 8 + 16;
-  if (device_alloc_optional(c, (void**)&z.d_exp, be + lists + bm) != cudaSuccess) {
+  const size_t be = aligned(2 * per * sizeof(int)), bs = aligned(scls.size()), bt = aligned(tiles.size() * sizeof(int4)),
+               bc = aligned(start.size() * sizeof(int));
+  const size_t lists = bs + bt + bc, bm = 2 * per * 8 + 16;
+  const int ld = (int)list.size();
+  double2* ordered = nullptr;
+  int* order = nullptr;
+  if (device_alloc_optional(c, (void**)&z.d_exp, be + lists + bm) != cudaSuccess ||
+      device_alloc_optional(c, (void**)&ordered, (size_t)rows * ld * sizeof(double2)) != cudaSuccess ||
+      device_alloc_optional(c, (void**)&order, ld * sizeof(int)) != cudaSuccess) {
+    if (ordered) cudaFree(ordered);
     zgemm_free(c);
     return LSMS_OK;                                // the FP64 pipe then (launch_zgemm_direct)
   }
+  // E_agg's columns class by class: gathered where they lie, its product took 246 instead of 103 us at 5000 discs
+  copy_up(c, order, list.data(), ld * sizeof(int));
+  k_order_columns<<<152 * 16, 256, 0, c->stream>>>(c->d_eagg, rows, n, order, ld, ordered);
+  cudaStreamSynchronize(c->stream);
+  cudaFree(c->d_eagg);
+  c->d_eagg = ordered;
+  c->d_eorder = order;
+  c->eagg_ld = ld;
   unsigned char* at = (unsigned char*)z.d_exp + be;
-  z.d_kidx = (int*)at;
-  z.d_scls = at + bl;
-  z.d_tiles = at + bl + bs;
-  z.d_start = (int*)(at + bl + bs + bt);
+  z.d_scls = at;
+  z.d_tiles = at + bs;
+  z.d_start = (int*)(at + bs + bt);
   std::vector<unsigned char> host(lists, 0);
-  std::memcpy(host.data(), list.data(), list.size() * sizeof(int));
-  std::memcpy(host.data() + bl, scls.data(), scls.size());
-  std::memcpy(host.data() + bl + bs, tiles.data(), tiles.size() * sizeof(int4));
-  std::memcpy(host.data() + bl + bs + bt, start.data(), start.size() * sizeof(int));
+  std::memcpy(host.data(), scls.data(), scls.size());
+  std::memcpy(host.data() + bs, tiles.data(), tiles.size() * sizeof(int4));
+  std::memcpy(host.data() + bs + bt, start.data(), start.size() * sizeof(int));
   unsigned long long* bits = (unsigned long long*)(at + lists);
   int* bad = (int*)(bits + 2 * per);
-  cudaMemcpyAsync(at, host.data(), lists, cudaMemcpyHostToDevice, c->stream);
+  copy_up(c, at, host.data(), lists);
   cudaMemsetAsync(bits, 0, bm, c->stream);
-  k_row_max<<<dim3((rows + 7) / 8, classes), 256, 0, c->stream>>>(c->d_eagg, rows, n, z.d_kidx, z.d_start, bits);
+  k_row_max<<<dim3((rows + 7) / 8, classes), 256, 0, c->stream>>>(c->d_eagg, rows, ld, z.d_start, bits);
   k_col_max<<<dim3((rows + 127) / 128, classes, std::min(64, (widest + 63) / 64)), 128, 0, c->stream>>>(
-      c->d_edis, rows, z.d_kidx, z.d_start, bits + per);
+      c->d_edis, rows, order, z.d_start, bits + per);
   k_exponents<<<(int)((2 * per + 255) / 256), 256, 0, c->stream>>>(bits, (int)(2 * per), z.d_exp, bad);
   int h = 0;
   cudaMemcpyAsync(&h, bad, sizeof(int), cudaMemcpyDeviceToHost, c->stream);
@@ -520,7 +539,11 @@ int zgemm_setup(lsms_ctx* c) {
   return check_cuda(c, "zgemm_setup");
 }
 
-// C[r][M][P] += table . B for the aggregate (M = 2 N_S, K = n) or the disaggregate (M = n, K = 2 N_S).
+void aggregate_direct(lsms_ctx* c, int nrhs, const double2* B, double2* G, cudaStream_t st) {
+  launch_zgemm_direct(c->d_eagg, 2 * c->ns, c->eagg_ld, B, G, c->P, nrhs, st, c->d_eorder, c->n);
+}
+
+// C[r][M][P] += table . B for the aggregate (M = 2 N_S, K = the discs) or the disaggregate (M = n, K = 2 N_S).
 int zgemm_f64(lsms_ctx* c, bool agg, int nrhs, const double2* B, double2* C, cudaStream_t st) {
   ZgemmTc& z = c->zgemm;
   Launch l;
@@ -529,12 +552,14 @@ int zgemm_f64(lsms_ctx* c, bool agg, int nrhs, const double2* B, double2* C, cud
   l.B = B;
   l.C = C;
   l.M = agg ? 2 * c->ns : c->n;
-  l.K = agg ? c->n : 2 * c->ns;
+  l.K = agg ? c->eagg_ld : 2 * c->ns;
   ++c->f64_launches;                                 // the direct product or the order maxima
-  if (!z.ready) {
-    launch_zgemm_direct(l.A, l.M, l.K, B, C, c->P, nrhs, st);
-    return LSMS_OK;
-  }
+  auto direct = [&] {
+    if (agg) aggregate_direct(c, nrhs, B, C, st);
+    else launch_zgemm_direct(l.A, l.M, l.K, B, C, c->P, nrhs, st);
+    return check_cuda(c, "zgemm_f64");
+  };
+  if (!z.ready) return direct();
   const int npad = pad_columns(c->p), dis_stages = (2 * c->ns + CK - 1) / CK;
   l.stages = agg ? z.stages : dis_stages;
   const int images = agg ? 1 : z.classes;
@@ -543,10 +568,7 @@ int zgemm_f64(lsms_ctx* c, bool agg, int nrhs, const double2* B, double2* C, cud
   const size_t one = sb * std::max(z.stages, z.classes * dis_stages);
   const int rb = (int)std::max<size_t>(1, std::min<size_t>(nrhs, kImageBytes / one));
   const size_t mbytes = aligned((size_t)nrhs * z.classes * 32 * 8);
-  if (!ensure_optional(c, c->ws_zgemm, mbytes + rb * one, st)) {   // as in translate_f64_tc
-    launch_zgemm_direct(l.A, l.M, l.K, B, C, c->P, nrhs, st);
-    return check_cuda(c, "zgemm_f64");
-  }
+  if (!ensure_optional(c, c->ws_zgemm, mbytes + rb * one, st)) return direct();   // as in translate_f64_tc
   unsigned long long* maxbits = (unsigned long long*)c->ws_zgemm.ptr;
   unsigned char* img = (unsigned char*)c->ws_zgemm.ptr + mbytes;
   l.maxbits = maxbits;
@@ -555,16 +577,16 @@ int zgemm_f64(lsms_ctx* c, bool agg, int nrhs, const double2* B, double2* C, cud
   const int* kexp = agg ? nullptr : l.aexp;
   int* err = tc_err_flag(c);
   cudaMemsetAsync(maxbits, 0, (size_t)nrhs * z.classes * 32 * 8, st);
-  const int mean = agg ? l.K / z.classes : l.K;
-  k_order_max<<<dim3(std::max(1, std::min(64, mean / 64)), nrhs, z.classes), 256, 0, st>>>(B, l.K, c->P, z.d_kidx, z.d_start, kexp,
-                                                                                         maxbits);
+  const int rows = agg ? c->n : l.K, mean = agg ? l.K / z.classes : l.K;       // rows of B, and of a class
+  k_order_max<<<dim3(std::max(1, std::min(64, mean / 16)), nrhs, z.classes), 256, 0, st>>>(
+      B, rows, c->P, c->d_eorder, z.d_start, kexp, maxbits);
   const int mt = agg ? (l.M + ROWS - 1) / ROWS : z.tiles;
   for (l.r0 = 0; l.r0 < nrhs; l.r0 += rb) {
     const int nr = std::min(rb, nrhs - l.r0);
     const int items = l.stages * KG * (npad / 2);
     c->f64_launches += 2;
     k_pack_columns<<<dim3(std::min((items + 127) / 128, 1024), nr, images), 128, 0, st>>>(
-        B, l.K, c->P, l.r0, l.stages, npad, z.classes, z.d_kidx, z.d_scls, kexp, maxbits, img);
+        B, rows, c->P, l.r0, l.stages, npad, z.classes, c->d_eorder, z.d_scls, kexp, maxbits, img);
     // K ranges: the fewest rounds of 152 CTAs times the stages of a CTA, plus a start and an end worth
     // about twelve stages
     int best = 1;

@@ -102,8 +102,7 @@ struct ZgemmTc {
   int classes = 0;                  // of discs, by depth
   int stages = 0, tiles = 0;        // K stages of the aggregate, row tiles of the disaggregate
   int* d_exp = nullptr;             // [classes][2ns] exponents of E_agg's rows, the same of E_dis's columns
-  int* d_kidx = nullptr;            // the discs class by class, padded with -1 to whole stages; behind d_exp, as
-  int* d_start = nullptr;           // [classes + 1] where each begins
+  int* d_start = nullptr;           // [classes + 1] where each begins in d_eorder; behind d_exp, as the others
   unsigned char* d_scls = nullptr;  // class of every stage
   void* d_tiles = nullptr;          // int4 (class, first position, rows, 0)
 };
@@ -159,7 +158,10 @@ struct lsms_ctx {
   // per-layout device data
   double* d_cx = nullptr;           // centred x, [n]
   double* d_cy = nullptr;           // [n]
-  double2* d_eagg = nullptr;        // [2ns][n]: exp(g2 y - i l x) rows, then exp(-g2 (y+d) - i l x)
+  double2* d_eagg = nullptr;        // [2ns][eagg_ld]: exp(g2 y - i l x) rows, then exp(-g2 (y+d) - i l x)
+  int eagg_ld = 0;                  // columns: the n discs, or
+  int* d_eorder = nullptr;          //   class by class in order of depth (contour_f64_tc.cu): the disc of each
+                                    //   column, -1 for a zero one
   double2* d_edis = nullptr;        // [n][2ns]: exp(g2 y + i l x), then exp(-g2 (y+d) + i l x)
   // low-precision copies for the mixed path (split BF16 hi/lo planes, see mixed.cu)
   void* d_eagg_lp = nullptr;
@@ -285,8 +287,9 @@ void launch_etables(const double* cx, const double* cy, int n, const double2* la
                     const double2* g2, int ns, double d, double2* eagg, double2* edis,
                     cudaStream_t st);
 // C[r][m][n] += sum_k A[m][k] B[r][k][n] on the FP64 pipe (contour_direct.cu; K ranges add atomically)
+// order: B has n rows, column k of A meets row order[k] (none if negative)
 void launch_zgemm_direct(const double2* A, int M, int K, const double2* B, double2* C, int P,
-                         int nrhs, cudaStream_t st);
+                         int nrhs, cudaStream_t st, const int* order = nullptr, int n = 0);
 // the aggregate, the reflection and V = U sigma in one kernel (small tables)
 void launch_node_direct(int ns, int n, int P, int nrhs, const double2* eagg, const double2* xs,
                         const double2* fagg, const double2* refl, const double2* udis, double2* V,

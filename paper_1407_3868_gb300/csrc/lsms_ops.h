@@ -52,6 +52,7 @@ int translate_f64(lsms_ctx* c, int nrhs, const double2* xs, double2* alpha, cuda
 constexpr double kZgemmMinTable = 1.5e5;   // complex elements of a table; smaller: contour_direct.cu
 int zgemm_setup(lsms_ctx* c);
 void zgemm_free(lsms_ctx* c);
+void aggregate_direct(lsms_ctx* c, int nrhs, const double2* B, double2* G, cudaStream_t st);   // FP64 pipe
 int zgemm_f64(lsms_ctx* c, bool agg, int nrhs, const double2* B, double2* C, cudaStream_t st);
 // drop the captured batched applications (their kernels depend on the context's settings)
 void batch_clear_graphs(lsms_ctx* c);

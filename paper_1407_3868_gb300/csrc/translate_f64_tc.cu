@@ -127,31 +127,47 @@ k_disc_max(const double2* __restrict__ x, int n, int P, unsigned long long* __re
   }
 }
 
+// The large discs of each right-hand side, one CTA each (counted by the CTAs of k_pack_digits, whose updates
+// of one address wait for each other, they took 14 us more at 2000 discs).
+__global__ void __launch_bounds__(256)
+k_large_discs(int n, const unsigned long long* __restrict__ dmax, RhsStats* __restrict__ stats) {
+  __shared__ int part[8], disc;
+  const int r = blockIdx.x, w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const unsigned long long mb = stats[r].maxbits;
+  const unsigned long long large = mb > (5ull << 52) ? mb - (4ull << 52) : 1;
+  int count = 0;
+  for (int l = threadIdx.x; l < n; l += 256)
+    if (dmax[(size_t)r * n + l] >= large) {
+      ++count;
+      disc = l;
+    }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) count += __shfl_xor_sync(0xffffffffu, count, o);
+  if (lane == 0) part[w] = count;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    for (int i = 1; i < 8; ++i) count += part[i];
+    stats[r].count = count;
+    stats[r].disc = disc;
+  }
+}
+
 // Digits of X for the sources src0 .. src0 + gridDim.x - 1 of right-hand side r0 + blockIdx.y:
 // per source [K group][plane][column][8 K values] FP16, K = 4 s + (A, B, C, D), column 2 q + (Re, Im); and
 // bound[source]: what the source adds to any element of the levels 0..4 at most, 128 sum |X digits of the
-// planes 0..4|, or a quarter of the same for level 5, whose sums may pass 2^24 up to 2^26 (rounded to 2^-51
-// of the scales).  The first run of sources (src0 = 0) also counts the right-hand side's large discs.
+// planes 0..4|, or to a quarter of level 5, whose sums may pass 2^24 up to 2^26 (rounded to 2^-51
+// of the scales).
 __global__ void __launch_bounds__(256)
 k_pack_digits(const double2* __restrict__ xs, int n, int p, int src0, int r0, int npad, int kgs,
-              const unsigned long long* __restrict__ dmax, RhsStats* __restrict__ stats,
-              unsigned char* __restrict__ img, int* __restrict__ bound) {
+              const RhsStats* __restrict__ stats, unsigned char* __restrict__ img, int* __restrict__ bound) {
   __shared__ long long re[128], im[128];          // beta_{nu +- s} at 48 + order, zero outside -p..p
-  __shared__ int l1[2][64];                       // sum of |digit| of the planes 0..4 and 0..5 per column
+  __shared__ int l1[64];                          // sum of |digit| per column, see the bound
   const int P = 2 * p + 1, r = r0 + blockIdx.y;
   const unsigned long long mb = stats[r].maxbits;
   if (mb == 0 || mb >= kInfBits) return;          // the product does not read the image then
-  if (src0 == 0 && threadIdx.x == 0) {
-    const unsigned long long large = mb > (5ull << 52) ? mb - (4ull << 52) : 1;
-    for (int l = blockIdx.x; l < n; l += gridDim.x)
-      if (dmax[(size_t)r * n + l] >= large) {
-        atomicAdd(&stats[r].count, 1);
-        stats[r].disc = l;
-      }
-  }
   const int sh = 46 - scale_exponent(mb);
   const double2* b = xs + ((size_t)r * n + src0 + blockIdx.x) * P;
-  if (threadIdx.x < 64) l1[0][threadIdx.x] = l1[1][threadIdx.x] = 0;
+  if (threadIdx.x < 64) l1[threadIdx.x] = 0;
   if (threadIdx.x < 128) {
     const int o = (int)threadIdx.x - 48 + p;
     double2 v = make_double2(0.0, 0.0);
@@ -195,7 +211,7 @@ k_pack_digits(const double2* __restrict__ xs, int n, int p, int src0, int r0, in
         w[j][2 * h + 1] = v[j];
       }
     }
-    int sum[2] = {0, 0};
+    int sum = 0, last = 0;
 #pragma unroll
     for (int j = 0; j < PL; ++j) {
       dst[((size_t)kg * PL + j) * npad + col] = make_uint4(w[j][0], w[j][1], w[j][2], w[j][3]);
@@ -203,16 +219,14 @@ k_pack_digits(const double2* __restrict__ xs, int n, int p, int src0, int r0, in
 #pragma unroll
       for (int i = 0; i < 4; ++i) h = __hadd2(h, __habs2(*reinterpret_cast<const __half2*>(&w[j][i])));
       const int d = (int)__low2float(h) + (int)__high2float(h);
-      if (j <= 4) sum[0] += d;
-      sum[1] += d;
+      if (j < 5) sum += d;
+      else last = d;
     }
-    atomicAdd(&l1[0][col], sum[0]);
-    atomicAdd(&l1[1][col], sum[1]);
+    atomicAdd(&l1[col], max(sum, (sum + last + 3) / 4));
   }
   __syncthreads();
   if (threadIdx.x < 32) {
-    int m = max(max(l1[0][threadIdx.x], l1[0][threadIdx.x + 32]),
-                max(l1[1][threadIdx.x], l1[1][threadIdx.x + 32]) / 4);
+    int m = max(l1[threadIdx.x], l1[threadIdx.x + 32]);
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
     if (threadIdx.x == 0) bound[(size_t)blockIdx.y * gridDim.x + blockIdx.x] = 128 * m;
@@ -672,6 +686,7 @@ int translate_f64_tc(lsms_ctx* c, int nrhs, const double2* xs, double2* alpha, c
   int* err = tc_err_flag(c);
   cudaMemsetAsync(stats, 0, (size_t)nrhs * sizeof(RhsStats), st);
   k_disc_max<<<dim3((n + 7) / 8, nrhs), 256, 0, st>>>(xs, n, P, dmax, stats);
+  k_large_discs<<<nrhs, 256, 0, st>>>(n, dmax, stats);
   const PairConsts pc = pair_consts(c->k2, pair_z_near(p));
   const int tiles = (nrows + ROWS - 1) / ROWS;
   for (int r0 = 0; r0 < nrhs; r0 += rb) {
@@ -679,7 +694,7 @@ int translate_f64_tc(lsms_ctx* c, int nrhs, const double2* xs, double2* alpha, c
     for (int s0 = 0; s0 < n; s0 += run) {
       const int ns = std::min(run, n - s0);
       c->f64_launches += 2;
-      k_pack_digits<<<dim3(ns, nr), 256, 0, st>>>(xs, n, p, s0, r0, npad, 2 * steps, dmax, stats, img, bound);
+      k_pack_digits<<<dim3(ns, nr), 256, 0, st>>>(xs, n, p, s0, r0, npad, 2 * steps, stats, img, bound);
       // source ranges: the fewest waves of 152 CTAs times the rounds of two sources of a CTA, plus
       // about two rounds of time per CTA for its start and end
       int best = 1;
@@ -704,7 +719,7 @@ int translate_f64_tc(lsms_ctx* c, int nrhs, const double2* xs, double2* alpha, c
   }
   k_dominant_row<<<dim3((n + 31) / 32, nrhs), 32, 0, st>>>(c->d_cx, c->d_cy, n, p, c->k2, pc, xs, stats, row0, nrows,
                                                           alpha);
-  c->f64_launches += 2 + (f.nnz > 0 ? 1 : 0);          // maxima, the dominant row, near pairs
+  c->f64_launches += 3 + (f.nnz > 0 ? 1 : 0);          // maxima, large discs, the dominant row, near pairs
   // lists cut so that the warps fill the chip (300 discs: 161 -> 107 us the translation, 1000: 478 -> 444)
   const int near_splits = (int)std::max<long long>(1, std::min<long long>(4, 152LL * 24 / std::max(1LL, (long long)nrows * nrhs)));
   if (f.nnz > 0)
