@@ -621,19 +621,15 @@ int f64tc_setup(lsms_ctx* c, const std::vector<int>& ptr, const std::vector<int>
   return check_cuda(c, "f64tc_setup");
 }
 
-// The stored near sequences (63 MB at 5000 discs, p = 14) exist while all-pairs FP64 translations
-// can run: not while every translation goes through boxes, nor in a mixed context that has had none
-// (its solves come to them with their first FP64 residual).
+// The near sequences (63 MB at 5000 discs, p = 14) are stored when all-pairs FP64 translations can first
+// run: not while every translation goes through boxes, nor in a mixed context that has had none
+// (its solves come to them with their first FP64 residual).  They stay for the layout: an application
+// captured before boxes were switched on refers to them.
 int f64tc_sequences(lsms_ctx* c) {
   F64Tc& f = c->f64tc;
   const bool want = f.ready && f.nnz > 0 && (c->precision != LSMS_MIXED || f.used) &&
                     !(c->fmm.ready && c->fmm.scope == LSMS_FMM_ALL);
-  if (want == (f.d_seq != nullptr)) return LSMS_OK;
-  if (!want) {
-    cudaFree(f.d_seq);
-    f.d_seq = nullptr;
-    return LSMS_OK;
-  }
+  if (!want || f.d_seq) return LSMS_OK;
   if (device_alloc_optional(c, &f.d_seq, (size_t)f.nnz * (4 * c->p + 1) * sizeof(double2)) != cudaSuccess) {
     f64tc_free(c);
     return LSMS_OK;

@@ -149,6 +149,27 @@ def test_batch_takes_optional_memory_back(L):
     ctx.close()
 
 
+def test_captured_application_outlives_a_change_to_boxes(L):
+    import torch
+    n, p = 300, 8
+    ctx, c, _, hs = context(L, n, p)
+    ctx.set_particles(c)
+    x = torch.from_numpy(inputs.random_coefficients(n, p, 1, 2) / hs).cuda()
+    y, ref = torch.zeros_like(x), torch.zeros_like(x)
+    ctx.apply_dev(x, ref)
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        ctx.apply_dev(x, y)
+    ctx.set_fmm(4.0)
+    other = [torch.full((1 << 20,), float("nan"), dtype=torch.float64, device="cuda") for _ in range(8)]
+    graph.replay()
+    torch.cuda.synchronize()
+    assert rel(y[0].cpu().numpy(), ref[0].cpu().numpy(), hs) <= TOL
+    del graph, other
+    ctx.close()
+
+
 @pytest.mark.parametrize("precision", [0, 1])
 def test_capture_allocates_nothing(L, precision):
     """A capture that begins before the digit products have run on this layout: after another layout of the
