@@ -52,9 +52,21 @@ typedef enum {
 } lsms_status;
 
 typedef enum {
-  LSMS_FP64 = 0,   /* float64 throughout (products of large sums as exact sums of digits)      */
+  LSMS_FP64 = 0,   /* float64; the large sums as products of fixed-point operands (see below)  */
   LSMS_MIXED = 1   /* FP32 translation, split-BF16 tensor-core contour contractions, FP64 refinement */
 } lsms_precision;
+/* FP64 sums.  The far pairs of the all-pairs translation (layouts from 96 discs on) are summed as
+ * products of 48-bit fixed-point operands: the Hankel factors with 48 fractional bits, the
+ * coefficients relative to the largest of their right-hand side.  The contour contractions of large
+ * tables (2 N_S N >= 1.5e5) use 56-bit operands, the tables and coefficients each relative to the
+ * largest in a class of discs of like depth.  Products are summed in integers.  Every disc's row of an
+ * output is as close to the exact sum as a plain FP64 sum is, also when the coefficients are uneven over
+ * discs or orders: the row of a disc whose coefficients alone exceed all others 16 times is a plain FP64
+ * sum.  lsms_aggregate and lsms_disaggregate, which show single contour nodes, are plain FP64 sums too.
+ * The operands' memory (up to 8 GB of sequences and 400 MB of images per context) is given back when
+ * another request fails (an application captured before that must not be replayed); plain FP64 sums
+ * run then.  Inside a stream capture none is allocated: an application captured before one of as many
+ * right-hand sides has run captures plain FP64 sums. */
 
 /* Discretised Sommerfeld contour (Sec. 5.1, Eq. "sommerseg"): Gamma3 = t + i b (t < 0),
  * Gamma2 = i s (s from b to -b), Gamma1 = t - i b (t > 0), truncated at |t| = t_max.

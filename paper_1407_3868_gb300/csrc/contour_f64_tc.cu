@@ -23,8 +23,10 @@
 // The FP64 tables are read once and cut into digits on the way to shared memory (a lane takes one
 // complex element, a warp one 8-row x 4-element core matrix: 64 contiguous bytes per row from
 // memory, 32 distinct banks on the store; E_agg's columns are stored in order of depth).  The whole reflected coupling of 5000 discs and 1024 nodes
-// takes 0.30 ms (0.27 ms with one scale per row and six digits, 5.1 ms on the FP64 pipe; the tables'
-// two reads are 0.05 ms), of 1000 discs and 512 nodes 116 us (FP64 pipe: 546 us), of 20,000 discs 0.83 ms (20 ms).
+// takes 0.28 ms (0.27 ms with one scale per row and six digits, 5.1 ms on the FP64 pipe; the tables'
+// two reads are 0.05 ms), of 1000 discs and 512 nodes 101 us (FP64 pipe: 546 us), of 20,000 discs 0.82 ms (20 ms).
+// The products are bound by the conversion (ALU pipe at half its peak) and the waits between it, the MMAs
+// and the drains.
 #include <algorithm>
 #include <cmath>
 #include <cstring>

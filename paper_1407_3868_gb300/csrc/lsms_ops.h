@@ -49,7 +49,10 @@ int translate_f64(lsms_ctx* c, int nrhs, const double2* xs, double2* alpha, cuda
                   int nrows = -1);
 // FP64 contour contractions: C[r][M][P] += E_agg . B (agg) or E_dis . B; tables for the tensor cores
 // (contour_f64_tc.cu)
-constexpr double kZgemmMinTable = 1.5e5;   // complex elements of a table; smaller: contour_direct.cu
+// complex elements of a table; smaller: contour_direct.cu (the reflected coupling at 512 nodes, p = 12: 96 discs
+// 87 us either way, 128 discs 106 us direct and 90 as digits, 150 discs 122 and 94, 400 discs 284 and 97); the
+// line lies where the digits win by a fifth
+constexpr double kZgemmMinTable = 1.5e5;
 int zgemm_setup(lsms_ctx* c);
 void zgemm_free(lsms_ctx* c);
 void aggregate_direct(lsms_ctx* c, int nrhs, const double2* B, double2* G, cudaStream_t st);   // FP64 pipe

@@ -18,7 +18,7 @@
 //
 // Why: this chip's FP64 pipe (2 FMA per SM and clock) bounds the direct form at 133 ms for 5000 discs
 // (k_translate_f64_sym: 168 ms); 21 products of FP16 digits take 4.7 ms at the tensor cores' measured
-// rate, and this kernel 8.2 ms (1000 discs at p = 12: 5.2 -> 0.33 ms).
+// rate, and this kernel 8.4 ms (1000 discs at p = 12, 26 products: 5.2 -> 0.33 ms).
 //
 // A CTA owns 128 targets and a range of sources.  Two warpgroups form the W rows of every second
 // source each (thread = target; the fixed-point sequence of pair_fixed.cuh), eight orders at a time
@@ -545,7 +545,10 @@ void launch_digits(dim3 grid, cudaStream_t st, const lsms_ctx* c, const PairCons
 }
 
 constexpr size_t kImageBytes = (size_t)256 << 20;   // digits of X held at once
+// p = 12: 96 discs 75 us from stored sequences and 86 as digits, 112 discs 101 and 87, 150 discs 155 and 89
 constexpr int kMinDiscs = 96;
+// mostly near pairs, p = 12: 320 discs (80 MB) 713 us stored and 732 on the FP64 pipe, 600 discs 2.27 and
+// 2.40 ms, 1000 discs (780 MB) 7.05 and 6.52 ms: too little either way for the memory
 constexpr double kStoreBytes = 64e6;
 constexpr double kNearBytes = 8e9;                  // near sequences beside the digits
 
