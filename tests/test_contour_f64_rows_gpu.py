@@ -74,6 +74,12 @@ def test_rows_and_nodes(L, kind, n, p, n_nodes):
             po, qo = pr.aggregate(x[r])
             assert np.all(np.abs(pp[r] - po) <= TOL * np.abs(po) + TINY), r
             assert np.all(np.abs(qm[r] - qo) <= TOL * np.abs(qo) + TINY), r
+    # incident coefficients of sources high above the layer and close to it
+    for src in ([0.3, 1.0], [-0.4, 0.05]):
+        ref = pr.incident_local(np.array(src))
+        got = ctx.incident([src])[0]
+        for w in (1.0, 1.0 / hs):
+            assert np.max(np.linalg.norm((got - ref) * w, axis=1) / np.linalg.norm(ref * w, axis=1)) <= TOL, src
     # one node alone: the deep discs' rows of an evanescent density
     s = np.zeros(len(lam), dtype=complex)
     s[int(np.argmin(np.abs(lam.real - 60.0)))] = 1.0
